@@ -191,6 +191,9 @@ static const void* panel_variant_cl(int q) {     // the same shapes as one threa
 constexpr int kPanelVariantsCl = 6;
 constexpr int kPanelVariantReg = 5;
 constexpr int kClusterMaxRows = 128;
+// Padded slabs have a pitch of 4 mod 16 doubles: the fragment loads of the matrix products (eight columns x four rows)
+// hit every bank pair once.
+constexpr int kPanelPitch = 4;
 struct PanelPlan { int G, R, Rp, variant; size_t smem; bool cl; };
 // ctas == 0: the panel is spread over every SM (short slabs, short passes).  ctas > 0: the panel is
 // confined to that many CTAs so that the other SMs stay free for the GEMM kernels of the look-ahead
@@ -212,11 +215,11 @@ static bool plan_panel_cl(const rrf_ctx* h, long long rows, int b, PanelPlan* p,
   int G = 1;
   while (G < ceil_div(ext, R)) G *= 2;
   if (G > kClusterMax) return false;
-  const size_t extra = (size_t)panel_extra_doubles(b) + (fix ? panel_fix_doubles(b) : 0) + panel_cluster_doubles(b);
+  const size_t extra = (size_t)panel_extra_doubles(b) + panel_work_doubles(b, fix) + panel_cluster_doubles(b);
   if (reg) {
     p->R = R;
     p->G = G;
-    p->Rp = kRegRows + 1;
+    p->Rp = kRegRows + kPanelPitch;
     p->variant = kPanelVariantReg;
     p->cl = true;
     p->smem = ((size_t)b * p->Rp + extra) * sizeof(double);
@@ -226,7 +229,7 @@ static bool plan_panel_cl(const rrf_ctx* h, long long rows, int b, PanelPlan* p,
     if (R > kVariantRows[q]) continue;
     p->R = R;
     p->G = G;
-    p->Rp = kVariantRows[q] + 1;
+    p->Rp = kVariantRows[q] + kPanelPitch;
     p->variant = q;
     p->cl = true;
     p->smem = ((size_t)b * p->Rp + extra) * sizeof(double);
@@ -243,11 +246,11 @@ static bool plan_panel(const rrf_ctx* h, long long rows, int b, PanelPlan* p, in
   p->R = R;
   p->G = ceil_div(ext, R);
   if (p->G > h->sms) return false;
-  const size_t extra = (size_t)panel_extra_doubles(b) + (fix ? panel_fix_doubles(b) : 0);
+  const size_t extra = (size_t)panel_extra_doubles(b) + panel_work_doubles(b, fix) + cqr_dinv_doubles(b);
   for (int q = 0; q < kPanelVariants; ++q) {
     if (R > kVariantRows[q]) continue;
     if (kVariantPad[q]) {
-      p->Rp = kVariantRows[q] + 1;          // odd pitch: the transposing load/store phases stay conflict free
+      p->Rp = kVariantRows[q] + kPanelPitch;
     } else {
       if (fix) continue;
       p->Rp = ((size_t)b * (R | 1) + extra) * sizeof(double) <= (size_t)h->panel_smem_max ? (R | 1) : R;
@@ -368,10 +371,10 @@ static bool plan_blk(const rrf_ctx* h, long long rows, int b, BlkPlan* p, int ct
 // Fewest CTAs whose shared memory holds a rows x b panel with the fix-up staging; 0 if none.
 static int panel_min_ctas(const rrf_ctx* h, long long rows, int b) {
   if (b > 64) return 0;
-  const size_t extra = (size_t)panel_extra_doubles(b) + panel_fix_doubles(b);
+  const size_t extra = (size_t)panel_extra_doubles(b) + panel_work_doubles(b, true) + cqr_dinv_doubles(b);
   int best = 0;
   for (int q = 0; q < kPanelVariants; ++q)
-    if (kVariantPad[q] && ((size_t)b * (kVariantRows[q] + 1) + extra) * sizeof(double) <= (size_t)h->panel_smem_max)
+    if (kVariantPad[q] && ((size_t)b * (kVariantRows[q] + kPanelPitch) + extra) * sizeof(double) <= (size_t)h->panel_smem_max)
       best = std::max(best, kVariantRows[q]);
   return best > 0 ? ceil_div(rows + b, best) : 0;
 }
@@ -429,7 +432,7 @@ struct PassModel {
 static size_t look_scratch_bytes(int b) {   // Gpart[kLookMaxCtas][b*b] + M[b*b]
   return align_up((size_t)(kLookMaxCtas + 1) * b * b * sizeof(double), 256);
 }
-struct PanelScratch { double *P, *piv, *gram, *tau; unsigned* bar; TsqrScratch ts; BlkScratch bk; unsigned* blk_tags; size_t blk_tag_bytes; double* gslab; };
+struct PanelScratch { double *P, *piv, *gram, *tau; unsigned* bar; TsqrScratch ts; BlkScratch bk; unsigned* blk_tags; size_t blk_tag_bytes; double* gslab; double* cqr; };
 // `sms`: the SM count the buffers were sized for (the handle's bound kMaxSms for caller workspaces)
 static PanelScratch carve_panel(unsigned char* base, int sms, int b, bool with_tree = true) {
   PanelScratch s;
@@ -443,10 +446,12 @@ static PanelScratch carve_panel(unsigned char* base, int sms, int b, bool with_t
   s.blk_tags = nullptr;
   s.blk_tag_bytes = 0;
   s.gslab = nullptr;
+  s.cqr = nullptr;
   if (with_tree && b <= kTsqrMaxB) {
     double* t = reinterpret_cast<double*>(base + direct_scratch_bytes(sms, b));
     const size_t blk = (size_t)sms * b * b;
     s.ts = TsqrScratch{t, t + blk, t + 2 * blk, t + 3 * blk};
+    s.cqr = t;            // a run uses the tree kernel or this, never both
   }
   if (with_tree) {
     unsigned char* q = base + direct_scratch_bytes(sms, b) + tsqr_scratch_bytes(sms, b);
@@ -702,7 +707,10 @@ static rrf_status_t launch_panel(rrf_ctx* h, int dtype, const void* Y, PanelSour
   PanelSource alt = o.alt;
   const int* fused_flag = o.fused_flag;
   unsigned bar_base = o.bar_base;
-  void* Tmerged = o.merge_t ? Tout : nullptr;
+  // Cholesky QR first, except for a square panel (its last column has nothing below the pivot: H = I there)
+  double* cqr = (b <= 64 && rows > b && !o.blocked) ? ps.cqr : nullptr;
+  const bool merge_t = o.merge_t || cqr != nullptr;    // it has T at hand
+  void* Tmerged = merge_t ? Tout : nullptr;
   double* csq = o.csq;
   const size_t tsmem = ((size_t)b * (b + 1) + (size_t)(b / 2) * (b / 2 + 1)) * sizeof(double);
   cudaError_t e;
@@ -723,7 +731,7 @@ static rrf_status_t launch_panel(rrf_ctx* h, int dtype, const void* Y, PanelSour
     void* args[] = {&Y, &src, &alt, &fused_flag, &rows_i, &b, &R, &Rp, &RS, &V, &ldv, &gram, &tau, &bk, &seq_base,
                     &ksplit, &c_in_smem, &bar, &ctrl, &done_flag, &fix, &bar_base, &Tmerged, &ldt, &csq, &gslab};
     size_t smem = bp.smem;
-    if (o.merge_t) smem = std::max(smem, tsmem);
+    if (merge_t) smem = std::max(smem, tsmem);
     if (o.bar_used != nullptr) *o.bar_used = (unsigned)(o.fix.enabled ? 2 : 0) * (unsigned)bp.G;
     if (o.g_out != nullptr) *o.g_out = bp.G;
     mark(RRF_PHASE_PANEL, step);
@@ -735,9 +743,9 @@ static rrf_status_t launch_panel(rrf_ctx* h, int dtype, const void* Y, PanelSour
     if (!as_cluster && !plan_panel(h, rows, b, &pp, o.ctas, o.fix.enabled != 0)) return RRF_ERR_WORKSPACE;
     int R = pp.R, Rp = pp.Rp;
     void* args[] = {&Y,   &src, &alt, &fused_flag, &rows_i, &b,    &R,    &Rp,        &V,   &ldv,      &P,
-                    &piv, &gram, &tau, &bar,       &ctrl,   &done_flag, &fix, &bar_base, &Tmerged, &ldt, &csq};
-    if (o.merge_t) pp.smem = std::max(pp.smem, tsmem);
-    if (o.bar_used != nullptr) *o.bar_used = as_cluster ? 0u : (unsigned)(b + (o.fix.enabled ? 2 : 0)) * (unsigned)pp.G;
+                    &piv, &gram, &tau, &bar,       &ctrl,   &done_flag, &fix, &bar_base, &Tmerged, &ldt, &csq, &cqr};
+    if (merge_t) pp.smem = std::max(pp.smem, tsmem);
+    if (o.bar_used != nullptr) *o.bar_used = as_cluster ? 0u : (unsigned)(b + (o.fix.enabled ? 2 : 0) + (cqr != nullptr ? kCqrBarriers : 0)) * (unsigned)pp.G;
     if (o.g_out != nullptr) *o.g_out = pp.G;
     mark(RRF_PHASE_PANEL, step);
     if (as_cluster) {
@@ -760,7 +768,8 @@ static rrf_status_t launch_panel(rrf_ctx* h, int dtype, const void* Y, PanelSour
       e = cudaLaunchCooperativeKernel(fn, dim3(pp.G), dim3(kPanelThreads), args, pp.smem, st);
     }
   }
-  if (e == cudaSuccess && !o.merge_t) {
+  if (e == cudaSuccess && merge_t && o.ev_join != nullptr) cudaEventRecord(o.ev_join, st);   // T is ready when the panel kernel is
+  if (e == cudaSuccess && !merge_t) {
     cudaStream_t tt = st;
     if (o.ev_fork != nullptr) {          // fork: the T factor runs on the side stream after the panel
       cudaEventRecord(o.ev_fork, st);

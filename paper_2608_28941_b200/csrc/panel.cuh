@@ -2,146 +2,9 @@
 // kernels around it: compact-WY T factor, Z <- op(T) Z, norms, stop rule, Gaussian fill.
 #pragma once
 
-#include "common.cuh"
+#include "panel_cqr.cuh"
 
 namespace rrf {
-
-constexpr int kPanelThreads = 512;
-constexpr int kPanelMaxG = 160;   // most CTAs a panel grid may have (one per SM)
-// doubles of shared memory the panel kernel needs besides the slab: w[b], p[2][b], pivot_row[b], scalars
-__host__ __device__ constexpr int panel_extra_doubles(int b) { return 4 * b + 4; }
-
-// Grid-wide barrier over a monotonically increasing arrival counter.  Needs all CTAs
-// co-resident (cooperative launch).  Bounded: gives up after kWaitLimitClocks.
-__device__ __forceinline__ bool grid_barrier(unsigned* ctr, unsigned target, Ctrl* ctrl,
-                                             long long limit = kWaitLimitClocks) {
-  __shared__ int ok_s;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    __threadfence();
-    atomicAdd(ctr, 1u);
-    int ok = 1;
-    const long long t0 = clock64();
-    while (true) {
-      unsigned v;
-      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(ctr) : "memory");
-      if (v >= target) break;
-      if (clock64() - t0 > limit) {
-        atomicExch(&ctrl->status, (int)RRF_ERR_TIMEOUT);
-        atomicExch(&ctrl->done, 1);        // kernels already enqueued behind this one return at once
-        ok = 0;
-        break;
-      }
-    }
-    ok_s = ok;
-  }
-  __syncthreads();
-  return ok_s != 0;
-}
-
-// ---------------------------------------------------------------- thread-block cluster exchange
-// A panel that fits the shared memory of at most 16 CTAs is factored by ONE cluster: the per-column sums
-// travel through distributed shared memory (every CTA writes its partials straight into every peer's
-// shared memory) and the barrier is an mbarrier per CTA on which every peer arrives - about 0.7 to 1 us per
-// column against the 2.4 us of an all-to-all exchange through L2.
-constexpr int kClusterMax = 16;
-#ifdef RRF_TSQR_TRACE
-__device__ unsigned long long g_pcl_trace[16];
-#define PCL_STAMP(k) if (j == 8 && blockIdx.x == 0 && threadIdx.x == 0) g_pcl_trace[k] = (unsigned long long)clock64()
-#else
-#define PCL_STAMP(k)
-#endif
-constexpr int kRegRows = 256;       // rows of a slab in the register-resident column loop
-// px [2][kClusterMax][2b], prx [2][b], ycol/vcol [kRegRows] each, prow [b], send buffers [2][2b]
-__host__ __device__ constexpr int panel_cluster_doubles(int b) {
-  return 2 * kClusterMax * 2 * b + 2 * b + 2 * kRegRows + b + 4 * b;
-}
-// One bulk copy from this CTA's shared memory into a peer's, which also counts its bytes on the peer's mbarrier:
-// data and signal in one message.
-__device__ __forceinline__ void cl_bulk_send(uint32_t dst_cluster, uint32_t src_cta, uint32_t bytes, uint32_t bar_cluster) {
-  asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-               ::"r"(dst_cluster), "r"(src_cta), "r"(bytes), "r"(bar_cluster)
-               : "memory");
-}
-
-__device__ __forceinline__ void proxy_fence_smem_async() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
-__device__ __forceinline__ uint32_t cl_map(uint32_t addr, uint32_t rank) {   // the same address in CTA `rank` of the cluster
-  uint32_t r;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
-  return r;
-}
-__device__ __forceinline__ void cl_st(uint32_t addr, double v) {
-  asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(addr), "d"(v) : "memory");
-}
-__device__ __forceinline__ void cl_st(uint32_t addr, int v) {
-  asm volatile("st.shared::cluster.b32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
-}
-__device__ __forceinline__ void cl_arrive(uint32_t bar_addr) {
-  asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar_addr) : "memory");
-}
-__device__ __forceinline__ uint32_t cl_try_wait(uint64_t* bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
-      "selp.u32 %0, 1, 0, p;\n\t}"
-      : "=r"(ok)
-      : "r"(smem_u32(bar)), "r"(parity)
-      : "memory");
-  return ok;
-}
-// the hardware barrier of the cluster (unbounded: used once, before any data-dependent exit)
-__device__ __forceinline__ void cl_hw_sync() {
-  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-// Barrier over the G CTAs of the cluster: every CTA arrives on every peer's mbarrier and waits, bounded, on its
-// own.  Everything this CTA stored before it - into peers' shared memory, or (with `global_too`) into global
-// memory - is visible to the peers behind it.  `nx` counts the barriers passed (the phase parity).
-__device__ __forceinline__ bool cluster_barrier(uint64_t* cbar, unsigned& nx, int G, bool global_too, Ctrl* ctrl) {
-  __shared__ int cl_ok_s;
-  __syncthreads();
-  if ((int)threadIdx.x < G) {
-    if (global_too) __threadfence();
-    cl_arrive(cl_map(smem_u32(cbar), threadIdx.x));
-  }
-  if (threadIdx.x == 0) {
-    int ok = 1;
-    if (!cl_try_wait(cbar, nx & 1u)) {
-      const long long t0 = clock64();
-      while (!cl_try_wait(cbar, nx & 1u)) {
-        if (clock64() - t0 > kWaitLimitClocks) {
-          atomicExch(&ctrl->status, (int)RRF_ERR_TIMEOUT);
-          atomicExch(&ctrl->done, 1);
-          ok = 0;
-          break;
-        }
-      }
-    }
-    cl_ok_s = ok;
-  }
-  ++nx;
-  __syncthreads();
-  return cl_ok_s != 0;
-}
-
-// Sums four per-lane values over the warp with 6 adds and 6 shuffles instead of 20: after the
-// exchanges with lanes ^16 and ^8 every lane carries one of the four sums (number 2*bit4 + bit3 of
-// its lane index), which three more butterfly steps complete.  Fixed order, so reproducible.
-__device__ __forceinline__ double warp_sum4(const double (&v)[4], int lane) {
-  const bool hi = lane & 16;
-  double a0 = hi ? v[2] : v[0], a1 = hi ? v[3] : v[1];
-  const double s0 = hi ? v[0] : v[2], s1 = hi ? v[1] : v[3];
-  a0 += __shfl_xor_sync(0xffffffffu, s0, 16);
-  a1 += __shfl_xor_sync(0xffffffffu, s1, 16);
-  const bool mid = lane & 8;
-  double k = mid ? a1 : a0;
-  const double snd = mid ? a0 : a1;
-  k += __shfl_xor_sync(0xffffffffu, snd, 8);
-  k += __shfl_xor_sync(0xffffffffu, k, 4);
-  k += __shfl_xor_sync(0xffffffffu, k, 2);
-  k += __shfl_xor_sync(0xffffffffu, k, 1);
-  return k;
-}
 
 // Self test of the bounded wait: one CTA arrives at a barrier that expects two.
 __global__ void __launch_bounds__(32) timeout_selftest_kernel(unsigned* ctr, Ctrl* ctrl, long long limit) {
@@ -193,6 +56,11 @@ constexpr int kFixChunk = 32;   // rows of Vp staged in shared memory at a time
 // doubles of shared memory the fix-up needs on top of panel_extra_doubles: the staged rows of Vp
 // (pitch b + 8 or b + 4) and a b x (b + 8) matrix (Tp, then M)
 __host__ __device__ constexpr int panel_fix_doubles(int b) { return kFixChunk * (b + 8) + b * (b + 8); }
+
+// doubles of that staging area, which the Cholesky QR uses after it
+__host__ __device__ constexpr int panel_work_doubles(int b, bool fix) {
+  return fix && panel_fix_doubles(b) > cqr_work_doubles(b) ? panel_fix_doubles(b) : cqr_work_doubles(b);
+}
 
 template <typename T>
 __device__ __forceinline__ double panel_entry(const T* __restrict__ Y, const PanelSource& src, int r, int c, int b) {
@@ -361,7 +229,8 @@ __global__ void __launch_bounds__(kPanelThreads)
                  unsigned* bar, Ctrl* ctrl, const int* done_flag, PanelFix fix,
                  unsigned bar_base,                 // value of the barrier counter when this launch starts
                  T* __restrict__ Tout, long long ldt,     // non-NULL: CTA 0 also builds the T factor at the end
-                 double* __restrict__ csq) {              // non-NULL: [b][Gp] per-CTA sums of squares of the panel's columns
+                 double* __restrict__ csq,                // non-NULL: [b][Gp] per-CTA sums of squares of the panel's columns
+                 double* __restrict__ cqr) {              // non-NULL: scratch of the Cholesky QR (panel_cqr.cuh), tried first
   __shared__ uint64_t cbar;      // cluster mode: this CTA's barrier, on which every CTA of the cluster arrives
   __shared__ uint64_t xbar[2];   // ... and the two on which the per-column messages of the peers are counted
   __shared__ int go_s;
@@ -397,7 +266,8 @@ __global__ void __launch_bounds__(kPanelThreads)
   double* pr_s = p_s + 2 * b;             // [b]
   double* sc_s = pr_s + b;                // [4]: tau_j, 1/(alpha - beta)
   // cluster mode: partial sums [2][kClusterMax][b] and pivot rows [2][b] written by the peers, behind everything else
-  double* px_s = sc_s + 4 + (fix.enabled ? panel_fix_doubles(b) : 0);
+  double* work_s = sc_s + 4;              // staging of the fix-up, then the small matrices of the Cholesky QR
+  double* px_s = work_s + panel_work_doubles(b, fix.enabled);
   double* prx_s = px_s + 2 * kClusterMax * 2 * b;
   double* ycol_s = prx_s + 2 * b;         // [kRegRows] column j below its pivot (register-resident loop)
   double* vcol_s = ycol_s + kRegRows;     // [kRegRows] v_{j-1}
@@ -506,7 +376,7 @@ __global__ void __launch_bounds__(kPanelThreads)
       }
     }
     if (CL) {
-      if (!cluster_barrier(&cbar, nx, G, true, ctrl)) return;
+      if (!cluster_barrier(&cbar, nx, G, ctrl)) return;
     } else if (!grid_barrier(bar, bar_base + (++nbar) * (unsigned)G, ctrl)) return;
     // Phase 2: CTA c owns columns c, c + G, ... of G = sum of the partials (in CTA order) and of
     // M = Tp^T G, column by column: M[k][c2] = sum_{l <= k} Tp[l][k] G[l][c2].
@@ -546,7 +416,7 @@ __global__ void __launch_bounds__(kPanelThreads)
       }
     }
     if (CL) {
-      if (!cluster_barrier(&cbar, nx, G, true, ctrl)) return;
+      if (!cluster_barrier(&cbar, nx, G, ctrl)) return;
     } else if (!grid_barrier(bar, bar_base + (++nbar) * (unsigned)G, ctrl)) return;
     // Phase 3: S -= Vp[slab] M.  A task is a 16-row x 8-column tile of a chunk.
     {
@@ -595,8 +465,36 @@ __global__ void __launch_bounds__(kPanelThreads)
     }
   }
 
+  // Cholesky QR with reconstruction where it is safe; the column loop below does the rest
+  const bool try_cqr = PAD && (!CL || REG) && cqr != nullptr && b <= 64 && rows > b;
+  bool have_v = false;
+  if constexpr (PAD && (!CL || REG)) {
+    if (try_cqr) {
+      CqrArgs ca;
+      ca.S = S; ca.Rp = Rp; ca.nloc = nloc; ca.gr0 = gr0; ca.row0 = row0;
+      ca.work = work_s;
+      // cluster: the peers' sums arrive in the message buffers of the column loop; the inverted blocks lie in the half
+      // of them that no peer writes before this CTA has sent its first column
+      ca.rbuf = px_s;
+      ca.dinv = CL ? px_s + max(kClusterMax * 2 * b, cqr_entries(b)) : px_s;
+      ca.small = w_s;
+      ca.gpart = cqr;
+      ca.gsum = cqr + (size_t)G * cqr_entries(b);
+      ca.gtop = ca.gsum + cqr_entries(b);
+      ca.G = G; ca.cta = cta; ca.bar = bar; ca.bar_base = bar_base; ca.nbar = &nbar; ca.cbar = &cbar; ca.nx = &nx; ca.ctrl = ctrl;
+      ca.want_t = Tout != nullptr && cta == G - 1;
+      ca.single = sizeof(T) == 4;
+      ca.vec = (reinterpret_cast<uintptr_t>(V) & (2 * sizeof(T) - 1)) == 0 && (ldv & 1) == 0;
+      ca.V = V; ca.ldv = ldv; ca.T = Tout; ca.ldt = ldt;
+      const int got = b == 64 ? cqr_panel<64, CL>(ca) : (b == 32 ? cqr_panel<32, CL>(ca) : cqr_panel<16, CL>(ca));
+      if (got < 0) return;
+      have_v = got > 0;
+    }
+  }
+
   double tau_prev = 0.0;
-  if constexpr (CL && REG) {
+  if (have_v) {
+  } else if constexpr (CL && REG) {
     static_assert(QMAX == 8 && RH == 1 && PAD, "the register tile is 8 rows x 4 columns per thread");
     const bool has = warp < (b >> 2);                  // warps that hold columns
     const int c0 = warp * 4;
@@ -839,7 +737,7 @@ __global__ void __launch_bounds__(kPanelThreads)
           const int q = idx >> lb, c = idx & (b - 1);
           cl_st(cl_map(smem_u32(prx_s + pb * b + c), q), S[(size_t)c * Rp + (pr - gr0)]);
         }
-      if (!cluster_barrier(&cbar, nx, G, false, ctrl)) return;
+      if (!cluster_barrier(&cbar, nx, G, ctrl)) return;
       if (tid < b) {
         double v = 0.0;
         for (int q = 0; q < G; ++q) v += px_s[((size_t)pb * kClusterMax + q) * 2 * b + tid];     // CTA order: reproducible
@@ -924,14 +822,21 @@ __global__ void __launch_bounds__(kPanelThreads)
     __syncthreads();
   }
 
-  for (int idx = tid; idx < nloc * b; idx += NT) {
-    const int r = idx >> lb, c = idx & (b - 1);
-    if (gr0 + r >= row0) V[(size_t)(gr0 + r - row0) * ldv + c] = (T)S[(size_t)c * Rp + r];
+  if (!have_v) {
+    for (int idx = tid; idx < nloc * b; idx += NT) {
+      const int r = idx >> lb, c = idx & (b - 1);
+      if (gr0 + r >= row0) V[(size_t)(gr0 + r - row0) * ldv + c] = (T)S[(size_t)c * Rp + r];
+    }
+    // CTA 0 wrote the Gram rows and tau itself: it can go on to the T factor without another launch
+    if (Tout != nullptr && cta == 0) {
+      __syncthreads();
+      tfactor_block<T>(gram, tau_out, b, Tout, ldt, psm);
+    }
   }
-  // CTA 0 wrote the Gram rows and tau itself: it can go on to the T factor without another launch
-  if (Tout != nullptr && cta == 0) {
-    __syncthreads();
-    tfactor_block<T>(gram, tau_out, b, Tout, ldt, psm);
+  // the barrier counter moves on by the same amount whichever way the panel was factored
+  if (!CL && tid == 0) {
+    const unsigned total = (unsigned)b + (fix.enabled ? 2u : 0u) + (try_cqr ? (unsigned)kCqrBarriers : 0u);
+    if (total > nbar) atomicAdd(bar, total - nbar);
   }
 }
 

@@ -1,0 +1,101 @@
+"""Panels through the Cholesky QR with Householder reconstruction, and those it hands to the column loop.
+
+The factors are held to the oracle's within c u cond, the first-order perturbation bound of a QR factorisation (u the
+unit round-off, cond the condition number of the panel with its columns scaled to unit length, which is what both
+factorisations see; c = 100 covers the sums over b columns).
+"""
+import numpy as np
+import pytest
+import torch
+
+from oracle import rrf_oracle as orc
+from paper_2608_28941_b200 import rrf
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def h():
+    handle = rrf.rrf_create(0)
+    yield handle
+    rrf.rrf_destroy(handle)
+
+
+def panel(kind, rows, b, rng):
+    Y = rng.standard_normal((rows, b))
+    if kind.startswith("cond"):                    # singular values from 1 down to 10^-x
+        s = 10.0 ** (-float(kind[4:]) * np.arange(b) / (b - 1))
+        Y = (np.linalg.qr(Y)[0] * s) @ rng.standard_normal((b, b))
+    elif kind == "graded":                         # columns of very different lengths
+        Y *= 10.0 ** (-12.0 * np.arange(b) / (b - 1))
+    elif kind == "dependent":                      # column loop: two equal columns
+        Y[:, b // 2] = Y[:, 1]
+    elif kind == "zero":                           # column loop: a column of zeros
+        Y[:, 3] = 0.0
+    elif kind == "nothing-below":                  # column loop, on the orthonormal panel: tau = 0 in some columns
+        Y[b:] = 0.0
+        Y[:b] = np.triu(Y[:b]) + 3.0 * np.eye(b)
+    elif kind == "huge":                           # column loop: squares overflow
+        Y *= 1e160
+    return Y
+
+
+def check(h, Y, dtype, c=100.0):
+    rows, b = Y.shape
+    Y = Y.astype(np.float32).astype(np.float64) if dtype == "f32" else Y
+    V, T = rrf.rrf_panel_qr(h, torch.from_numpy(Y.astype(np.float32) if dtype == "f32" else Y).cuda())
+    assert rrf.rrf_last_status(h) == rrf.RRF_OK
+    V, T = V.cpu().numpy().astype(np.float64), T.cpu().numpy().astype(np.float64)
+    Vo, _, To, _ = orc.panel_qr(Y)
+    norms = np.linalg.norm(Y, axis=0)
+    s = np.linalg.svd(Y / np.where(norms > 0, norms, 1.0), compute_uv=False)
+    cond = s[0] / s[-1] if s[-1] > 1e-12 * s[0] else None
+    store = 2.0 ** -24 if dtype == "f32" else 0.0
+    Q = np.eye(rows, b) - V @ (T @ V[:b].T)
+    assert np.linalg.norm(Q.T @ Q - np.eye(b)) <= (5e-6 if dtype == "f32" else 1e-13) * b
+    if cond is not None:
+        tol = c * 1.1e-16 * cond + store
+        assert np.max(np.abs(V - Vo)) <= tol * np.max(np.abs(Vo))
+        assert np.max(np.abs(T - To)) <= 10 * tol * np.max(np.abs(To))
+    return V, T
+
+
+@pytest.mark.parametrize("b", [16, 32, 64])
+@pytest.mark.parametrize("extra", [1, 7, 48, 65, 1023, 3072, 4097, 9000])
+def test_heights(h, b, extra):
+    """One row more than columns, strips of 16 and slabs that end in a remainder, one cluster and the whole grid."""
+    rows = b + extra
+    check(h, panel("gauss", rows, b, np.random.default_rng(rows)), "f64")
+
+
+@pytest.mark.parametrize("b", [16, 32, 64])
+@pytest.mark.parametrize("rows", [700, 6000])
+@pytest.mark.parametrize("kind", ["cond3", "cond6", "cond7", "cond9", "graded", "dependent", "zero", "nothing-below"])
+def test_conditioning(h, b, rows, kind):
+    """First-order and full second factorisation, and every way into the column loop."""
+    Y = panel(kind, rows, b, np.random.default_rng(rows + b))
+    V, T = check(h, Y, "f64")
+    if kind == "nothing-below":      # nothing to annihilate: H = I for every column, as in LAPACK
+        assert not T.any()
+        assert np.array_equal(V, np.eye(rows, b))
+
+
+@pytest.mark.parametrize("b", [32, 64])
+@pytest.mark.parametrize("rows", [100, 2049, 7001])
+def test_single_precision(h, b, rows):
+    check(h, panel("gauss", rows, b, np.random.default_rng(rows)), "f32")
+
+
+@pytest.mark.parametrize("zero", [0.0, -0.0])
+@pytest.mark.parametrize("rows,b", [(500, 16), (9000, 64)])
+def test_zero_first_pivot_keeps_its_sign(h, rows, b, zero):
+    Y = panel("gauss", rows, b, np.random.default_rng(5))
+    Y[0, 0] = zero
+    check(h, Y, "f64")
+
+
+def test_squares_that_overflow(h):
+    """The column loop's sums of squares overflow too; all that is asked is that the call ends and the context lives."""
+    rrf.rrf_panel_qr(h, torch.from_numpy(panel("huge", 900, 32, np.random.default_rng(1))).cuda())
+    torch.cuda.synchronize()
+    check(h, panel("gauss", 900, 32, np.random.default_rng(2)), "f64")
