@@ -80,56 +80,92 @@ __device__ __forceinline__ double panel_entry(const T* __restrict__ Y, const Pan
   return s;
 }
 
-// The same sums for a whole slab, S[c][r] (pitch Rp) = entry (gr0 + r - row0, c), with the loads of eight entries
-// in flight per thread: the terms of one entry are a dependent chain of global loads (up to a dozen partial
-// panels), and a CTA that holds a tall slab has dozens of entries per thread.  Same order of additions as
-// panel_entry, so the same bits.
+// The same sums for a whole slab, S[c][r] (pitch Rp) = entry (gr0 + r - row0, c), in the same order of additions, so
+// the same bits.  The terms of an entry are a dependent chain of global loads (up to a dozen partial panels), and a
+// confined panel has dozens of entries per thread: 16-byte loads, 64 KB of them in flight per CTA, and where a slab's
+// partial results lie is worked out once per slab and not per entry (26 CTAs x 320 rows x 64 spent 120 us here beside
+// the GEMM kernels, most of it on four integer divisions per entry).  A warp takes tiles of eight rows x four vectors:
+// whole 64-byte pieces of the rows, and shared-memory stores without bank conflicts at a pitch of 4 mod 16.
 template <typename T>
 __device__ __forceinline__ void panel_load_slab(const T* __restrict__ Y, const PanelSource& src, double* __restrict__ S, int Rp,
                                                 int nloc, int b, int lb, int gr0, int row0, int tid, int nthr) {
-  constexpr int E = 8;
-  const int total = nloc * b;
+  constexpr int VEC = 16 / (int)sizeof(T), E = 16 / VEC;
+  __shared__ int2 tab[16];                 // slots: index of the first partial result of a row slab, and how many
+  const int lr0 = gr0 - row0 + src.row_off;
+  const int sbm = src.slots ? 31 - __clz(src.bm) : 0;      // slab heights are powers of two
+  const int sl0 = src.slots ? lr0 >> sbm : 0;
+  if (src.slots && nloc > 0 && tid <= ((lr0 + nloc - 1) >> sbm) - sl0) {
+    const int sl = sl0 + tid;
+    const int p_lo = slot_cta(src, sl * src.nc), p_hi = slot_cta(src, (sl + 1) * src.nc - 1);
+    tab[tid] = make_int2((p_lo + sl) * src.wn, (p_hi - p_lo + 1) * src.wn);
+  }
+  __syncthreads();
   const size_t tstride = src.slots ? (size_t)src.bm * b : (size_t)src.seg_stride;
-  for (int base = tid; base < total; base += E * nthr) {
-    const T* ptr[E];
-    int cnt[E];
-    double v[E];
-    int maxcnt = 0;
+  if ((reinterpret_cast<uintptr_t>(Y) & 15) == 0 && (src.slots || (src.ldy % VEC == 0 && src.seg_stride % VEC == 0))) {
+    struct __align__(16) Vec { T v[VEC]; };
+    const int lane = tid & 31, nw = nthr >> 5;
+    const int lcb = lb - (sizeof(T) == 8 ? 3 : 4);         // log2 of the tiles across a row
+    const int ntile = ((nloc + 7) >> 3) << lcb;
+    for (int base = tid >> 5; base < ntile; base += E * nw) {
+      const T* ptr[E];
+      int cnt[E], at[E];
+      double v[E][VEC];
+      int maxcnt = 0;
 #pragma unroll
-    for (int e = 0; e < E; ++e) {
-      const int idx = base + e * nthr;
-      const int r = idx >> lb, c = idx & (b - 1);
-      cnt[e] = 0;
-      ptr[e] = Y;
-      if (idx < total) {
-        const int lr = gr0 + r - row0 + src.row_off;
-        if (src.slots) {
-          const int sl = lr / src.bm, rl = lr - sl * src.bm;
-          const int p_lo = slot_cta(src, sl * src.nc), p_hi = slot_cta(src, (sl + 1) * src.nc - 1);
-          cnt[e] = (p_hi - p_lo + 1) * src.wn;
-          ptr[e] = Y + (size_t)(p_lo + sl) * src.wn * tstride + (size_t)rl * b + c;
-        } else {
-          cnt[e] = src.nseg;
-          ptr[e] = Y + (size_t)lr * src.ldy + c;
+      for (int e = 0; e < E; ++e) {
+        const int tile = base + e * nw;
+        const int r = (tile >> lcb) * 8 + (lane & 7), c = ((tile & ((1 << lcb) - 1)) * 4 + (lane >> 3)) * VEC;
+        cnt[e] = 0;
+        ptr[e] = Y;
+        at[e] = c * Rp + r;
+        if (tile < ntile && r < nloc) {
+          const int lr = lr0 + r;
+          if (src.slots) {
+            const int2 s = tab[(lr >> sbm) - sl0];
+            cnt[e] = s.y;
+            ptr[e] = Y + (size_t)s.x * tstride + (size_t)(lr & (src.bm - 1)) * b + c;
+          } else {
+            cnt[e] = src.nseg;
+            ptr[e] = Y + (size_t)lr * src.ldy + c;
+          }
         }
+        maxcnt = max(maxcnt, cnt[e]);
       }
-      maxcnt = max(maxcnt, cnt[e]);
-    }
-#pragma unroll
-    for (int e = 0; e < E; ++e) {
-      const double first = cnt[e] > 0 ? (double)ptr[e][0] : 0.0;
-      v[e] = src.slots ? 0.0 + first : first;      // as panel_entry: a lone -0.0 of a stacked panel keeps its sign
-    }
-    for (int t = 1; t < maxcnt; ++t) {
+      Vec x[E];
 #pragma unroll
       for (int e = 0; e < E; ++e)
-        if (t < cnt[e]) v[e] += (double)ptr[e][(size_t)t * tstride];
-    }
+        if (cnt[e] > 0) x[e] = *reinterpret_cast<const Vec*>(ptr[e]);
 #pragma unroll
-    for (int e = 0; e < E; ++e) {
-      const int idx = base + e * nthr;
-      if (idx < total) S[(size_t)(idx & (b - 1)) * Rp + (idx >> lb)] = v[e];
+      for (int e = 0; e < E; ++e)
+#pragma unroll
+        for (int u = 0; u < VEC; ++u) {
+          const double first = cnt[e] > 0 ? (double)x[e].v[u] : 0.0;
+          v[e][u] = src.slots ? 0.0 + first : first;       // as panel_entry: a lone -0.0 of a stacked panel keeps its sign
+        }
+      for (int t = 1; t < maxcnt; ++t) {
+#pragma unroll
+        for (int e = 0; e < E; ++e)
+          if (t < cnt[e]) x[e] = *reinterpret_cast<const Vec*>(ptr[e] + (size_t)t * tstride);
+#pragma unroll
+        for (int e = 0; e < E; ++e)
+          if (t < cnt[e]) {
+#pragma unroll
+            for (int u = 0; u < VEC; ++u) v[e][u] += (double)x[e].v[u];
+          }
+      }
+#pragma unroll
+      for (int e = 0; e < E; ++e)
+        if (cnt[e] > 0) {
+#pragma unroll
+          for (int u = 0; u < VEC; ++u) S[at[e] + u * Rp] = v[e][u];
+        }
     }
+    return;
+  }
+  // a caller's panel whose rows do not start on 16-byte boundaries
+  for (int idx = tid; idx < nloc * b; idx += nthr) {
+    const int r = idx >> lb, c = idx & (b - 1);
+    S[(size_t)c * Rp + r] = panel_entry<T>(Y, src, gr0 + r - row0, c, b);
   }
 }
 
@@ -470,25 +506,30 @@ __global__ void __launch_bounds__(kPanelThreads)
   bool have_v = false;
   if constexpr (PAD && (!CL || REG)) {
     if (try_cqr) {
-      CqrArgs ca;
-      ca.S = S; ca.Rp = Rp; ca.nloc = nloc; ca.gr0 = gr0; ca.row0 = row0;
-      ca.work = work_s;
-      // cluster: the peers' sums arrive in the message buffers of the column loop; the inverted blocks lie in the half
-      // of them that no peer writes before this CTA has sent its first column
-      ca.rbuf = px_s;
-      ca.dinv = CL ? px_s + max(kClusterMax * 2 * b, cqr_entries(b)) : px_s;
-      ca.small = w_s;
-      ca.gpart = cqr;
-      ca.gsum = cqr + (size_t)G * cqr_entries(b);
-      ca.gtop = ca.gsum + cqr_entries(b);
-      ca.G = G; ca.cta = cta; ca.bar = bar; ca.bar_base = bar_base; ca.nbar = &nbar; ca.cbar = &cbar; ca.nx = &nx; ca.ctrl = ctrl;
-      ca.want_t = Tout != nullptr && cta == G - 1;
-      ca.single = sizeof(T) == 4;
-      ca.vec = (reinterpret_cast<uintptr_t>(V) & (2 * sizeof(T) - 1)) == 0 && (ldv & 1) == 0;
-      ca.V = V; ca.ldv = ldv; ca.T = Tout; ca.ldt = ldt;
+      __shared__ CqrArgs ca;
+      if (tid == 0) {
+        ca.S = S; ca.Rp = Rp; ca.nloc = nloc; ca.gr0 = gr0; ca.row0 = row0;
+        ca.work = work_s;
+        // cluster: the peers' sums arrive in the message buffers of the column loop; the inverted blocks lie in the half
+        // of them that no peer writes before this CTA has sent its first column
+        ca.rbuf = px_s;
+        ca.dinv = CL ? px_s + max(kClusterMax * 2 * b, cqr_entries(b)) : px_s;
+        ca.small = w_s;
+        ca.gpart = cqr;
+        ca.gsum = cqr + (size_t)G * cqr_entries(b);
+        ca.gtop = ca.gsum + cqr_entries(b);
+        ca.G = G; ca.cta = cta; ca.bar = bar; ca.bar_base = bar_base; ca.nbar = nbar; ca.cbar = &cbar; ca.nx = nx; ca.ctrl = ctrl;
+        ca.want_t = Tout != nullptr && cta == G - 1;
+        ca.single = sizeof(T) == 4;
+        ca.vec = (reinterpret_cast<uintptr_t>(V) & (2 * sizeof(T) - 1)) == 0 && (ldv & 1) == 0;
+        ca.V = V; ca.ldv = ldv; ca.T = Tout; ca.ldt = ldt;
+      }
+      __syncthreads();
       const int got = b == 64 ? cqr_panel<64, CL>(ca) : (b == 32 ? cqr_panel<32, CL>(ca) : cqr_panel<16, CL>(ca));
       if (got < 0) return;
-      have_v = got > 0;
+      have_v = got & 1;
+      if (CL) nx += (unsigned)got >> 1;
+      else nbar += (unsigned)got >> 1;
     }
   }
 

@@ -84,9 +84,9 @@ struct CqrArgs {
   int G, cta;
   unsigned* bar;
   unsigned bar_base;
-  unsigned* nbar;       // grid barriers passed so far
+  unsigned nbar;        // grid barriers passed before the call
   uint64_t* cbar;
-  unsigned* nx;         // cluster barriers passed so far
+  unsigned nx;          // cluster barriers passed before the call
   Ctrl* ctrl;
   bool want_t;          // this CTA writes T
   bool single, vec;     // V and T are single precision; two elements of a row of V can be stored at once
@@ -344,6 +344,7 @@ __device__ __noinline__ void cqr_gram(const double* __restrict__ S, int Rp, int 
 // b x b block the CTAs left in a.gtop is loaded behind the first step.  Returns false when a wait gave up.
 template <int B, bool CL>
 __device__ __forceinline__ bool cqr_reduce(const CqrArgs& a, bool top, int tid) {
+  unsigned nb = top ? 2 : 0, nx = a.nx + nb;      // barriers of this call so far
   using C = Cqr<B>;
   constexpr int NT = 512;
   auto mine = [&](int e) {
@@ -358,7 +359,7 @@ __device__ __forceinline__ bool cqr_reduce(const CqrArgs& a, bool top, int tid) 
       const int owner = e / epc;
       cl_st(cl_map(smem_u32(a.rbuf + a.cta * epc + (e - owner * epc)), owner), mine(e));
     }
-    if (!cluster_barrier(a.cbar, *a.nx, a.G, a.ctrl)) return false;
+    if (!cluster_barrier(a.cbar, nx, a.G, a.ctrl)) return false;
     const int e0 = a.cta * epc, ne = min(epc, C::E - e0);
     double* own = a.work;       // every CTA has read its partial triangles: the peers may write sums there
     for (int e = tid; e < ne; e += NT) {
@@ -370,10 +371,10 @@ __device__ __forceinline__ bool cqr_reduce(const CqrArgs& a, bool top, int tid) 
       double* A = a.work + C::E;
       for (int idx = tid; idx < B * B; idx += NT) A[(idx / B) * C::PA + (idx & (B - 1))] = __ldcg(a.gtop + idx);
     }
-    return cluster_barrier(a.cbar, *a.nx, a.G, a.ctrl);
+    return cluster_barrier(a.cbar, nx, a.G, a.ctrl);
   } else {
     for (int e = tid; e < C::E; e += NT) a.gpart[(size_t)a.cta * C::E + e] = mine(e);
-    if (!grid_barrier(a.bar, a.bar_base + (++*a.nbar) * (unsigned)a.G, a.ctrl)) return false;
+    if (!grid_barrier(a.bar, a.bar_base + (a.nbar + ++nb) * (unsigned)a.G, a.ctrl)) return false;
     const int e0 = a.cta * epc, ne = min(epc, C::E - e0);
     if (ne > 0) {
       int tpe = 1;                              // threads that share an entry
@@ -410,7 +411,7 @@ __device__ __forceinline__ bool cqr_reduce(const CqrArgs& a, bool top, int tid) 
         }
       }
     }
-    if (!grid_barrier(a.bar, a.bar_base + (++*a.nbar) * (unsigned)a.G, a.ctrl)) return false;
+    if (!grid_barrier(a.bar, a.bar_base + (a.nbar + ++nb) * (unsigned)a.G, a.ctrl)) return false;
     for (int e = tid; e < C::E; e += NT) a.work[e] = __ldcg(a.gsum + e);
     if (top) {
       double* A = a.work + C::E;
@@ -578,9 +579,12 @@ __device__ __forceinline__ void cqr_put(void* base, size_t at, double v0, double
   }
 }
 
-// The whole of it, called by every thread of every CTA with the panel in the slabs.  1: V and T are written; 0: the column loop has to do it, on what the slabs hold; -1: a wait gave up.
+// The whole of it, called by every thread of every CTA with the panel in the slabs; the arguments lie in shared memory
+// (on the stack they go through what is left of the L1: 4 us a call).  Negative: a wait gave up.  Else bit 0 says
+// whether V and T are written (if not, the column loop has to do it, on what the slabs hold) and the rest is the
+// number of barriers passed.
 template <int B, bool CL>
-__device__ __noinline__ int cqr_panel(const CqrArgs a) {
+__device__ __noinline__ int cqr_panel(const CqrArgs& a) {
   using C = Cqr<B>;
   constexpr int NB = C::NB, PA = C::PA;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
@@ -596,7 +600,7 @@ __device__ __noinline__ int cqr_panel(const CqrArgs a) {
   __syncthreads();
   cqr_gram<B>(a.S, Rp, a.nloc, a.work, tid);
   if (!cqr_reduce<B, CL>(a, false, tid)) return -1;
-  if (!cqr_chol<B>(M, dinv_r, small, kCqrPivot, tid)) return 0;
+  if (!cqr_chol<B>(M, dinv_r, small, kCqrPivot, tid)) return 2 << 1;
 
   const bool has00 = row0 >= a.gr0 && row0 < a.gr0 + a.nloc;
   const double y00 = has00 ? a.S[row0 - a.gr0] : 0.0;
@@ -663,9 +667,9 @@ __device__ __noinline__ int cqr_panel(const CqrArgs a) {
     if (far) defect_s[1] = 1;
   }
   __syncthreads();
-  if (defect_s[1]) return 0;
+  if (defect_s[1]) return 4 << 1;
   if (defect_s[0]) {
-    if (!cqr_chol<B>(M, dinv_r, small, 0.25, tid)) return 0;
+    if (!cqr_chol<B>(M, dinv_r, small, 0.25, tid)) return 4 << 1;
   } else {
     if (tid < B) {
       double* d = M + cqr_blk(tid >> 3, tid >> 3) + (tid & 7) * 9;
@@ -675,7 +679,7 @@ __device__ __noinline__ int cqr_panel(const CqrArgs a) {
   }
   double* sgn = small + 2 * B;
   double* rinv = small + 3 * B;
-  if (!cqr_lu<B>(A, M, sgn, rinv, tid)) return 0;
+  if (!cqr_lu<B>(A, M, sgn, rinv, tid)) return 4 << 1;
 
   // the inverted diagonal blocks the products below need: of U', and for T of R2 and V1^T (the latter in place of R2's
   // diagonal blocks, which nothing reads any more)
@@ -748,7 +752,7 @@ __device__ __noinline__ int cqr_panel(const CqrArgs a) {
       }
     }
   }
-  return 1;
+  return 4 << 1 | 1;
 }
 
 }  // namespace rrf
