@@ -411,23 +411,30 @@ struct PassModel {
   int b;
   bool f64;
   bool tc;      // single precision on tcgen05
-  bool cl;      // the confined panel runs as one thread-block cluster with its slab in registers
-  // flop per microsecond the two GEMM kernels sustain on the whole device
-  double vtw() const { return 2.0 * rows * n * b / (f64 ? 33e6 : (tc ? 75e6 : 45e6)) + 10.0; }
-  double upd() const { return 4.0 * rows * n * b / (f64 ? 27e6 : (tc ? 100e6 : 32e6)) + 15.0; }
-  // fix-up + panel + T factor on `ctas` SMs, with the launch and event hand-overs of the side stream
+  // flop per microsecond the two GEMM kernels sustain on the whole device; narrow blocks read and write W for less
+  double rate(double wide) const { return b >= 64 ? wide : (f64 ? wide * (b == 32 ? 0.75 : 0.5) : wide * 0.5); }
+  double vtw() const { return 2.0 * rows * n * b / rate(f64 ? 34e6 : (tc ? 86e6 : 45e6)) + 10.0; }
+  double upd() const { return 4.0 * rows * n * b / rate(f64 ? 33e6 : (tc && b <= 64 ? 117e6 : 32e6)) + 15.0; }
+  // T Z, the stop rule, the split planes and the hand-overs between them
+  double rest() const { return f64 ? 20.0 : 35.0; }
+  // load + fix-up + panel on `ctas` SMs, with the launch and event hand-overs of the side stream: the b x b
+  // factorisations, the products over a slab, the partial results read beside the GEMM kernels (measured inside runs:
+  // 31 us for 1024 x 16 on 16 SMs, 92 for 4096 x 32 and 158 for 4096 x 64 on 16, 116 for 5003 x 64 on 45, 225 for
+  // 8192 x 64 on 26)
   double panel_chain(int ctas) const {
     const double R = std::max(64.0, (rows + b) / ctas);
-    if (cl)     // one cluster, slab in registers: 4096 x 64 takes 232 us, 4096 x 32 107 us, 1024 x 16 55 us on their own
-      return (b * (3700.0 + 42.0 * b) + 40000.0 + 0.07 * R * b * b) / 1965.0 + 20.0;
-    const double cycles = b * (7000.0 + 0.14 * R * b) + 20000.0 + 0.07 * R * b * b;
-    return cycles / 1965.0 + 0.3 * b + (f64 ? 45.0 : 85.0);
+    return 12.0 + 0.8 * b + 7.6e-5 * R * b * b + 2e-3 * R * b;
+  }
+  // the same on every SM, nothing to fix up (72 us for 8192 x 64, 50 for 20000 x 32); the column loop beyond b = 64
+  double panel_alone() const {
+    const double R = std::max(64.0, rows / sms);
+    return b > 64 ? b * 4.2 + 25.0 : 10.0 + 0.9 * b + 4e-5 * R * b * b + 1e-3 * R * b;
   }
   // the stream-K GEMMs lose a little more than the SMs they give up (tile quantisation)
-  double scale(int ctas) const { return std::pow((double)sms / (sms - ctas), 1.15); }
-  double step_ungated(int ctas) const { return std::max(panel_chain(ctas), (vtw() + upd()) * scale(ctas)); }
-  double step_gated(int ctas) const { return vtw() + std::max(panel_chain(ctas), upd() * scale(ctas)); }
-  double step_serial() const { return vtw() + upd() + b * 4.2 + 25.0; }
+  double scale(int ctas) const { return std::pow((double)sms / (sms - ctas), 1.1); }
+  double step_ungated(int ctas) const { return std::max(panel_chain(ctas), (vtw() + upd()) * scale(ctas)) + rest(); }
+  double step_gated(int ctas) const { return vtw() + std::max(panel_chain(ctas), upd() * scale(ctas)) + rest(); }
+  double step_serial() const { return vtw() + upd() + panel_alone() + rest(); }
 };
 static size_t look_scratch_bytes(int b) {   // Gpart[kLookMaxCtas][b*b] + M[b*b]
   return align_up((size_t)(kLookMaxCtas + 1) * b * b * sizeof(double), 256);
@@ -1465,25 +1472,20 @@ rrf_status_t rrf_run(rrf_handle_t h, const rrf_params_t* p, void* dA, int64_t ld
              plan_panel_cl(h, m, b, &pcl_probe0, false)) {
     // every panel of the chain fits one thread-block cluster (the first as it is, the later ones with the b rows
     // of the fix-up): the chain takes only that many SMs
-    const PassModel pm{h->sms, (double)m, (double)n, b, p->dtype == RRF_F64, p->dtype == RRF_F32 && h->f32_engine == 1, true};
+    const PassModel pm{h->sms, (double)m, (double)n, b, p->dtype == RRF_F64, p->dtype == RRF_F32 && h->f32_engine == 1};
     const double t = std::min(pm.step_ungated(kClusterMax), pm.step_gated(kClusterMax));
     if ((p->flags & RRF_FLAG_TWO_QUEUES) || t < pm.step_serial()) {
-      // A cluster needs its SMs inside one GPC, and where the GEMM kernels' CTAs land cannot be chosen: with exactly
-      // the cluster's SMs kept free the panel often waits for a GEMM kernel to drain.  Where the panel chain is the
-      // critical path the GEMM kernels therefore leave 44 SMs free (measured on 4096 x 11008 fp32: 2.61 ms against
-      // 2.69 with 16, 2.67 with 20, 2.72 with 32); where the GEMMs are, they get every SM the cluster does not
-      // take (4096 x 4096 fp64, b = 32: 2.51 ms with 16 against 2.88 with 44).
+      // The GEMM kernels get every SM the cluster does not take (4096 x 11008 fp32: 2.00 ms with 16 SMs kept free, 2.08
+      // with 26, 2.33 with 44; 4096 x 4096 fp64, b = 32: 1.80 with 16, 2.05 with 44; 5003 x 3001 likewise on a grid)
       const int gcl = std::max(pcl_probe.G, pcl_probe0.G);
-      const bool chain_critical = pm.panel_chain(gcl) > (pm.vtw() + pm.upd()) * pm.scale(gcl);
-      const int keep = chain_critical ? std::max(gcl, std::min(44, h->sms / 3)) : gcl;
-      look_ctas = p->tune_panel_ctas > 0 ? std::max(gcl, std::min((int)p->tune_panel_ctas, h->sms / 3)) : keep;
+      look_ctas = p->tune_panel_ctas > 0 ? std::max(gcl, std::min((int)p->tune_panel_ctas, h->sms / 3)) : gcl;
       look_cl = true;
     }
   } else if (!(p->flags & RRF_FLAG_ONE_QUEUE) && !unchanged && steps_total >= 2) {
     const int fewest = panel_min_ctas(h, m, b);
     const int cap = std::min(kLookMaxCtas, h->sms / 3);
     if (fewest > 0 && fewest <= cap) {
-      const PassModel pm{h->sms, (double)m, (double)n, b, p->dtype == RRF_F64, p->dtype == RRF_F32 && h->f32_engine == 1, false};
+      const PassModel pm{h->sms, (double)m, (double)n, b, p->dtype == RRF_F64, p->dtype == RRF_F32 && h->f32_engine == 1};
       int best = fewest;
       double best_t = std::min(pm.step_ungated(fewest), pm.step_gated(fewest));
       for (int c = fewest + 1; c <= cap; ++c) {
@@ -1531,7 +1533,7 @@ rrf_status_t rrf_run(rrf_handle_t h, const rrf_params_t* p, void* dA, int64_t ld
   } else if (p->flags & RRF_FLAG_SAMPLE_NEVER) {
     predict = 2;
   } else if (!(p->flags & RRF_FLAG_SAMPLE_ALWAYS) && !(p->flags & RRF_FLAG_FIXED_RANK)) {
-    const PassModel pm{h->sms, (double)m, (double)n, b, p->dtype == RRF_F64, false, false};
+    const PassModel pm{h->sms, (double)m, (double)n, b, p->dtype == RRF_F64, false};
     if (pm.vtw() + pm.upd() > 600.0) predict = 0;
   }
   const bool predicting = predict != 1;
@@ -1786,7 +1788,7 @@ rrf_status_t rrf_run(rrf_handle_t h, const rrf_params_t* p, void* dA, int64_t ld
     auto gated = [&](int rows_i) {
       if (p->tune_gate != 0) return p->tune_gate == 2;
       if (look_cl) return false;       // a cluster takes so few SMs that holding it back never pays (measured)
-      const PassModel pm{h->sms, (double)rows_i, (double)n, b, p->dtype == RRF_F64, tc, look_cl};
+      const PassModel pm{h->sms, (double)rows_i, (double)n, b, p->dtype == RRF_F64, tc};
       return pm.step_gated(look_ctas) < pm.step_ungated(look_ctas);
     };
     PanelSource src1 = src;           // panel 1: sampled from A by the sample kernel
@@ -1895,13 +1897,13 @@ rrf_status_t rrf_run(rrf_handle_t h, const rrf_params_t* p, void* dA, int64_t ld
       // tiles as they can do in the time the first launch still needs (by the schedule model, with a wide margin).
       int t1 = 0, tpc2 = 0;
       if (gate && !look_cl && !utc_on && i + 1 < steps_run && !h->profiling) {
-        const PassModel pm{h->sms, (double)rows, (double)n, b, p->dtype == RRF_F64, tc, false};
+        const PassModel pm{h->sms, (double)rows, (double)n, b, p->dtype == RRF_F64, tc};
         const double t_upd = pm.upd() * pm.scale(look_ctas), t_pan = pm.panel_chain(look_ctas);
         if (t_pan < 0.9 * t_upd) {
           const double t_all = ((double)gsms * t_upd + (double)look_ctas * t_pan) / h->sms;   // both launches end together
-          // 0.35 of what the model allows: measured on 8192 x 8192, b = 64 (8.685 ms without the second launch):
-          // 8.654 / 8.607 / 8.653 / 8.94 / 9.28 ms with 0.2 / 0.4 / 0.6 / 0.8 / 1.0 of it
-          const double share = 0.35 * (double)look_ctas * (t_all - t_pan) / ((double)gsms * t_upd);
+          // 0.95 of what the model allows: measured on 8192 x 8192, b = 64, 26 SMs: 7.82 / 7.76 / 7.55 / 7.39 / 7.37 ms
+          // with 0.2 / 0.35 / 0.65 / 0.9 / 1.0 of it
+          const double share = 0.95 * (double)look_ctas * (t_all - t_pan) / ((double)gsms * t_upd);
           const int tiles_h = (int)(share * up.total);
           if (tiles_h >= 4 * look_ctas) {
             tpc2 = ceil_div(tiles_h, look_ctas);
