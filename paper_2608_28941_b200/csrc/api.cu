@@ -551,7 +551,9 @@ struct Ops {
       e = cudaFuncSetAttribute(upd_tc_kernel<B>, cudaFuncAttributeMaxDynamicSharedMemorySize, UtcCfg<B>::SMEM);
       if (e != cudaSuccess) return e;
     }
-    e = cudaFuncSetAttribute(tz_kernel<T, B>, cudaFuncAttributeMaxDynamicSharedMemorySize, Z_SMEM);
+    e = cudaFuncSetAttribute(tz_kernel<T, B, kTzCols>, cudaFuncAttributeMaxDynamicSharedMemorySize, Z_SMEM);
+    if (e != cudaSuccess) return e;
+    e = cudaFuncSetAttribute(tz_kernel<T, B, kTzCols / 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, Z_SMEM);
     return e;
   }
   static void sample(const CUtensorMap& tmW, const CUtensorMap& tmO, void* Ypart, int r0, int rows, int n, int j0,
@@ -572,11 +574,17 @@ struct Ops {
     vtw_sk_kernel<T, B, V_BN, kVtwBK, V_WM, V_WN, V_STAGES>
         <<<p.P, 9 * 32, V_SMEM, st>>>(tmV, tmC, (T*)Zpart, r0, cv0, p.KT, p.total, p.tpc, ctrl);
   }
-  static constexpr int Z_SMEM = (B * (B + 4) + B * (kTzCols + 4)) * (int)sizeof(T);
+  static constexpr int Z_SMEM = (B * (B + 4) + B * (kTzCols + 4)) * (int)sizeof(T);   // enough for the narrow form too
   static void tz(const void* Zpart, const VtwPlan& vp, const void* Tm, long long ldt, int transpose_t, void* Zt,
                  const int* done_flag, cudaStream_t st) {
-    tz_kernel<T, B><<<vp.npad / kTzCols, kTzThreads, Z_SMEM, st>>>((const T*)Zpart, vp.bn, vp.nct, vp.KT, vp.tpc, (const T*)Tm,
-                                                            ldt, transpose_t, (T*)Zt, done_flag);
+    // half as many columns a CTA where that still is at most one CTA per SM: a column tile then has few CTAs and many
+    // partial slots, and each thread has twice as many of them in flight (512 columns, 33 slots: TZ_OLD -> TZ_NEW us)
+    if (vp.npad / (kTzCols / 2) <= 148)
+      tz_kernel<T, B, kTzCols / 2><<<vp.npad / (kTzCols / 2), kTzThreads, Z_SMEM, st>>>(
+          (const T*)Zpart, vp.bn, vp.nct, vp.KT, vp.tpc, (const T*)Tm, ldt, transpose_t, (T*)Zt, done_flag);
+    else
+      tz_kernel<T, B, kTzCols><<<vp.npad / kTzCols, kTzThreads, Z_SMEM, st>>>(
+          (const T*)Zpart, vp.bn, vp.nct, vp.KT, vp.tpc, (const T*)Tm, ldt, transpose_t, (T*)Zt, done_flag);
   }
   static void update(const CUtensorMap& tmV, const CUtensorMap& tmZ, const CUtensorMap& tmC, const CUtensorMap& tmO,
                      void* C, long long ldc, void* top, long long ldtop, int r0, int rows, int ncols, int cv0,
@@ -1277,10 +1285,13 @@ rrf_status_t rrf_apply_workspace_bytes(int32_t dtype, int64_t m, int64_t ncols, 
 
 namespace rrf {
 
-// C <- Q^T C (forward over the blocks, T^T) or C <- Q C (backward, T).
+// C <- Q^T C (forward over the blocks, T^T) or C <- Q C (backward, T).  `identity`: C is the first ncols = k columns of the
+// identity and Q is applied; column c is then zero from row c + 1 on until its own block has been applied, so block l
+// only touches columns l b and later, half of the work.
 static rrf_status_t apply_blocks(rrf_handle_t h, int dtype, long long m, int b, int k, const void* dV, long long ldv,
                                  const void* dT, long long ldt, void* dC, long long ldc, long long ncols,
-                                 void* d_workspace, size_t workspace_bytes, cudaStream_t st, bool transpose) {
+                                 void* d_workspace, size_t workspace_bytes, cudaStream_t st, bool transpose,
+                                 bool identity = false) {
   if (h == nullptr || dV == nullptr || dT == nullptr || dC == nullptr || d_workspace == nullptr)
     return RRF_ERR_INVALID_ARG;
   const int esize = dtype == RRF_F64 ? 8 : 4;
@@ -1321,14 +1332,22 @@ static rrf_status_t apply_blocks(rrf_handle_t h, int dtype, long long m, int b, 
   for (int q = 0; q < nblk; ++q) {
     const int l = transpose ? q : nblk - 1 - q;
     const int r0 = l * b, rows = (int)(m - r0);
-    VtwPlan vp = plan_vtw(h->sms, rows, ncols, ops->v_bn);
+    const int c0 = identity ? r0 : 0, nc = (int)ncols - c0;       // columns this block touches
+    void* C = (char*)dC + (size_t)c0 * esize;
+    if (identity && (!make_map(h, &tmC_k, dtype, C, m, nc, ldc, kbox, tc) || !make_map(h, &tmC_u, dtype, C, m, nc, ldc, ops->u_bm)))
+      return RRF_ERR_INVALID_ARG;
+    VtwPlan vp = plan_vtw(h->sms, rows, nc, ops->v_bn);
     vp.tc = tc;
     vp.chunk = h->tc_chunk;
     ops->vtw(tmV_k, tmC_k, Zpart, r0, r0, vp, h->d_ctrl, st);
     ops->tz(Zpart, vp, (const char*)dT + (size_t)r0 * esize, ldt, transpose ? 1 : 0, Zt, &h->d_ctrl->done, st);
-    UpdPlan up = plan_upd(h->sms, rows, ncols, ops->u_bm, ops->u_bn, ops->u_wn);
-    if (utc_on) up.tc = &utc;
-    ops->update(tmV_u, tmZ, tmC_u, tmC_u, dC, ldc, dC, ldc, r0, rows, (int)ncols, r0, 0, -1, nullptr, nullptr, up,
+    UpdPlan up = plan_upd(h->sms, rows, nc, ops->u_bm, ops->u_bn, ops->u_wn);
+    if (utc_on) {
+      utc.npad = vp.npad;
+      if (!make_map(h, &utc.tmZs, dtype, utc.zsplit, 2ull * vp.npad, b, b, kUtcBN)) return RRF_ERR_INVALID_ARG;
+      up.tc = &utc;
+    }
+    ops->update(tmV_u, tmZ, tmC_u, tmC_u, C, ldc, C, ldc, r0, rows, nc, r0, 0, -1, nullptr, nullptr, up,
                 h->d_ctrl, nullptr, st);
   }
   const cudaError_t e = cudaGetLastError();
@@ -1368,7 +1387,7 @@ rrf_status_t rrf_form_q(rrf_handle_t h, int32_t dtype, int64_t m, int32_t b, int
     eye_kernel<double><<<grid, 256, 0, st>>>((double*)dQ, ldq, m, k);
   else
     eye_kernel<float><<<grid, 256, 0, st>>>((float*)dQ, ldq, m, k);
-  return apply_blocks(h, dtype, m, b, k, dV, ldv, dT, ldt, dQ, ldq, k, d_workspace, workspace_bytes, st, false);
+  return apply_blocks(h, dtype, m, b, k, dV, ldv, dT, ldt, dQ, ldq, k, d_workspace, workspace_bytes, st, false, true);
 }
 
 rrf_status_t rrf_transfer_workspace_bytes(int32_t dtype, int64_t m, int64_t ncols, int32_t b, size_t* bytes) {
@@ -1397,6 +1416,47 @@ rrf_status_t rrf_subspace_transfer(rrf_handle_t h, int32_t dtype, int64_t m, int
   unsigned char* ws = (unsigned char*)d_workspace;
   void* Cm = ws;
   cudaStream_t st = (cudaStream_t)cuda_stream;
+  // Q_new^T (Q_old M) by way of the small k_old x k_new matrix S^T = Q_old^T Q_new: the reflectors then pass over m x k_new
+  // numbers instead of m x ncols, and M is read once per block of S (4096 x 11008, k 256 -> 128: 1114 -> TRANSFER_US us;
+  // at ncols = 2 k_new the two take the same time).  M has to be readable by TMA, and the result must not overwrite it.
+  const char *mi = (const char*)dM, *mo = (const char*)dMout;
+  const bool apart = mo + ((size_t)(k_new - 1) * ldmo + ncols) * esize <= mi || mi + ((size_t)(k_old - 1) * ldm + ncols) * esize <= mo;
+  if (apart && k_new % b == 0 && k_old % b == 0 && ncols > 2LL * k_new && ld_ok(ldm, ncols, esize) && aligned16(dM) &&
+      m <= 0x7fffffffLL && ncols <= 0x7fffffffLL) {
+    const long long lds = (long long)align_up((size_t)k_new, 16);
+    rrf_status_t s = rrf_form_q(h, dtype, m, b, k_new, dV_new, ldv_new, dT_new, ldt_new, Cm, lds, ws + cbytes,
+                                workspace_bytes - cbytes, cuda_stream);
+    if (s != RRF_OK) return s;
+    s = apply_blocks(h, dtype, m, b, k_old, dV_old, ldv_old, dT_old, ldt_old, Cm, lds, k_new, ws + cbytes,
+                     workspace_bytes - cbytes, st, true);
+    if (s != RRF_OK) return s;
+    const OpTable* ops = get_ops(dtype, b);
+    const bool tc = dtype == RRF_F32 && h->f32_engine == 1;
+    const unsigned kbox = tc ? kTcSub : kVtwBK;
+    CUtensorMap tmS, tmM;
+    if (!make_map(h, &tmS, dtype, Cm, k_old, k_new, lds, kbox, tc) || !make_map(h, &tmM, dtype, dM, k_old, ncols, ldm, kbox, tc))
+      return RRF_ERR_INVALID_ARG;
+    void* Zpart = ws + cbytes;
+    VtwPlan vp = plan_vtw(h->sms, k_old, ncols, ops->v_bn);
+    vp.tc = tc;
+    vp.chunk = h->tc_chunk;
+    const int zgrid = (int)std::min<long long>((b * ncols + 255) / 256, (long long)h->sms * 16);
+    for (int j0 = 0; j0 < k_new; j0 += b) {
+      ops->vtw(tmS, tmM, Zpart, 0, j0, vp, h->d_ctrl, st);
+      if (dtype == RRF_F64)
+        zrows_kernel<double><<<zgrid, 256, 0, st>>>((const double*)Zpart, b, vp.bn, vp.KT, vp.tpc, ncols,
+                                                    (double*)dMout + (size_t)j0 * ldmo, ldmo);
+      else
+        zrows_kernel<float><<<zgrid, 256, 0, st>>>((const float*)Zpart, b, vp.bn, vp.KT, vp.tpc, ncols,
+                                                   (float*)dMout + (size_t)j0 * ldmo, ldmo);
+    }
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) {
+      h->last_cuda = (int)e;
+      return RRF_ERR_CUDA;
+    }
+    return RRF_OK;
+  }
   const int grid = (int)std::min<long long>(((long long)m * ncols + 255) / 256, (long long)h->sms * 16);
   if (dtype == RRF_F64)
     copy_rows_kernel<double><<<grid, 256, 0, st>>>((double*)Cm, ldc, (const double*)dM, ldm, k_old, m, ncols);

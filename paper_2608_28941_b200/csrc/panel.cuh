@@ -904,51 +904,52 @@ __global__ void __launch_bounds__(256)
 // Zt[col][0:B] = (op(T) * sum of the partial slots of Z[:, col])   with op(T) = T^T (apply Q^T) or
 // T (apply Q).  Zpart is in the slot layout of vtw_sk_kernel: column tile ct (bn columns) is the sum
 // of slots p + ct for the CTAs p whose tile range [p*tpc, (p+1)*tpc) meets [ct*kt, (ct+1)*kt),
-// summed in CTA order.  Each CTA owns kTzCols columns: it stages op(T) (as the A operand, K = row)
+// summed in CTA order.  Each CTA owns COLS columns: it stages op(T) (as the A operand, K = row)
 // and the summed columns in shared memory with a pitch of 4 mod 16 elements, which makes the scalar
 // fragment loads conflict free, and multiplies on the tensor cores.  The output is the transposed
 // (K-contiguous) operand of upd_sk_kernel.
 // ------------------------------------------------------------------------------------------
 constexpr int kTzCols = 32;
 constexpr int kTzThreads = 512;
-template <typename T, int B>
+template <typename T, int B, int COLS>
 __global__ void __launch_bounds__(kTzThreads)
     tz_kernel(const T* __restrict__ Zpart, int bn, int nct, int kt, int tpc, const T* __restrict__ Tm, long long ldt,
               int transpose_t, T* __restrict__ Zt, const int* done_flag) {
   if (*reinterpret_cast<const volatile int*>(done_flag)) return;
-  constexpr int PA = B + 4, PB = kTzCols + 4;
+  constexpr int PA = B + 4, PB = COLS + 4;
   constexpr int NWARP = kTzThreads / 32;
-  constexpr int MTILES = B / 16, NTILES = kTzCols / 8;
+  constexpr int MTILES = B / 16, NTILES = COLS / 8;
   extern __shared__ unsigned char zsm_raw[];
   T* As = reinterpret_cast<T*>(zsm_raw);          // [B][PA]: As[l][j] = op(T)[j][l]
   T* Bs = As + (size_t)B * PA;                    // [B][PB]: summed Z[l][col]
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
-  const int col0 = blockIdx.x * kTzCols;
-  {
-    constexpr int EA = (B * B + kTzThreads - 1) / kTzThreads;
-    T v[EA];
+  const int col0 = blockIdx.x * COLS;
+  constexpr int EA = (B * B + kTzThreads - 1) / kTzThreads;
+  T tv[EA];                                       // op(T), on its way while the slots are summed
 #pragma unroll
-    for (int e = 0; e < EA; ++e) {
-      const int idx = tid + e * kTzThreads, l = idx / B, j = idx - l * B;
-      v[e] = T(0);
-      if (idx < B * B) {
-        if (transpose_t) { if (l <= j) v[e] = Tm[(size_t)l * ldt + j]; }     // (T^T)[j][l] = T[l][j], upper triangular
-        else             { if (j <= l) v[e] = Tm[(size_t)j * ldt + l]; }     // T[j][l]
-      }
-    }
-#pragma unroll
-    for (int e = 0; e < EA; ++e) {
-      const int idx = tid + e * kTzThreads, l = idx / B, j = idx - l * B;
-      if (idx < B * B) As[l * PA + j] = v[e];
+  for (int e = 0; e < EA; ++e) {
+    const int idx = tid + e * kTzThreads, l = idx / B, j = idx - l * B;
+    tv[e] = T(0);
+    if (idx < B * B) {
+      if (transpose_t) { if (l <= j) tv[e] = Tm[(size_t)l * ldt + j]; }     // (T^T)[j][l] = T[l][j], upper triangular
+      else             { if (j <= l) tv[e] = Tm[(size_t)j * ldt + l]; }     // T[j][l]
     }
   }
-  const int ct = col0 / bn, cin = col0 - ct * bn;   // kTzCols divides bn; tiles past the last hold no data
+  auto stage_t = [&]() {
+#pragma unroll
+    for (int e = 0; e < EA; ++e) {
+      const int idx = tid + e * kTzThreads, l = idx / B, j = idx - l * B;
+      if (idx < B * B) As[l * PA + j] = tv[e];
+    }
+  };
+  if (B > 64) stage_t();                          // the widest block has no registers to keep it
+  const int ct = col0 / bn, cin = col0 - ct * bn;   // COLS divides bn; tiles past the last hold no data
   const int p_lo = (ct * kt) / tpc, p_hi = ((ct + 1) * kt - 1) / tpc;
   {
-    // every thread owns EPT entries; the loads of up to eight slots are in flight together and are
+    // every thread owns EPT entries; the loads of a batch of slots are in flight together and are
     // then added in slot (= CTA) order
-    constexpr int EPT = (B * kTzCols + kTzThreads - 1) / kTzThreads;
-    constexpr int SB = EPT >= 8 ? 4 : 8;            // slots per batch, bounded by registers
+    constexpr int EPT = (B * COLS + kTzThreads - 1) / kTzThreads;
+    constexpr int SB = EPT >= 8 ? 4 : (EPT >= 4 ? 8 : 16);     // slots per batch, bounded by registers
     double sum[EPT];
 #pragma unroll
     for (int e = 0; e < EPT; ++e) sum[e] = 0.0;
@@ -960,8 +961,8 @@ __global__ void __launch_bounds__(kTzThreads)
           const T* slot = Zpart + (size_t)(p0 + u + ct) * (size_t)(B * bn) + cin;
 #pragma unroll
           for (int e = 0; e < EPT; ++e) {
-            const int idx = tid + e * kTzThreads, l = idx / kTzCols, cl = idx - l * kTzCols;
-            v[u][e] = (p0 + u <= p_hi && idx < B * kTzCols) ? __ldcg(slot + (size_t)l * bn + cl) : T(0);
+            const int idx = tid + e * kTzThreads, l = idx / COLS, cl = idx - l * COLS;
+            v[u][e] = (p0 + u <= p_hi && idx < B * COLS) ? __ldcg(slot + (size_t)l * bn + cl) : T(0);
           }
         }
 #pragma unroll
@@ -972,10 +973,11 @@ __global__ void __launch_bounds__(kTzThreads)
     }
 #pragma unroll
     for (int e = 0; e < EPT; ++e) {
-      const int idx = tid + e * kTzThreads, l = idx / kTzCols, cl = idx - l * kTzCols;
-      if (idx < B * kTzCols) Bs[l * PB + cl] = (T)sum[e];
+      const int idx = tid + e * kTzThreads, l = idx / COLS, cl = idx - l * COLS;
+      if (idx < B * COLS) Bs[l * PB + cl] = (T)sum[e];
     }
   }
+  if (B <= 64) stage_t();
   __syncthreads();
   for (int tile = warp; tile < MTILES * NTILES; tile += NWARP) {
     const int j0 = (tile / NTILES) * 16, n0 = (tile % NTILES) * 8;
@@ -993,6 +995,22 @@ __global__ void __launch_bounds__(kTzThreads)
     Zt[(size_t)(col + 1) * B + j] = acc[1];
     Zt[(size_t)col * B + j + 8] = acc[2];
     Zt[(size_t)(col + 1) * B + j + 8] = acc[3];
+  }
+}
+
+// Z itself, row by row: out (b x ncols, leading dimension ldo) = the partial slots of vtw_sk_kernel summed in CTA order
+template <typename T>
+__global__ void __launch_bounds__(256)
+    zrows_kernel(const T* __restrict__ Zpart, int b, int bn, int kt, int tpc, long long ncols, T* __restrict__ out, long long ldo) {
+  const long long total = (long long)b * ncols;
+  for (long long idx = (long long)blockIdx.x * 256 + threadIdx.x; idx < total; idx += (long long)gridDim.x * 256) {
+    const long long l = idx / ncols, col = idx - l * ncols;
+    const int ct = (int)(col / bn), cin = (int)(col - (long long)ct * bn);
+    const int p_lo = (ct * kt) / tpc, p_hi = ((ct + 1) * kt - 1) / tpc;
+    const T* slot = Zpart + (size_t)(p_lo + ct) * (size_t)(b * bn) + (size_t)l * bn + cin;
+    double s = 0.0;
+    for (int p = p_lo; p <= p_hi; ++p, slot += (size_t)b * bn) s += (double)__ldcg(slot);
+    out[l * ldo + col] = (T)s;
   }
 }
 
@@ -1050,20 +1068,22 @@ __global__ void __launch_bounds__(256)
     stop_kernel(const double* __restrict__ norm_part, int npart, int b, int max_rank, int estimator,
                 int fixed_rank, double* __restrict__ tr_sub, double* __restrict__ tr_dir, Ctrl* ctrl,
                 int* __restrict__ done_after, int reset_bar, int* __restrict__ samp, int predict) {
-  if (*reinterpret_cast<volatile int*>(&ctrl->done)) return;
+  // the loop state is read at once, ahead of the sums, and not field by field behind them
+  const int done0 = *reinterpret_cast<volatile int*>(&ctrl->done), status0 = ctrl->status, i = ctrl->steps;
+  const double esub0 = ctrl->E_sub, sigma2 = ctrl->sigma2, eprev0 = ctrl->E_prev, rprev0 = ctrl->r_prev;
+  if (done0) return;
   __shared__ double red[64];
   double st = 0.0, sr = 0.0;
-  for (int i = threadIdx.x; i < npart; i += 256) {
-    st += norm_part[2 * i];
-    sr += norm_part[2 * i + 1];
+  for (int q = threadIdx.x; q < npart; q += 256) {
+    st += norm_part[2 * q];
+    sr += norm_part[2 * q + 1];
   }
   const double top = block_sum(st, red);
   const double trail = block_sum(sr, red + 32);
   if (threadIdx.x == 0) {
-    const double e_sub = ctrl->E_sub - top;
+    const double e_sub = esub0 - top;
     ctrl->E_sub = e_sub;
     ctrl->E_dir = trail;
-    const int i = ctrl->steps;
     tr_sub[i] = e_sub;
     tr_dir[i] = trail;
     ctrl->steps = i + 1;
@@ -1071,10 +1091,10 @@ __global__ void __launch_bounds__(256)
     if (reset_bar) ctrl->bar = 0;
     const double E = estimator == 0 ? trail : e_sub;
     // the sampled rules (estimator >= 2) decide in est_kernel; here only the rank cap ends the loop
-    const bool below = estimator < 2 && !(E > ctrl->sigma2);
+    const bool below = estimator < 2 && !(E > sigma2);
     const bool met = !fixed_rank && below;
     const bool cap = (i + 2) * b > max_rank;
-    if (ctrl->status == RRF_OK && !below && cap) ctrl->status = RRF_MAX_RANK_REACHED;
+    if (status0 == RRF_OK && !below && cap) ctrl->status = RRF_MAX_RANK_REACHED;
     if (met || cap) ctrl->done = 1;
     if (done_after != nullptr) done_after[i + 1] = (met || cap) ? 1 : 0;
     // Sampling predictor.  The update of pass i+1 also samples a later panel, which is wasted work if
@@ -1084,15 +1104,15 @@ __global__ void __launch_bounds__(256)
     // skipped panel is sampled by a kernel of its own.  predict: 0 = by this rule, 1 = always sample,
     // 2 = never sample.
     if (samp != nullptr) {
-      const double Ep = ctrl->E_prev;
+      const double Ep = eprev0;
       double r = (Ep > 0.0) ? E / Ep : 1.0;
       r = r < 0.0 ? 0.0 : (r > 1.0 ? 1.0 : r);
-      const double rp = ctrl->r_prev;
+      const double rp = rprev0;
       const double dr = (rp >= 0.0 && r > rp) ? r - rp : 0.0;
       const double rr = r + dr > 1.0 ? 1.0 : r + dr;
       const double e = E * rr;
       const bool steady = rp >= 0.0 && fabs(r - rp) <= 0.3 * fmax(r, rp);
-      int want = fixed_rank || !steady || e > 0.9 * ctrl->sigma2;
+      int want = fixed_rank || !steady || e > 0.9 * sigma2;
       if (predict == 1) want = 1;
       if (predict == 2) want = 0;
       samp[i + 1] = want;
