@@ -135,7 +135,6 @@ struct UpdTc {
   const rrf_ctx* h;       // for the tensor maps built per launch
   const void* V;          // reflectors (read directly, not through a tensor map)
   long long ldv;
-  const void* Zt;         // [npad][b], written by the T Z kernel
   int npad;
   const void* Om;         // OmegaT as the run sees it
   long long ldom;
@@ -145,6 +144,21 @@ struct UpdTc {
   int chunk;
   CUtensorMap tmZs, tmOs;
 };
+// what the T Z kernel writes for it: the planes of its result and, with j0 >= 0, of the rows of OmegaT sampled with
+static TzSplit tz_split(const UpdTc* x, int j0, long long ncols) {
+  TzSplit sp{};
+  if (x == nullptr) return sp;
+  sp.z = (float*)x->zsplit;
+  sp.npad = x->npad;
+  if (j0 >= 0) {
+    sp.om = (const float*)x->Om + (size_t)j0 * x->ldom;
+    sp.ldom = x->ldom;
+    sp.ncols = (int)ncols;
+    sp.o = (float*)x->osplit;
+    sp.ldo = x->ldo2;
+  }
+  return sp;
+}
 // p0, Lb: this launch's CTAs are numbers p0 ... of the pass and start at tile Lb (a pass split over two launches)
 struct UpdPlan { int NS, NC, total, tpc, P, slots; const UpdTc* tc; int p0, Lb; };
 static UpdPlan plan_upd(int sms, long long rows, long long ncols, int bm, int bn, int wn) {
@@ -499,6 +513,21 @@ static bool b_ok(int dtype, int b) {
 }
 
 // ------------------------------------------------------------------ typed launchers
+// Launch as a programmatic dependent of the kernel before it on `st` (pdl_wait in common.cuh), or the ordinary way.
+template <typename... P, typename... A>
+static void launch_after(bool dependent, void (*kernel)(P...), int grid, int block, size_t smem, cudaStream_t st, A... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(block);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = dependent ? 1 : 0;
+  cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
 template <typename T, int B>
 struct Ops {
   static constexpr int KE = 128 / (int)sizeof(T);
@@ -563,41 +592,39 @@ struct Ops {
                                                                                   p.nseg, p.kt_per_seg, ctrl, only_if_zero, sq_part);
   }
   static void vtw(const CUtensorMap& tmV, const CUtensorMap& tmC, void* Zpart, int r0, int cv0, const VtwPlan& p,
-                  Ctrl* ctrl, cudaStream_t st) {
+                  Ctrl* ctrl, bool dep, cudaStream_t st) {
     if constexpr (std::is_same<T, float>::value) {
       if (p.tc) {     // the maps then have 32-row boxes
-        vtw_tc_kernel<B, TC_RS, TC_OS><<<p.P, kTcThreads, TcCfg<B, TC_RS, TC_OS>::SMEM, st>>>(
-            tmV, tmC, (float*)Zpart, r0, cv0, p.KT, p.total, p.tpc, p.chunk, ctrl);
+        launch_after(dep, vtw_tc_kernel<B, TC_RS, TC_OS>, p.P, kTcThreads, TcCfg<B, TC_RS, TC_OS>::SMEM, st, tmV, tmC,
+                     (float*)Zpart, r0, cv0, p.KT, p.total, p.tpc, p.chunk, ctrl);
         return;
       }
     }
-    vtw_sk_kernel<T, B, V_BN, kVtwBK, V_WM, V_WN, V_STAGES>
-        <<<p.P, 9 * 32, V_SMEM, st>>>(tmV, tmC, (T*)Zpart, r0, cv0, p.KT, p.total, p.tpc, ctrl);
+    launch_after(dep, vtw_sk_kernel<T, B, V_BN, kVtwBK, V_WM, V_WN, V_STAGES>, p.P, 9 * 32, V_SMEM, st, tmV, tmC, (T*)Zpart,
+                 r0, cv0, p.KT, p.total, p.tpc, ctrl);
   }
   static constexpr int Z_SMEM = (B * (B + 4) + B * (kTzCols + 4)) * (int)sizeof(T);   // enough for the narrow form too
   static void tz(const void* Zpart, const VtwPlan& vp, const void* Tm, long long ldt, int transpose_t, void* Zt,
-                 const int* done_flag, cudaStream_t st) {
+                 const int* done_flag, TzSplit sp, bool dep, cudaStream_t st) {
     // half as many columns a CTA where that still is at most one CTA per SM: a column tile then has few CTAs and many
-    // partial slots, and each thread has twice as many of them in flight (512 columns, 33 slots: TZ_OLD -> TZ_NEW us)
-    if (vp.npad / (kTzCols / 2) <= 148)
-      tz_kernel<T, B, kTzCols / 2><<<vp.npad / (kTzCols / 2), kTzThreads, Z_SMEM, st>>>(
-          (const T*)Zpart, vp.bn, vp.nct, vp.KT, vp.tpc, (const T*)Tm, ldt, transpose_t, (T*)Zt, done_flag);
+    // partial slots, and each thread has twice as many of them in flight
+    const bool narrow = vp.npad / (kTzCols / 2) <= 148;
+    sp.ntz = vp.npad / (narrow ? kTzCols / 2 : kTzCols);
+    const int grid = sp.ntz + (sp.o != nullptr ? B : 0);      // one CTA per row of OmegaT
+    if (narrow)
+      launch_after(dep, tz_kernel<T, B, kTzCols / 2>, grid, kTzThreads, Z_SMEM, st, (const T*)Zpart, vp.bn, vp.nct, vp.KT, vp.tpc,
+                   (const T*)Tm, ldt, transpose_t, (T*)Zt, done_flag, sp);
     else
-      tz_kernel<T, B, kTzCols><<<vp.npad / kTzCols, kTzThreads, Z_SMEM, st>>>(
-          (const T*)Zpart, vp.bn, vp.nct, vp.KT, vp.tpc, (const T*)Tm, ldt, transpose_t, (T*)Zt, done_flag);
+      launch_after(dep, tz_kernel<T, B, kTzCols>, grid, kTzThreads, Z_SMEM, st, (const T*)Zpart, vp.bn, vp.nct, vp.KT, vp.tpc,
+                   (const T*)Tm, ldt, transpose_t, (T*)Zt, done_flag, sp);
   }
   static void update(const CUtensorMap& tmV, const CUtensorMap& tmZ, const CUtensorMap& tmC, const CUtensorMap& tmO,
                      void* C, long long ldc, void* top, long long ldtop, int r0, int rows, int ncols, int cv0,
                      int top_rows, int j0, void* Ypart, double* norm_part, const UpdPlan& p, Ctrl* ctrl,
-                     const int* samp_flag, cudaStream_t st) {
+                     const int* samp_flag, bool dep, cudaStream_t st) {
     if constexpr (kHasUpdTc) {
       if (p.tc != nullptr) {
         const UpdTc& x = *p.tc;
-        split_planes_kernel<<<std::min(1024, ceil_div((long long)x.npad * B, 256)), 256, 0, st>>>(
-            (const float*)x.Zt, B, x.npad, B, (float*)x.zsplit, B, &ctrl->done);
-        if (j0 >= 0)
-          split_planes_kernel<<<std::min(1024, ceil_div((long long)ncols * B, 256)), 256, 0, st>>>(
-              (const float*)x.Om + (size_t)j0 * x.ldom, x.ldom, B, ncols, (float*)x.osplit, x.ldo2, &ctrl->done);
         // where the updated tiles go: the working matrix, and the rows of B that this pass completes
         CUtensorMap tmCs, tmTs;
         bool maps_ok = make_map(x.h, &tmCs, RRF_F32, C, (unsigned long long)r0 + rows, ncols, ldc, 32);
@@ -610,14 +637,14 @@ struct Ops {
           cudaMemcpyAsync(ctrl, kErr, sizeof(kErr), cudaMemcpyHostToDevice, st);
           return;
         }
-        upd_tc_kernel<B><<<p.P, kUtcThreads, UtcCfg<B>::SMEM, st>>>(
-            tmC, x.tmZs, x.tmOs, tmCs, tmTs, (const float*)x.V, x.ldv, r0, rows, ncols, cv0, top_rows, j0 >= 0 ? 1 : 0,
+        launch_after(
+            dep, upd_tc_kernel<B>, p.P, kUtcThreads, UtcCfg<B>::SMEM, st, tmC, x.tmZs, x.tmOs, tmCs, tmTs, (const float*)x.V, x.ldv, r0, rows, ncols, cv0, top_rows, j0 >= 0 ? 1 : 0,
             x.npad, (float*)Ypart, norm_part, p.NC, p.total, p.tpc, x.chunk * kUtcYChunkFactor, ctrl);
         return;
       }
     }
-    upd_sk_kernel<T, B, U_BM, U_BNB, U_WM, U_WN, U_STAGES, U_PW><<<p.P, (U_PW ? 9 : 8) * 32, U_SMEM, st>>>(
-        tmV, tmZ, tmC, tmO, (T*)C, ldc, (T*)top, ldtop, r0, rows, ncols, cv0, top_rows, j0, (T*)Ypart, norm_part, p.NC,
+    launch_after(
+        dep, upd_sk_kernel<T, B, U_BM, U_BNB, U_WM, U_WN, U_STAGES, U_PW>, p.P, (U_PW ? 9 : 8) * 32, U_SMEM, st, tmV, tmZ, tmC, tmO, (T*)C, ldc, (T*)top, ldtop, r0, rows, ncols, cv0, top_rows, j0, (T*)Ypart, norm_part, p.NC,
         p.total, p.tpc, ctrl, samp_flag, p.p0, p.Lb);
   }
 };
@@ -627,11 +654,11 @@ struct OpTable {
   cudaError_t (*setup)();
   void (*sample)(const CUtensorMap&, const CUtensorMap&, void*, int, int, int, int, const SamplePlan&, Ctrl*,
                  const int*, double*, cudaStream_t);
-  void (*vtw)(const CUtensorMap&, const CUtensorMap&, void*, int, int, const VtwPlan&, Ctrl*, cudaStream_t);
-  void (*tz)(const void*, const VtwPlan&, const void*, long long, int, void*, const int*, cudaStream_t);
+  void (*vtw)(const CUtensorMap&, const CUtensorMap&, void*, int, int, const VtwPlan&, Ctrl*, bool, cudaStream_t);
+  void (*tz)(const void*, const VtwPlan&, const void*, long long, int, void*, const int*, TzSplit, bool, cudaStream_t);
   void (*update)(const CUtensorMap&, const CUtensorMap&, const CUtensorMap&, const CUtensorMap&, void*, long long,
                  void*, long long, int, int, int, int, int, int, void*, double*, const UpdPlan&, Ctrl*, const int*,
-                 cudaStream_t);
+                 bool, cudaStream_t);
 };
 template <typename T, int B>
 static OpTable make_ops() {
@@ -681,6 +708,7 @@ struct PanelOpts {
   bool global_slab = false;        // blocked kernel: keep the slabs in global memory
   unsigned seq_base = 0;           // blocked kernel: first tag value of this launch (tags only grow within a run)
   double* csq = nullptr;           // [b][Gp]: the panel kernel leaves the column sums of squares of the panel here
+  bool* t_aside = nullptr;         // out: T is built on the side stream; ev_join has to be waited for
   int* g_out = nullptr;            // out: CTAs of the per-column panel kernel (Gp = g rounded up to 32)
 };
 template <typename Mark = NoMark>
@@ -712,7 +740,7 @@ static rrf_status_t launch_panel(rrf_ctx* h, int dtype, const void* Y, PanelSour
       h->last_cuda = (int)e;
       return RRF_ERR_CUDA;
     }
-    if (o.ev_join != nullptr) cudaEventRecord(o.ev_join, st);   // T is ready when the panel kernel is
+    if (o.t_aside != nullptr) *o.t_aside = false;
     return RRF_OK;
   }
   int rows_i = (int)rows;
@@ -783,7 +811,7 @@ static rrf_status_t launch_panel(rrf_ctx* h, int dtype, const void* Y, PanelSour
       e = cudaLaunchCooperativeKernel(fn, dim3(pp.G), dim3(kPanelThreads), args, pp.smem, st);
     }
   }
-  if (e == cudaSuccess && merge_t && o.ev_join != nullptr) cudaEventRecord(o.ev_join, st);   // T is ready when the panel kernel is
+  if (o.t_aside != nullptr) *o.t_aside = !merge_t;
   if (e == cudaSuccess && !merge_t) {
     cudaStream_t tt = st;
     if (o.ev_fork != nullptr) {          // fork: the T factor runs on the side stream after the panel
@@ -1321,7 +1349,6 @@ static rrf_status_t apply_blocks(rrf_handle_t h, int dtype, long long m, int b, 
     utc.h = h;
     utc.V = dV;
     utc.ldv = ldv;
-    utc.Zt = Zt;
     utc.npad = vp0.npad;
     utc.zsplit = (unsigned char*)Zpart + align_up((size_t)(kMaxSms + vp0.nct) * b * vp0.bn * esize, 256);
     utc.chunk = h->tc_chunk;
@@ -1339,16 +1366,17 @@ static rrf_status_t apply_blocks(rrf_handle_t h, int dtype, long long m, int b, 
     VtwPlan vp = plan_vtw(h->sms, rows, nc, ops->v_bn);
     vp.tc = tc;
     vp.chunk = h->tc_chunk;
-    ops->vtw(tmV_k, tmC_k, Zpart, r0, r0, vp, h->d_ctrl, st);
-    ops->tz(Zpart, vp, (const char*)dT + (size_t)r0 * esize, ldt, transpose ? 1 : 0, Zt, &h->d_ctrl->done, st);
     UpdPlan up = plan_upd(h->sms, rows, nc, ops->u_bm, ops->u_bn, ops->u_wn);
     if (utc_on) {
       utc.npad = vp.npad;
       if (!make_map(h, &utc.tmZs, dtype, utc.zsplit, 2ull * vp.npad, b, b, kUtcBN)) return RRF_ERR_INVALID_ARG;
       up.tc = &utc;
     }
+    ops->vtw(tmV_k, tmC_k, Zpart, r0, r0, vp, h->d_ctrl, q > 0, st);
+    ops->tz(Zpart, vp, (const char*)dT + (size_t)r0 * esize, ldt, transpose ? 1 : 0, Zt, &h->d_ctrl->done,
+            tz_split(up.tc, -1, nc), true, st);
     ops->update(tmV_u, tmZ, tmC_u, tmC_u, C, ldc, C, ldc, r0, rows, nc, r0, 0, -1, nullptr, nullptr, up,
-                h->d_ctrl, nullptr, st);
+                h->d_ctrl, nullptr, true, st);
   }
   const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) {
@@ -1417,7 +1445,7 @@ rrf_status_t rrf_subspace_transfer(rrf_handle_t h, int32_t dtype, int64_t m, int
   void* Cm = ws;
   cudaStream_t st = (cudaStream_t)cuda_stream;
   // Q_new^T (Q_old M) by way of the small k_old x k_new matrix S^T = Q_old^T Q_new: the reflectors then pass over m x k_new
-  // numbers instead of m x ncols, and M is read once per block of S (4096 x 11008, k 256 -> 128: 1114 -> TRANSFER_US us;
+  // numbers instead of m x ncols, and M is read once per block of S (4096 x 11008, k 256 -> 128: 1115 -> 303 us;
   // at ncols = 2 k_new the two take the same time).  M has to be readable by TMA, and the result must not overwrite it.
   const char *mi = (const char*)dM, *mo = (const char*)dMout;
   const bool apart = mo + ((size_t)(k_new - 1) * ldmo + ncols) * esize <= mi || mi + ((size_t)(k_old - 1) * ldm + ncols) * esize <= mo;
@@ -1442,7 +1470,7 @@ rrf_status_t rrf_subspace_transfer(rrf_handle_t h, int32_t dtype, int64_t m, int
     vp.chunk = h->tc_chunk;
     const int zgrid = (int)std::min<long long>((b * ncols + 255) / 256, (long long)h->sms * 16);
     for (int j0 = 0; j0 < k_new; j0 += b) {
-      ops->vtw(tmS, tmM, Zpart, 0, j0, vp, h->d_ctrl, st);
+      ops->vtw(tmS, tmM, Zpart, 0, j0, vp, h->d_ctrl, false, st);
       if (dtype == RRF_F64)
         zrows_kernel<double><<<zgrid, 256, 0, st>>>((const double*)Zpart, b, vp.bn, vp.KT, vp.tpc, ncols,
                                                     (double*)dMout + (size_t)j0 * ldmo, ldmo);
@@ -1648,7 +1676,6 @@ rrf_status_t rrf_run(rrf_handle_t h, const rrf_params_t* p, void* dA, int64_t ld
     utc.h = h;
     utc.V = dV;
     utc.ldv = ldv;
-    utc.Zt = Zt;
     utc.npad = npad;
     utc.Om = Om;
     utc.ldom = ldom;
@@ -1741,12 +1768,12 @@ rrf_status_t rrf_run(rrf_handle_t h, const rrf_params_t* p, void* dA, int64_t ld
         vp.tc = tc;
         vp.chunk = h->tc_chunk;
         mark(RRF_PHASE_VTW, i);
-        ops->vtw(tmV_k, tmP_k, Zpart, q0, q0, vp, ctrl, st);
+        ops->vtw(tmV_k, tmP_k, Zpart, q0, q0, vp, ctrl, true, st);
         mark(RRF_PHASE_TZ, i);
-        ops->tz(Zpart, vp, Tblk(q0), p->max_rank, 1, Zt, &ctrl->done, st);
+        ops->tz(Zpart, vp, Tblk(q0), p->max_rank, 1, Zt, &ctrl->done, TzSplit{}, true, st);
         const UpdPlan up = plan_upd(h->sms, rl, b, ops->u_bm, ops->u_bn, ops->u_wn);
         mark(RRF_PHASE_UPDATE, i);
-        ops->update(tmV_u, tmZp, tmP_u, tmP_u, Pbuf, b, Pbuf, b, q0, rl, b, q0, 0, -1, nullptr, nullptr, up, ctrl, nullptr, st);
+        ops->update(tmV_u, tmZp, tmP_u, tmP_u, Pbuf, b, Pbuf, b, q0, rl, b, q0, 0, -1, nullptr, nullptr, up, ctrl, nullptr, true, st);
       }
       PanelSource sd{};
       sd.nseg = 1;
@@ -1788,6 +1815,8 @@ rrf_status_t rrf_run(rrf_handle_t h, const rrf_params_t* p, void* dA, int64_t ld
       int pg = 0;
       if (sampled) po.csq = csq_buf(i);
       po.g_out = &pg;
+      bool t_aside = false;
+      po.t_aside = &t_aside;
       s = launch_panel(h, p->dtype, Ypart, src, rows, b, Vblk(r0), ldv, Tblk(r0), p->max_rank, ps, ctrl, &ctrl->done,
                        st, mark, i, po);
       if (s != RRF_OK) return panel_failed(s);
@@ -1798,19 +1827,19 @@ rrf_status_t rrf_run(rrf_handle_t h, const rrf_params_t* p, void* dA, int64_t ld
       vp.tc = tc;
       vp.chunk = h->tc_chunk;
       mark(RRF_PHASE_VTW, i);
-      ops->vtw(tmV_k, i == 0 ? tmA_k : tmW_k, Zpart, r0, r0, vp, ctrl, st);
+      ops->vtw(tmV_k, i == 0 ? tmA_k : tmW_k, Zpart, r0, r0, vp, ctrl, false, st);
       mark(RRF_PHASE_TZ, i);
-      cudaStreamWaitEvent(st, h->sync_events[2 * i + 1], 0);   // join: T_i is needed from here on
-      ops->tz(Zpart, vp, Tblk(r0), p->max_rank, 1, Zt, &ctrl->done, st);
+      if (t_aside) cudaStreamWaitEvent(st, h->sync_events[2 * i + 1], 0);   // join: T_i is needed from here on
       UpdPlan up = plan_upd(h->sms, rows, n, ops->u_bm, ops->u_bn, ops->u_wn);
       if (utc_on) up.tc = &utc;
       const int j0 = (i + 1 < steps) ? r0 + b : -1;   // Omega rows of the next pass, if there is one
+      ops->tz(Zpart, vp, Tblk(r0), p->max_rank, 1, Zt, &ctrl->done, tz_split(up.tc, j0, n), !t_aside, st);
       mark(RRF_PHASE_UPDATE, i);
       ops->update(tmV_u, tmZ, i == 0 ? tmA_u : tmW_u, tmO, W, ldw, (char*)dB + (size_t)r0 * ldb * esize, ldb, r0, rows, (int)n, r0, b,
-                  j0, Ypart, norm_part, up, ctrl, samp + i, st);
+                  j0, Ypart, norm_part, up, ctrl, samp + i, true, st);
       mark(RRF_PHASE_STOP, i);
-      stop_kernel<<<1, 256, 0, st>>>(norm_part, up.P, b, p->max_rank, p->estimator, fixed ? 1 : 0, tr_sub, tr_dir, ctrl,
-                                     done_after, 1, predicting ? samp : nullptr, predict);
+      launch_after(true, stop_kernel, 1, 256, 0, st, norm_part, up.P, b, p->max_rank, p->estimator, fixed ? 1 : 0, tr_sub, tr_dir,
+                   ctrl, done_after, 1, predicting ? samp : nullptr, predict);
       if (j0 >= 0 && predicting) {
         // the next panel, sampled on its own if the loop goes on and the update had been told to skip it
         const SamplePlan sp2 = plan_sample(h->sms, rows - b, n, esize, ops->s_kbs);
@@ -1940,17 +1969,17 @@ rrf_status_t rrf_run(rrf_handle_t h, const rrf_params_t* p, void* dA, int64_t ld
       vp.tc = tc;
       vp.chunk = h->tc_chunk;
       mark(RRF_PHASE_VTW, i);
-      ops->vtw(tmV_k, i == 0 ? tmA_k : tmW_k, Zpart, r0, r0, vp, ctrl, st);
+      ops->vtw(tmV_k, i == 0 ? tmA_k : tmW_k, Zpart, r0, r0, vp, ctrl, false, st);
       mark(RRF_PHASE_TZ, i);
-      ops->tz(Zpart, vp, Tblk(r0), p->max_rank, 1, Zt, &ctrl->done, st);
+      UpdPlan up = plan_upd(gsms, rows, n, ops->u_bm, ops->u_bn, ops->u_wn);
+      if (utc_on) up.tc = &utc;
+      const int j0 = (i + 2 < steps) ? r0 + 2 * b : -1;   // Omega rows of the pass after the next
+      ops->tz(Zpart, vp, Tblk(r0), p->max_rank, 1, Zt, &ctrl->done, tz_split(up.tc, j0, n), true, st);
       if (i + 1 < steps_run && gate) {
         cudaEventRecord(evZ(i), st);
         s = next_panel();
         if (s != RRF_OK) return panel_failed(s);
       }
-      UpdPlan up = plan_upd(gsms, rows, n, ops->u_bm, ops->u_bn, ops->u_wn);
-      if (utc_on) up.tc = &utc;
-      const int j0 = (i + 2 < steps) ? r0 + 2 * b : -1;   // Omega rows of the pass after the next
       // Gated passes: the panel kernel, started together with the update, is done long before it, and its SMs
       // would idle.  The last tiles of the pass are therefore left to a second launch of the update kernel that
       // follows the panel kernel on ITS stream and so runs on the SMs it leaves: `look_ctas` CTAs with as many
@@ -1982,22 +2011,22 @@ rrf_status_t rrf_run(rrf_handle_t h, const rrf_params_t* p, void* dA, int64_t ld
         uh.tpc = tpc2;
         uh.P = ceil_div(up.total - t1, tpc2);
         ops->update(tmV_u, tmZ, i == 0 ? tmA_u : tmW_u, tmO, W, ldw, (char*)dB + (size_t)r0 * ldb * esize, ldb, r0, rows, (int)n,
-                    r0, b, j0, Ybuf[i & 1], norm_part, um, ctrl, samp + i, st);
+                    r0, b, j0, Ybuf[i & 1], norm_part, um, ctrl, samp + i, true, st);
         // behind the panel kernel of pass i+1 on the side stream (which has waited for T Z of this pass)
         ops->update(tmV_u, tmZ, i == 0 ? tmA_u : tmW_u, tmO, W, ldw, (char*)dB + (size_t)r0 * ldb * esize, ldb, r0, rows, (int)n,
-                    r0, b, j0, Ybuf[i & 1], norm_part, uh, ctrl, samp + i, h->aux);
+                    r0, b, j0, Ybuf[i & 1], norm_part, uh, ctrl, samp + i, false, h->aux);
         cudaEventRecord(evH(i), h->aux);
         cudaStreamWaitEvent(st, evH(i), 0);
         up.tpc = um.tpc;          // what the loader of the sampled panel needs to find the partial results
         up.P = um.P + uh.P;
       } else {
         ops->update(tmV_u, tmZ, i == 0 ? tmA_u : tmW_u, tmO, W, ldw, (char*)dB + (size_t)r0 * ldb * esize, ldb, r0, rows, (int)n, r0, b,
-                    j0, Ybuf[i & 1], norm_part, up, ctrl, samp + i, st);
+                    j0, Ybuf[i & 1], norm_part, up, ctrl, samp + i, true, st);
       }
       const int up_t1 = t1, up_p1 = t1 > 0 ? ceil_div(t1, up.tpc) : 0, up_tpc2 = tpc2;
       mark(RRF_PHASE_STOP, i);
-      stop_kernel<<<1, 256, 0, st>>>(norm_part, up.P, b, p->max_rank, p->estimator, fixed ? 1 : 0, tr_sub, tr_dir, ctrl,
-                                     done_after, 0, predicting ? samp : nullptr, predict);
+      launch_after(t1 == 0, stop_kernel, 1, 256, 0, st, norm_part, up.P, b, p->max_rank, p->estimator, fixed ? 1 : 0, tr_sub,
+                   tr_dir, ctrl, done_after, 0, predicting ? samp : nullptr, predict);
       if (j0 >= 0 && predicting) {
         // the panel of pass i+2, sampled on its own if the loop goes on and the update had been told to skip it;
         // its first b rows are the rows above that panel which the fix-up needs

@@ -40,6 +40,13 @@ __device__ __forceinline__ uint32_t smem_u32(const void* p) {
   return static_cast<uint32_t>(__cvta_generic_to_shared(p));
 }
 
+// ---------------------------------------------------------------- programmatic dependent launch
+// The kernels of a pass follow one another on one stream.  A kernel launched as a programmatic dependent is put on the
+// SMs while the one before it drains and waits here, before its first access to global memory, until that one has
+// completed and its writes are visible.  Launched the ordinary way both calls do nothing.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
 // ---------------------------------------------------------------- mbarrier / TMA
 
 __device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {

@@ -53,6 +53,8 @@ __global__ void __launch_bounds__((WM * WN + 1) * 32)
     vtw_sk_kernel(const __grid_constant__ CUtensorMap tmV,  // V [m][ldv], box [BK][KE]
                   const __grid_constant__ CUtensorMap tmC,  // C [m][ncols], box [BK][KE]
                   T* __restrict__ Zpart, int r0, int cv0, int KT, int total, int tpc, Ctrl* ctrl) {
+  pdl_wait();
+  pdl_trigger();
   if (*reinterpret_cast<volatile int*>(&ctrl->done)) return;
   constexpr int KE = Elem<T>::KE;
   constexpr int NCW = WM * WN;
@@ -203,6 +205,8 @@ __global__ void __launch_bounds__((WM * WN + (PW ? 1 : 0)) * 32, 1)
                   int NC, int total, int tpc, Ctrl* ctrl,
                   const int* __restrict__ samp_flag,     // non-NULL: sample only if *samp_flag != 0
                   int p0, int Lb) {                      // this launch is CTAs p0 ... of the pass and starts at tile Lb
+  pdl_wait();
+  pdl_trigger();
   if (*reinterpret_cast<volatile int*>(&ctrl->done)) return;
   constexpr int KE = Elem<T>::KE, NV = Elem<T>::NV, KS = Elem<T>::KS;
   constexpr int U = KE / 8;            // n-tiles per 128-byte column group

@@ -10,7 +10,7 @@
 // The left operand of both products sits in TENSOR MEMORY (lane = row of the slab, one column per
 // contraction index): V is written there once per slab, Wnew once per tile by the very threads that
 // compute it, each split into its two TF32 planes on the way.  The right operands are Zt and OmegaT
-// rows, which arrive by TMA already split (split_planes_kernel wrote the planes to global memory:
+// rows, which arrive by TMA already split (tz_kernel wrote the planes to global memory:
 // both are small and stay in L2), K-contiguous with the ordinary 128-byte swizzle.  So shared memory
 // carries only what TMA brings - W, Zt planes, OmegaT planes - and is read once by the tensor core
 // and (W) once by the epilogue: about 220 KB of shared-memory traffic per 64 KB of HBM traffic.
@@ -33,21 +33,6 @@
 #include "panel_tsqr.cuh"
 
 namespace rrf {
-
-// dst[0][r][c] = tf32(src[r][c]), dst[1][r][c] = tf32(src[r][c] - dst[0][r][c]); dst planes have leading dimension ldd
-__global__ void split_planes_kernel(const float* __restrict__ src, long long lds, int rows, int cols,
-                                    float* __restrict__ dst, long long ldd, const int* __restrict__ done_flag) {
-  if (done_flag != nullptr && *done_flag) return;
-  const long long total = (long long)rows * cols;
-  const size_t plane = (size_t)rows * (size_t)ldd;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total; i += (long long)gridDim.x * blockDim.x) {
-    const int r = (int)(i / cols), c = (int)(i - (long long)r * cols);
-    const float x = src[(size_t)r * lds + c];
-    const float h = tf32_rn(x);
-    dst[(size_t)r * ldd + c] = h;
-    dst[plane + (size_t)r * ldd + c] = tf32_rn(x - h);
-  }
-}
 
 // K-contiguous shared-memory operand with the 128-byte swizzle: rows of 128 bytes, groups of eight rows 1024 bytes apart
 __device__ __forceinline__ uint64_t tc_desc_k(uint32_t addr) {
@@ -140,6 +125,8 @@ __global__ void __launch_bounds__(kUtcThreads, 1)
                   const float* __restrict__ V, long long ldv, int r0, int rows, int ncols, int cv0, int top_rows,
                   int sample, int npad, float* __restrict__ Ypart, double* __restrict__ norm_part,
                   int NC, int total, int tpc, int chunk, Ctrl* ctrl) {
+  pdl_wait();
+  pdl_trigger();
   if (*reinterpret_cast<volatile int*>(&ctrl->done)) return;
   using Cfg = UtcCfg<B>;
   constexpr int NW = Cfg::NW, NZ = Cfg::NZ, NO = Cfg::NO, W_BOX = Cfg::W_BOX, W_BYTES = Cfg::W_BYTES, Z_BOX = Cfg::Z_BOX,

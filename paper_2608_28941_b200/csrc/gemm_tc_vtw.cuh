@@ -52,6 +52,8 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     vtw_tc_kernel(const __grid_constant__ CUtensorMap tmV,  // V [m][ldv], box [32][32], 32-byte-atom swizzle
                    const __grid_constant__ CUtensorMap tmC,  // C [m][ncols], box [32][32], 32-byte-atom swizzle
                    float* __restrict__ Zpart, int r0, int cv0, int KT, int total, int tpc, int chunk, Ctrl* ctrl) {
+  pdl_wait();
+  pdl_trigger();
   if (*reinterpret_cast<volatile int*>(&ctrl->done)) return;
   using Cfg = TcCfg<B, RS, OS>;
   constexpr int NBV = Cfg::NBV, NBC = Cfg::NBC, BOX = Cfg::BOX, RAW = Cfg::RAW, OPS = Cfg::OPS, TA = Cfg::TA;

@@ -911,11 +911,54 @@ __global__ void __launch_bounds__(256)
 // ------------------------------------------------------------------------------------------
 constexpr int kTzCols = 32;
 constexpr int kTzThreads = 512;
+// With `sp` (the single-precision update on tcgen05 follows) the result goes out as its two TF32 planes instead, and the
+// CTAs past the first sp.ntz split the rows of OmegaT that update samples with: two small launches less per pass.
+struct TzSplit {
+  float* z;             // [2][npad][B] planes of the result; NULL: plain output
+  int npad;
+  const float* om;      // rows j0 ... j0 + B of OmegaT, 16-byte aligned
+  long long ldom;
+  int ncols;
+  float* o;             // [2][B][ldo] planes of them
+  long long ldo;
+  int ntz;              // CTAs that work on Z
+};
 template <typename T, int B, int COLS>
 __global__ void __launch_bounds__(kTzThreads)
     tz_kernel(const T* __restrict__ Zpart, int bn, int nct, int kt, int tpc, const T* __restrict__ Tm, long long ldt,
-              int transpose_t, T* __restrict__ Zt, const int* done_flag) {
+              int transpose_t, T* __restrict__ Zt, const int* done_flag, TzSplit sp) {
+  pdl_wait();
+  pdl_trigger();
   if (*reinterpret_cast<const volatile int*>(done_flag)) return;
+  if constexpr (sizeof(T) == 4) {
+    if ((int)blockIdx.x >= sp.ntz) {
+      const int nv = (sp.ncols + 3) >> 2;
+      const size_t plane = (size_t)B * (size_t)sp.ldo;
+      for (int r = blockIdx.x - sp.ntz; r < B; r += gridDim.x - sp.ntz) {
+#pragma unroll 4
+        for (int q = threadIdx.x; q < nv; q += kTzThreads) {
+          const float* src = sp.om + (size_t)r * sp.ldom + 4 * q;
+          float x[4], hi[4], lo[4];
+          if (4 * q + 4 <= sp.ncols) {
+            const float4 v = *reinterpret_cast<const float4*>(src);
+            x[0] = v.x; x[1] = v.y; x[2] = v.z; x[3] = v.w;
+          } else {
+#pragma unroll
+            for (int e = 0; e < 4; ++e) x[e] = 4 * q + e < sp.ncols ? src[e] : 0.f;
+          }
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            hi[e] = __uint_as_float(to_tf32(x[e]));
+            lo[e] = __uint_as_float(to_tf32(x[e] - hi[e]));
+          }
+          float* d = sp.o + (size_t)r * sp.ldo + 4 * q;      // ldo is a multiple of four
+          *reinterpret_cast<float4*>(d) = make_float4(hi[0], hi[1], hi[2], hi[3]);
+          *reinterpret_cast<float4*>(d + plane) = make_float4(lo[0], lo[1], lo[2], lo[3]);
+        }
+      }
+      return;
+    }
+  }
   constexpr int PA = B + 4, PB = COLS + 4;
   constexpr int NWARP = kTzThreads / 32;
   constexpr int MTILES = B / 16, NTILES = COLS / 8;
@@ -991,6 +1034,19 @@ __global__ void __launch_bounds__(kTzThreads)
       mma16x8x8(acc, af, bf);
     }
     const int j = j0 + g, col = col0 + n0 + 2 * t;
+    if constexpr (sizeof(T) == 4) {
+      if (sp.z != nullptr) {
+        const size_t plane = (size_t)sp.npad * B;
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          float* d = sp.z + (size_t)(col + (e & 1)) * B + j + 8 * (e >> 1);
+          const float hi = __uint_as_float(to_tf32(acc[e]));
+          d[0] = hi;
+          d[plane] = __uint_as_float(to_tf32(acc[e] - hi));
+        }
+        continue;
+      }
+    }
     Zt[(size_t)col * B + j] = acc[0];
     Zt[(size_t)(col + 1) * B + j] = acc[1];
     Zt[(size_t)col * B + j + 8] = acc[2];
@@ -1068,6 +1124,7 @@ __global__ void __launch_bounds__(256)
     stop_kernel(const double* __restrict__ norm_part, int npart, int b, int max_rank, int estimator,
                 int fixed_rank, double* __restrict__ tr_sub, double* __restrict__ tr_dir, Ctrl* ctrl,
                 int* __restrict__ done_after, int reset_bar, int* __restrict__ samp, int predict) {
+  pdl_wait();
   // the loop state is read at once, ahead of the sums, and not field by field behind them
   const int done0 = *reinterpret_cast<volatile int*>(&ctrl->done), status0 = ctrl->status, i = ctrl->steps;
   const double esub0 = ctrl->E_sub, sigma2 = ctrl->sigma2, eprev0 = ctrl->E_prev, rprev0 = ctrl->r_prev;
