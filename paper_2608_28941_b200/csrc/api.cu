@@ -439,10 +439,11 @@ struct PassModel {
     const double R = std::max(64.0, (rows + b) / ctas);
     return 12.0 + 0.8 * b + 7.6e-5 * R * b * b + 2e-3 * R * b;
   }
-  // the same on every SM, nothing to fix up (72 us for 8192 x 64, 50 for 20000 x 32); the column loop beyond b = 64
+  // the same on every SM, nothing to fix up (72 us for 8192 x 64, 50 for 20000 x 32); for b = 128 two halves and a fix-up, or
+  // in single precision the column loop
   double panel_alone() const {
     const double R = std::max(64.0, rows / sms);
-    return b > 64 ? b * 4.2 + 25.0 : 10.0 + 0.9 * b + 4e-5 * R * b * b + 1e-3 * R * b;
+    return b > 64 ? (f64 ? 190.0 + 0.2 * R : b * 4.2 + 25.0) : 10.0 + 0.9 * b + 4e-5 * R * b * b + 1e-3 * R * b;
   }
   // the stream-K GEMMs lose a little more than the SMs they give up (tile quantisation)
   double scale(int ctas) const { return std::pow((double)sms / (sms - ctas), 1.1); }
@@ -580,6 +581,7 @@ struct Ops {
       e = cudaFuncSetAttribute(upd_tc_kernel<B>, cudaFuncAttributeMaxDynamicSharedMemorySize, UtcCfg<B>::SMEM);
       if (e != cudaSuccess) return e;
     }
+    if (Z_SMEM <= 48 * 1024) return cudaSuccess;
     e = cudaFuncSetAttribute(tz_kernel<T, B, kTzCols>, cudaFuncAttributeMaxDynamicSharedMemorySize, Z_SMEM);
     if (e != cudaSuccess) return e;
     e = cudaFuncSetAttribute(tz_kernel<T, B, kTzCols / 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, Z_SMEM);
@@ -743,6 +745,62 @@ static rrf_status_t launch_panel(rrf_ctx* h, int dtype, const void* Y, PanelSour
     if (o.t_aside != nullptr) *o.t_aside = false;
     return RRF_OK;
   }
+  if (dtype == RRF_F64 && b == 2 * kHalf && !o.blocked && !o.global_slab && ps.gslab != nullptr && !o.fix.enabled && rows <= (long long)h->sms * 320) {
+    // two panels of 64 columns (see corner_part_kernel); their scratch lies where slabs in global memory would.  Not in
+    // single precision: the second half would see the first one's V and T rounded to 24 bits, where the column loop
+    // keeps the whole panel in 53 (largest error of V on a square Gaussian panel 1.8e-7 against 6e-8).
+    const int G = std::min(h->sms, ceil_div(rows, 64));
+    PanelScratch half = ps;
+    double* gpart = ps.gslab;
+    double* gm = gpart + (size_t)G * kHalf * kHalf;
+    half.cqr = gm + kHalf * kHalf;
+    const int esize = 8;
+    PanelSource s1 = src, s2 = src, a1 = o.alt, a2 = o.alt;
+    s1.sb = s2.sb = a1.sb = a2.sb = b;
+    s2.row_off += kHalf;
+    a2.row_off += kHalf;
+    PanelOpts po = o;
+    unsigned used1 = 0, used2 = 0;
+    po.merge_t = true;
+    po.bar_used = &used1;
+    po.alt = a1;
+    po.no_cluster = true;
+    po.ev_fork = po.ev_join = nullptr;
+    po.t_aside = nullptr;
+    int g1 = 0;
+    po.g_out = &g1;               // both launches have the same grid: their slabs cover the same rows
+    rrf_status_t hs = launch_panel(h, dtype, Y, s1, rows, kHalf, V, ldv, Tout, ldt, half, ctrl, done_flag, st, mark, step, po);
+    if (hs != RRF_OK) return hs;
+    po.alt = a2;
+    po.bar_base = o.bar_base + used1;
+    po.bar_used = &used2;
+    po.fix.enabled = 1;
+    po.fix.Vp = V;
+    po.fix.ldvp = ldv;
+    po.fix.Tp = Tout;
+    po.fix.ldtp = ldt;
+    po.fix.Gpart = gpart;
+    po.fix.M = gm;
+    po.fix.csq_before = 1;
+    if (o.csq != nullptr) po.csq = o.csq + (size_t)kHalf * ((g1 + 31) & ~31);
+    hs = launch_panel(h, dtype, (const char*)Y + (size_t)kHalf * esize, s2, rows - kHalf, kHalf,
+                      (char*)V + ((size_t)kHalf * ldv + kHalf) * esize, ldv, (char*)Tout + ((size_t)kHalf * ldt + kHalf) * esize, ldt,
+                      half, ctrl, done_flag, st, NoMark(), step, po);
+    if (hs != RRF_OK) return hs;
+    if (o.bar_used != nullptr) *o.bar_used = used1 + used2;
+    if (o.t_aside != nullptr) *o.t_aside = false;
+    if (o.g_out != nullptr) *o.g_out = g1;
+    const int per = std::max(64, (ceil_div(rows - kHalf, h->sms) + 31) / 32 * 32), parts = std::max(1, ceil_div(rows - kHalf, per));
+    corner_part_kernel<<<parts, kPanelThreads, 0, st>>>((const double*)V, ldv, (int)rows, per, gpart, done_flag);
+    corner_sum_kernel<<<kHalf, 256, 0, st>>>(gpart, parts, gm, done_flag);
+    corner_t_kernel<<<1, kPanelThreads, kCornerSmem, st>>>(gm, (double*)Tout, ldt, (double*)V, ldv, done_flag);
+    const cudaError_t ce = cudaGetLastError();
+    if (ce != cudaSuccess) {
+      h->last_cuda = (int)ce;
+      return RRF_ERR_CUDA;
+    }
+    return RRF_OK;
+  }
   int rows_i = (int)rows;
   double *P = ps.P, *piv = ps.piv, *gram = ps.gram, *tau = ps.tau;
   unsigned* bar = ps.bar;
@@ -782,7 +840,10 @@ static rrf_status_t launch_panel(rrf_ctx* h, int dtype, const void* Y, PanelSour
     e = cudaLaunchCooperativeKernel(fn, dim3(bp.G), dim3(kPanelThreads), args, smem, st);
   } else {
     PanelPlan pp;
-    const bool as_cluster = !o.no_cluster && !o.blocked && plan_panel_cl(h, rows, b, &pp, o.fix.enabled != 0);
+    // on a free device a tall panel is faster spread over the grid (4096 x 64: 62 us against 78 as one cluster, whose
+    // 16 SMs are then bound by their matrix products)
+    const bool spread = o.ctas == 0 && b == 64 && rows > 2048;
+    const bool as_cluster = !o.no_cluster && !spread && !o.blocked && plan_panel_cl(h, rows, b, &pp, o.fix.enabled != 0);
     if (!as_cluster && !plan_panel(h, rows, b, &pp, o.ctas, o.fix.enabled != 0)) return RRF_ERR_WORKSPACE;
     int R = pp.R, Rp = pp.Rp;
     void* args[] = {&Y,   &src, &alt, &fused_flag, &rows_i, &b,    &R,    &Rp,        &V,   &ldv,      &P,
@@ -935,6 +996,8 @@ static cudaError_t setup_all(int smem_optin, int* panel_smem_max, int* cluster_o
     e = get_ops(RRF_F32, b)->setup();
     if (e != cudaSuccess) return e;
   }
+  e = cudaFuncSetAttribute(corner_t_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kCornerSmem);
+  if (e != cudaSuccess) return e;
   return setup_panel_kernels(smem_optin, panel_smem_max, cluster_ok);
 }
 
@@ -2176,14 +2239,16 @@ rrf_status_t rrf_run(rrf_handle_t h, const rrf_params_t* p, void* dA, int64_t ld
     // without the predictor every executed pass that has a later panel to sample samples it
     out->fused_samples = predicting ? hc.fused_samples : std::min(hc.steps, std::max(0, steps - lag));
     const int sl = steps_run;      // passes whose kernels were launched
+    // panel: one kernel with T in it; two halves and the corner for b = 128; the T factor apart where neither applies
+    const bool two_halves = p->dtype == RRF_F64 && b == 2 * kHalf && !blocked && m <= (long long)h->sms * 320;
+    const bool t_apart = !two_halves && look_ctas == 0 && !tree && !unchanged && (b > 64 || blocked);
+    const int pl = two_halves ? 5 : (t_apart ? 2 : 1);
+    const int first = 2 + (dOmegaT == nullptr ? 1 : 0);           // sample, loop state, the library's own vectors
     if (unchanged)
-      out->kernel_launches = (dOmegaT == nullptr ? 1 : 0) + 1 + 4 * sl + 3 * sl * (sl - 1) / 2;
+      out->kernel_launches = first - 1 + (3 + pl) * sl + 3 * sl * (sl - 1) / 2;
     else
-    out->kernel_launches = (sampled ? sl : 0) + 1 + (dOmegaT == nullptr ? 1 : 0) + 1 + ((look_ctas > 0 && steps > 1) ? 1 : 0) +
-                           ((look_ctas > 0 || tree) ? 5 : 6) * sl +   // look-ahead, tree kernel: the panel kernel builds T itself
-                           (predicting ? std::max(0, std::min(sl, steps - lag)) : 0) +
-                           ((p->dtype == RRF_F32 && h->f32_engine == 1 && get_ops(p->dtype, b)->has_upd_tc)   // TF32 planes of Zt, OmegaT's rows
-                                ? sl + std::max(0, std::min(sl, steps - lag)) : 0);
+      out->kernel_launches = first + ((look_ctas > 0 && steps > 1) ? 1 : 0) + (pl + 4 + (sampled ? 1 : 0)) * sl +
+                             (predicting ? std::max(0, std::min(sl, steps - lag)) : 0);
   }
   out->extra_samples = hc.extra_samples;
   out->panel_ctas = look_ctas;

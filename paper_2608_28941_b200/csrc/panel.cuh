@@ -32,6 +32,7 @@ struct PanelSource {
   int ldy;                 // stacked: leading dimension
   int row_off;             // panel row 0 is row `row_off` of the producer's row numbering
   int bm, nc, tpc, wn;     // slots: slab height, tiles per slab, tiles per CTA, warp columns
+  int sb;                  // slots: columns of a partial result (0: those of the panel)
   int t1, p1, tpc2;        // slots: tiles from t1 on belong to CTAs p1, p1 + 1, ... at tpc2 tiles each (t1 <= 0: none)
 };
 // CTA (= slot) that computed tile L of a pass
@@ -51,6 +52,7 @@ struct PanelFix {
   long long ldtp;
   double* Gpart;           // [gridDim.x][b*b] per-CTA partial Vp^T P
   double* M;               // [b*b] Tp^T (Vp^T P)
+  int csq_before;          // the column sums of squares are those of P, all rows, and not of Y
 };
 constexpr int kFixChunk = 32;   // rows of Vp staged in shared memory at a time
 // doubles of shared memory the fix-up needs on top of panel_extra_doubles: the staged rows of Vp
@@ -70,12 +72,13 @@ __device__ __forceinline__ double panel_entry(const T* __restrict__ Y, const Pan
     s = (double)p[0];                     // not 0.0 + p[0]: a lone -0.0 keeps its sign (it decides a reflector's)
     for (int sg = 1; sg < src.nseg; ++sg) s += (double)p[(size_t)sg * src.seg_stride];
   } else {
+    const int sb = src.sb > 0 ? src.sb : b;
     const int lr = r + src.row_off;
     const int sl = lr / src.bm, rl = lr - sl * src.bm;
     const int p_lo = slot_cta(src, sl * src.nc), p_hi = slot_cta(src, (sl + 1) * src.nc - 1);
     for (int p = p_lo; p <= p_hi; ++p)
       for (int w = 0; w < src.wn; ++w)
-        s += (double)Y[((size_t)(p + sl) * src.wn + w) * (size_t)(src.bm * b) + (size_t)rl * b + c];
+        s += (double)Y[((size_t)(p + sl) * src.wn + w) * (size_t)(src.bm * sb) + (size_t)rl * sb + c];
   }
   return s;
 }
@@ -100,7 +103,8 @@ __device__ __forceinline__ void panel_load_slab(const T* __restrict__ Y, const P
     tab[tid] = make_int2((p_lo + sl) * src.wn, (p_hi - p_lo + 1) * src.wn);
   }
   __syncthreads();
-  const size_t tstride = src.slots ? (size_t)src.bm * b : (size_t)src.seg_stride;
+  const int sb = src.sb > 0 ? src.sb : b;
+  const size_t tstride = src.slots ? (size_t)src.bm * sb : (size_t)src.seg_stride;
   if ((reinterpret_cast<uintptr_t>(Y) & 15) == 0 && (src.slots || (src.ldy % VEC == 0 && src.seg_stride % VEC == 0))) {
     struct __align__(16) Vec { T v[VEC]; };
     const int lane = tid & 31, nw = nthr >> 5;
@@ -123,7 +127,7 @@ __device__ __forceinline__ void panel_load_slab(const T* __restrict__ Y, const P
           if (src.slots) {
             const int2 s = tab[(lr >> sbm) - sl0];
             cnt[e] = s.y;
-            ptr[e] = Y + (size_t)s.x * tstride + (size_t)(lr & (src.bm - 1)) * b + c;
+            ptr[e] = Y + (size_t)s.x * tstride + (size_t)(lr & (src.bm - 1)) * sb + c;
           } else {
             cnt[e] = src.nseg;
             ptr[e] = Y + (size_t)lr * src.ldy + c;
@@ -338,6 +342,21 @@ __global__ void __launch_bounds__(kPanelThreads)
   }
   __syncthreads();
 
+  // Sums of squares of the columns from slab row `first` on: the sampled stopping rules estimate the residual from those
+  // of the panel as sampled (est_kernel).  One warp per column, fixed order.
+  auto column_squares = [&](int first) {
+    for (int c = warp; c < b; c += NW) {
+      double a = 0.0;
+      for (int r = lane; r < nloc; r += 32) {
+        const double v = (gr0 + r >= first) ? S[(size_t)c * Rp + r] : 0.0;
+        a += v * v;
+      }
+      a = warp_sum(a);
+      if (lane == 0) csq[(size_t)c * Gp + cta] = a;
+    }
+  };
+  if (csq != nullptr && fix.csq_before) column_squares(0);
+
   if (fix.enabled) {
     // ---- S <- P - Vp (Tp^T (Vp^T P)) on the tensor cores (FP64 m16n8k8)
     const int g = lane >> 2, t = lane & 3;
@@ -487,19 +506,7 @@ __global__ void __launch_bounds__(kPanelThreads)
     __syncthreads();
   }
 
-  // Sums of squares of the columns of the panel as sampled (after the fix-up): the sampled stopping rules
-  // estimate the residual from them (est_kernel).  One warp per column, fixed order.
-  if (csq != nullptr) {
-    for (int c = warp; c < b; c += NW) {
-      double a = 0.0;
-      for (int r = lane; r < nloc; r += 32) {
-        const double v = (gr0 + r >= row0) ? S[(size_t)c * Rp + r] : 0.0;
-        a += v * v;
-      }
-      a = warp_sum(a);
-      if (lane == 0) csq[(size_t)c * Gp + cta] = a;
-    }
-  }
+  if (csq != nullptr && !fix.csq_before) column_squares(row0);
 
   // Cholesky QR with reconstruction where it is safe; the column loop below does the rest
   const bool try_cqr = PAD && (!CL || REG) && cqr != nullptr && b <= 64 && rows > b;
@@ -880,6 +887,138 @@ __global__ void __launch_bounds__(kPanelThreads)
     if (total > nbar) atomicAdd(bar, total - nbar);
   }
 }
+
+// ------------------------------------------------------------------------------------------
+// In double precision a block of 128 columns is factored as two panels of 64: the second is the panel of P = columns 64 ... with the first
+// block's reflectors still to be applied, which is the fix-up of the look-ahead schedule.  V is then the two blocks of
+// Householder vectors side by side, and T = [T1  -T1 (V1^T V2) T2; 0  T2].  These kernels add the corner: partial
+// V1^T V2 over ranges of rows, their sum, the two products.
+// (As one panel of 128 the slab fills shared memory and only the column loop is left: 32768 x 128 in 980 us.)
+// ------------------------------------------------------------------------------------------
+constexpr int kHalf = 64;
+__global__ void __launch_bounds__(kPanelThreads)
+    corner_part_kernel(const double* __restrict__ V, long long ldv, int rows, int per, double* __restrict__ part, const int* done_flag) {
+  if (*reinterpret_cast<const volatile int*>(done_flag)) return;
+  constexpr int PV = kHalf + 8;
+  __shared__ double s1[32 * PV], s2[32 * PV];
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
+  const int lo = kHalf + blockIdx.x * per, hi = min(rows, lo + per);      // V2 is zero above row 64
+  const int mt = warp >> 2, np = warp & 3;
+  double acc[2][4] = {};
+  double p1[4], p2[4];
+  auto fetch = [&](int r0) {
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      const int idx = tid + e * kPanelThreads, r = r0 + (idx >> 6), c = idx & 63;
+      p1[e] = r < hi ? V[(size_t)r * ldv + c] : 0.0;
+      p2[e] = r < hi ? V[(size_t)r * ldv + kHalf + c] : 0.0;
+    }
+  };
+  fetch(lo);
+  for (int r0 = lo; r0 < hi; r0 += 32) {
+    __syncthreads();
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      const int idx = tid + e * kPanelThreads;
+      s1[(idx >> 6) * PV + (idx & 63)] = p1[e];
+      s2[(idx >> 6) * PV + (idx & 63)] = p2[e];
+    }
+    __syncthreads();
+    fetch(r0 + 32);
+#pragma unroll
+    for (int ks = 0; ks < 4; ++ks) {
+      const double* va = s1 + (ks * 8 + t) * PV + mt * 16 + g;
+      const double af[4] = {va[0], va[8], va[4 * PV], va[4 * PV + 8]};
+#pragma unroll
+      for (int i = 0; i < 2; ++i) {
+        const double* sb = s2 + (ks * 8 + t) * PV + (np * 2 + i) * 8 + g;
+        const double bf[2] = {sb[0], sb[4 * PV]};
+        mma16x8x8(acc[i], af, bf);
+      }
+    }
+  }
+  double* gp = part + (size_t)blockIdx.x * kHalf * kHalf;
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {
+    const int col = (np * 2 + i) * 8 + 2 * t, row = mt * 16 + g;
+    *reinterpret_cast<double2*>(gp + row * kHalf + col) = make_double2(acc[i][0], acc[i][1]);
+    *reinterpret_cast<double2*>(gp + (row + 8) * kHalf + col) = make_double2(acc[i][2], acc[i][3]);
+  }
+}
+// entry e of the sum over the parts, in a fixed order: four threads an entry
+__global__ void __launch_bounds__(256)
+    corner_sum_kernel(const double* __restrict__ part, int np, double* __restrict__ sum, const int* done_flag) {
+  if (*reinterpret_cast<const volatile int*>(done_flag)) return;
+  __shared__ double red[4][64];
+  const int e = threadIdx.x & 63, q = threadIdx.x >> 6, at = blockIdx.x * 64 + e;
+  double s = 0.0;
+  for (int x0 = q; x0 < np; x0 += 32) {
+    double v[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) v[u] = x0 + 4 * u < np ? __ldcg(part + (size_t)(x0 + 4 * u) * kHalf * kHalf + at) : 0.0;
+#pragma unroll
+    for (int u = 0; u < 8; ++u) s += v[u];
+  }
+  red[q][e] = s;
+  __syncthreads();
+  if (q == 0) sum[at] = (red[0][e] + red[1][e]) + (red[2][e] + red[3][e]);
+}
+// T12 = -T1 G T2, T21 = 0, and the zeros of V above its second block
+__global__ void __launch_bounds__(kPanelThreads)
+    corner_t_kernel(const double* __restrict__ G, double* __restrict__ Tm, long long ldt, double* __restrict__ V, long long ldv,
+                    const int* done_flag) {
+  if (*reinterpret_cast<const volatile int*>(done_flag)) return;
+  constexpr int P = kHalf + 4, N = kHalf * kHalf;
+  extern __shared__ double csm[];
+  double *A = csm, *Bm = csm + kHalf * P, *X = Bm + kHalf * P;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
+  auto product = [&](const double* L, const double* R, double (&acc)[2][4]) {      // 16 x 16 of L R a warp
+    const int mt = warp >> 2, np = warp & 3;
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+#pragma unroll
+      for (int e = 0; e < 4; ++e) acc[i][e] = 0.0;
+#pragma unroll
+    for (int ks = 0; ks < 8; ++ks) {
+      const double* l = L + (mt * 16 + g) * P + ks * 8 + t;
+      const double af[4] = {l[0], l[8 * P], l[4], l[8 * P + 4]};
+#pragma unroll
+      for (int i = 0; i < 2; ++i) {
+        const double* r = R + (ks * 8 + t) * P + (np * 2 + i) * 8 + g;
+        const double bf[2] = {r[0], r[4 * P]};
+        mma16x8x8(acc[i], af, bf);
+      }
+    }
+  };
+  for (int idx = tid; idx < N; idx += kPanelThreads) {
+    const int r = idx >> 6, c = idx & 63;
+    A[r * P + c] = c >= r ? Tm[(size_t)r * ldt + c] : 0.0;
+    Bm[r * P + c] = __ldcg(G + idx);
+    Tm[(size_t)(kHalf + r) * ldt + c] = 0.0;
+    V[(size_t)r * ldv + kHalf + c] = 0.0;
+  }
+  __syncthreads();
+  double acc[2][4];
+  product(A, Bm, acc);
+  const int r0 = (warp >> 2) * 16 + g;
+#pragma unroll
+  for (int i = 0; i < 2; ++i)
+#pragma unroll
+    for (int e = 0; e < 4; ++e) X[(r0 + 8 * (e >> 1)) * P + ((warp & 3) * 2 + i) * 8 + 2 * t + (e & 1)] = acc[i][e];
+  __syncthreads();
+  for (int idx = tid; idx < N; idx += kPanelThreads) {
+    const int r = idx >> 6, c = idx & 63;
+    A[r * P + c] = c >= r ? Tm[(size_t)(kHalf + r) * ldt + kHalf + c] : 0.0;
+  }
+  __syncthreads();
+  product(X, A, acc);
+#pragma unroll
+  for (int i = 0; i < 2; ++i)
+#pragma unroll
+    for (int e = 0; e < 4; ++e)
+      Tm[(size_t)(r0 + 8 * (e >> 1)) * ldt + kHalf + ((warp & 3) * 2 + i) * 8 + 2 * t + (e & 1)] = -acc[i][e];
+}
+constexpr int kCornerSmem = 3 * kHalf * (kHalf + 4) * 8;
 
 // ------------------------------------------------------------------------------------------
 // Compact-WY factor from the Gram rows (Eq. "Q_i = I_m - V_i T_i V_i^T").  The column recurrence

@@ -86,6 +86,22 @@ def test_single_precision(h, b, rows):
     check(h, panel("gauss", rows, b, np.random.default_rng(rows)), "f32")
 
 
+@pytest.mark.parametrize("dtype", ["f64", "f32"])
+@pytest.mark.parametrize("rows", [128, 129, 192, 200, 1000, 4097, 30000])
+def test_two_halves(h, rows, dtype):
+    """128 columns are two panels of 64 in double precision (in single the column loop does them): square, with a square
+    second half, ragged ends, many slabs."""
+    check(h, panel("gauss", rows, 128, np.random.default_rng(rows)), dtype)
+
+
+@pytest.mark.parametrize("kind", ["cond6", "cond9", "dependent", "zero", "nothing-below"])
+def test_two_halves_conditioning(h, kind):
+    V, T = check(h, panel(kind, 1500, 128, np.random.default_rng(3)), "f64")
+    if kind == "nothing-below":
+        assert not T.any()
+        assert np.array_equal(V, np.eye(1500, 128))
+
+
 @pytest.mark.parametrize("zero", [0.0, -0.0])
 @pytest.mark.parametrize("rows,b", [(500, 16), (9000, 64)])
 def test_zero_first_pivot_keeps_its_sign(h, rows, b, zero):
