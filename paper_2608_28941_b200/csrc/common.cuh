@@ -112,8 +112,23 @@ __device__ __forceinline__ void mma16x8x8(double (&c)[4], const double (&a)[4], 
 }
 
 // x rounded to TF32, nearest, ties away from zero, by two integer operations: the bits of cvt.rna.tf32.f32 for every
-// number that is not a NaN, at half its cost (2.1 against 4.1 cycles a warp)
+// number that is not a NaN, at half its cost (2.1 against 4.1 cycles a warp).  The NaN that GPU arithmetic produces
+// (0x7fffffff) wraps to -0, so operands are rounded by split_tf32 only.
 __device__ __forceinline__ uint32_t to_tf32(float x) { return (__float_as_uint(x) + 0x1000u) & 0xffffe000u; }
+// x = hi + lo in two TF32 numbers, hi = tf32(x), lo = tf32(x - hi).  A NaN or infinity in x is a NaN in lo, whatever
+// became of hi, and so in every product that takes the pair: 0 d is NaN for such a remainder and adds nothing to any
+// other, for one instruction of the FP32 pipe (a comparison and a selection would go to the pipe the rounding fills).
+__device__ __forceinline__ void split_tf32(float x, float& hi, float& lo) {
+  hi = __uint_as_float(to_tf32(x));
+  const float d = x - hi;
+  lo = fmaf(d, 0.f, __uint_as_float(to_tf32(d)));
+}
+__device__ __forceinline__ void split_tf32(float x, uint32_t& hi, uint32_t& lo) {
+  float h, l;
+  split_tf32(x, h, l);
+  hi = __float_as_uint(h);
+  lo = __float_as_uint(l);
+}
 __device__ __forceinline__ void mma_tf32(float (&c)[4], const uint32_t (&a)[4], const uint32_t (&b)[2]) {
   asm(
       "mma.sync.aligned.m16n8k8.row.col.f32.tf32.tf32.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
@@ -127,15 +142,9 @@ __device__ __forceinline__ void mma_tf32(float (&c)[4], const uint32_t (&a)[4], 
 __device__ __forceinline__ void mma16x8x8(float (&c)[4], const float (&a)[4], const float (&b)[2]) {
   uint32_t ah[4], al[4], bh[2], bl[2];
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    ah[i] = to_tf32(a[i]);
-    al[i] = to_tf32(a[i] - __uint_as_float(ah[i]));
-  }
+  for (int i = 0; i < 4; ++i) split_tf32(a[i], ah[i], al[i]);
 #pragma unroll
-  for (int i = 0; i < 2; ++i) {
-    bh[i] = to_tf32(b[i]);
-    bl[i] = to_tf32(b[i] - __uint_as_float(bh[i]));
-  }
+  for (int i = 0; i < 2; ++i) split_tf32(b[i], bh[i], bl[i]);
   float d[4] = {0.f, 0.f, 0.f, 0.f};
   mma_tf32(d, al, bh);
   mma_tf32(d, ah, bl);
@@ -160,8 +169,7 @@ struct Op<float> {
 __device__ __forceinline__ Op<double> prep(double x) { return Op<double>{x}; }
 __device__ __forceinline__ Op<float> prep(float x) {
   Op<float> o;
-  o.hi = to_tf32(x);
-  o.lo = to_tf32(x - __uint_as_float(o.hi));
+  split_tf32(x, o.hi, o.lo);
   return o;
 }
 __device__ __forceinline__ void mma_op(double (&c)[4], const Op<double>& a0, const Op<double>& a1, const Op<double>& a2,

@@ -99,11 +99,6 @@ __device__ __forceinline__ void tmem_ld16x4(uint32_t t0, uint32_t t1, uint32_t t
   }
 }
 
-// x rounded to TF32 (nearest, ties away from zero - what cvt.rna.tf32.f32 returns) with two integer
-// instructions, which issue at the full rate where the conversion instruction does not.  A NaN may come out as a
-// signed zero; the kernels below use the planes only as tensor-core operands and keep x itself for everything else.
-__device__ __forceinline__ float tf32_rn(float x) { return __uint_as_float((__float_as_uint(x) + 0x1000u) & 0xFFFFE000u); }
-
 constexpr int kTcBN = 128;     // columns of W per accumulator = rows of D = tensor-memory lanes
 constexpr int kTcSub = 32;     // rows (contraction indices) per ring stage; a 64-row tile is two stages
 constexpr int kTcConv = 8;     // warps that split operands and drain the accumulator

@@ -354,10 +354,7 @@ __global__ void __launch_bounds__(kUtcThreads, 1)
             if (lr < rows) x = *reinterpret_cast<const float4*>(vrow + g * 16 + e4 * 4);
             const float xs[4] = {x.x, x.y, x.z, x.w};
 #pragma unroll
-            for (int e = 0; e < 4; ++e) {
-              hi[e4 * 4 + e] = tf32_rn(xs[e]);
-              lo[e4 * 4 + e] = tf32_rn(xs[e] - hi[e4 * 4 + e]);
-            }
+            for (int e = 0; e < 4; ++e) split_tf32(xs[e], hi[e4 * 4 + e], lo[e4 * 4 + e]);
           }
           tmem_st16(tlane + TV + half * HB + g * 16, hi);
           tmem_st16(tlane + TV + B + half * HB + g * 16, lo);
@@ -445,10 +442,7 @@ __global__ void __launch_bounds__(kUtcThreads, 1)
         for (int g = 0; g < 2; ++g) {
           float hi[16], lo[16];
 #pragma unroll
-          for (int e = 0; e < 16; ++e) {
-            hi[e] = tf32_rn(y[g * 16 + e]);
-            lo[e] = tf32_rn(y[g * 16 + e] - hi[e]);
-          }
+          for (int e = 0; e < 16; ++e) split_tf32(y[g * 16 + e], hi[e], lo[e]);
           tmem_st16(tlane + TW + half * 32 + g * 16, hi);
           tmem_st16(tlane + TW + BN + half * 32 + g * 16, lo);
         }

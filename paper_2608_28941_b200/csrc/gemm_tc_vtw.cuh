@@ -167,8 +167,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
         for (int kk = 0; kk < 16; ++kk) {
           const int k = half * 16 + kk;
           const float x = lds32(wbox + k * 128 + ((((uint32_t)lane >> 3) ^ ((uint32_t)k & 3u)) << 5));
-          hi[kk] = tf32_rn(x);
-          lo[kk] = tf32_rn(x - hi[kk]);
+          split_tf32(x, hi[kk], lo[kk]);
         }
         tmem_st16(tlane + TA + o * 64 + half * 16, hi);
         tmem_st16(tlane + TA + o * 64 + 32 + half * 16, lo);
@@ -182,14 +181,10 @@ __global__ void __launch_bounds__(kTcThreads, 1)
 #pragma unroll
         for (int bx = 0; bx < NBV; ++bx) {
           float4 h, l;
-          h.x = tf32_rn(x[bx].x);
-          h.y = tf32_rn(x[bx].y);
-          h.z = tf32_rn(x[bx].z);
-          h.w = tf32_rn(x[bx].w);
-          l.x = tf32_rn(x[bx].x - h.x);
-          l.y = tf32_rn(x[bx].y - h.y);
-          l.z = tf32_rn(x[bx].z - h.z);
-          l.w = tf32_rn(x[bx].w - h.w);
+          split_tf32(x[bx].x, h.x, l.x);
+          split_tf32(x[bx].y, h.y, l.y);
+          split_tf32(x[bx].z, h.z, l.z);
+          split_tf32(x[bx].w, h.w, l.w);
           sts128(dst + bx * BOX, h);
           sts128(dst + (NBV + bx) * BOX, l);
         }

@@ -10,6 +10,10 @@ namespace rrf {
 __global__ void __launch_bounds__(32) timeout_selftest_kernel(unsigned* ctr, Ctrl* ctrl, long long limit) {
   grid_barrier(ctr, 2u, ctrl, limit);
 }
+// The library's own arithmetic, element by element, for tests.
+__global__ void __launch_bounds__(256) split_selftest_kernel(long long n, const float* __restrict__ x, float* __restrict__ hi, float* __restrict__ lo) {
+  for (long long i = blockIdx.x * 256LL + threadIdx.x; i < n; i += gridDim.x * 256LL) split_tf32(x[i], hi[i], lo[i]);
+}
 
 // ------------------------------------------------------------------------------------------
 // Householder QR of a rows x b panel.  Each CTA keeps a slab of R consecutive rows in shared
@@ -1086,10 +1090,7 @@ __global__ void __launch_bounds__(kTzThreads)
             for (int e = 0; e < 4; ++e) x[e] = 4 * q + e < sp.ncols ? src[e] : 0.f;
           }
 #pragma unroll
-          for (int e = 0; e < 4; ++e) {
-            hi[e] = __uint_as_float(to_tf32(x[e]));
-            lo[e] = __uint_as_float(to_tf32(x[e] - hi[e]));
-          }
+          for (int e = 0; e < 4; ++e) split_tf32(x[e], hi[e], lo[e]);
           float* d = sp.o + (size_t)r * sp.ldo + 4 * q;      // ldo is a multiple of four
           *reinterpret_cast<float4*>(d) = make_float4(hi[0], hi[1], hi[2], hi[3]);
           *reinterpret_cast<float4*>(d + plane) = make_float4(lo[0], lo[1], lo[2], lo[3]);
@@ -1179,9 +1180,7 @@ __global__ void __launch_bounds__(kTzThreads)
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
           float* d = sp.z + (size_t)(col + (e & 1)) * B + j + 8 * (e >> 1);
-          const float hi = __uint_as_float(to_tf32(acc[e]));
-          d[0] = hi;
-          d[plane] = __uint_as_float(to_tf32(acc[e] - hi));
+          split_tf32(acc[e], d[0], d[plane]);
         }
         continue;
       }

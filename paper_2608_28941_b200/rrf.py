@@ -45,7 +45,7 @@ class rrf_profile_t(C.Structure):
     _fields_ = [("ms", C.c_double * 9), ("launches", C.c_int32 * 9), ("pad", C.c_int32)]
 
 
-EXPORTS = ["rrf_run_colmajor", "rrf_colmajor_workspace_bytes", "rrf_transpose", "rrf_set_single_engine", "rrf_sample_workspace_bytes", "rrf_sample_panel", "rrf_frobenius_sq", "rrf_panel_qr_blocked", "rrf_panel_qr_tree", "rrf_transfer_workspace_bytes", "rrf_subspace_transfer", "rrf_selftest_timeout", "rrf_panel_qr_static", "rrf_set_profiling", "rrf_get_profile", "rrf_measure_peak", "rrf_create", "rrf_destroy", "rrf_workspace_bytes", "rrf_run", "rrf_panel_workspace_bytes",
+EXPORTS = ["rrf_run_colmajor", "rrf_colmajor_workspace_bytes", "rrf_transpose", "rrf_set_single_engine", "rrf_sample_workspace_bytes", "rrf_sample_panel", "rrf_frobenius_sq", "rrf_panel_qr_blocked", "rrf_panel_qr_tree", "rrf_transfer_workspace_bytes", "rrf_subspace_transfer", "rrf_selftest_timeout", "rrf_selftest_arithmetic", "rrf_panel_qr_static", "rrf_set_profiling", "rrf_get_profile", "rrf_measure_peak", "rrf_create", "rrf_destroy", "rrf_workspace_bytes", "rrf_run", "rrf_panel_workspace_bytes",
            "rrf_panel_qr", "rrf_apply_workspace_bytes", "rrf_apply_qt", "rrf_apply_q", "rrf_form_q",
            "rrf_fill_omega", "rrf_last_status", "rrf_status_string"]
 
@@ -87,6 +87,7 @@ def load():
                                           vp, i64, vp, sz, vp]
     lib.rrf_last_status.argtypes = [vp, vp]
     lib.rrf_selftest_timeout.argtypes = [vp, C.c_double, vp]
+    lib.rrf_selftest_arithmetic.argtypes = [vp, C.c_int32, C.c_int64, vp, vp, vp, vp]
     lib.rrf_set_single_engine.argtypes = [vp, i32, i32]
     lib.rrf_set_profiling.argtypes = [vp, i32]
     lib.rrf_get_profile.argtypes = [vp, C.POINTER(rrf_profile_t)]
@@ -471,3 +472,13 @@ def rrf_selftest_timeout(h, limit_ms: float = 50.0) -> int:
     if s != RRF_OK:
         raise RrfError(s, "rrf_selftest_timeout")
     return rrf_last_status(h)
+
+
+def rrf_selftest_arithmetic(h, which: int, x: torch.Tensor):
+    """The kernels' own arithmetic on the elements of x (see rrf.h): two tensors of x's type."""
+    first, second = torch.empty_like(x), torch.empty_like(x)
+    s = load().rrf_selftest_arithmetic(h, which, x.numel(), C.c_void_p(x.data_ptr()), C.c_void_p(first.data_ptr()),
+                                       C.c_void_p(second.data_ptr()), _stream())
+    if s != RRF_OK:
+        raise RrfError(s, "rrf_selftest_arithmetic")
+    return first, second
