@@ -145,6 +145,7 @@ __device__ __forceinline__ bool cqr_chol8(double* __restrict__ blk, const double
     for (int j = p; j < 8; ++j) a[j * (j + 1) / 2 + p] *= q;
     thr[p] = q;
   }
+  __syncwarp();                      // every lane has its copy before the first one is overwritten
   // every lane stores the same value
 #pragma unroll
   for (int j = 0; j < 8; ++j)
@@ -461,7 +462,9 @@ __device__ __forceinline__ bool cqr_lu8(double* __restrict__ A, const double* __
       x[i] *= ri;
       l[i * (i - 1) / 2 + c] = x[i];
     }
-    // every lane stores the same value: a branch here would end the block the compiler schedules over
+    // every lane stores the same value: a branch here would end the block the compiler schedules over.  All of them
+    // have loaded this column by then (nx, one column ago).
+    __syncwarp();
 #pragma unroll
     for (int i = 0; i < 8; ++i) blk[i * PA + c] = x[i];
     sgn[8 * K + c] = sv[c];

@@ -115,3 +115,15 @@ def test_squares_that_overflow(h):
     rrf.rrf_panel_qr(h, torch.from_numpy(panel("huge", 900, 32, np.random.default_rng(1))).cuda())
     torch.cuda.synchronize()
     check(h, panel("gauss", 900, 32, np.random.default_rng(2)), "f64")
+
+
+@pytest.mark.parametrize("b", [16, 32, 64])
+@pytest.mark.parametrize("rows", [700, 6000])
+@pytest.mark.parametrize("kind", ["gauss", "cond6"])
+def test_repeats_itself(h, b, rows, kind):
+    """Warps that factor a block in place, all lanes alike, keep their lanes apart: the same bits two hundred times."""
+    Y = torch.from_numpy(panel(kind, rows, b, np.random.default_rng(rows))).cuda()
+    V, T = rrf.rrf_panel_qr(h, Y)
+    for _ in range(200):
+        v, t = rrf.rrf_panel_qr(h, Y)
+        assert torch.equal(v, V) and torch.equal(t, T)
