@@ -224,9 +224,11 @@ rrf_status_t rrf_transpose(rrf_handle_t h, int32_t dtype, int64_t rows, int64_t 
  * tall device panel Y (rows x b, ldy >= b) into V (rows x b, ldv >= b, unit lower trapezoidal,
  * explicit ones and zeros) and the compact-WY factor T (b x b, ldt >= b, upper triangular) with
  * H_0 ... H_{b-1} = I - V T V^T.  Reflector convention: beta = -sign(alpha) ||x||, v_0 = 1,
- * tau = (beta - alpha)/beta.  R is not returned.  Workspace: rrf_panel_workspace_bytes().
- * Any height: a panel whose slabs do not fit in the SMs' shared memory (more than about 32000 x 128 or
- * 47000 x 64 doubles on 148 SMs) is factored by the blocked kernel with its slabs in global memory.
+ * tau = (beta - alpha)/beta.  R is not returned.  Workspace: rrf_panel_workspace_bytes(), 16-byte aligned (on 8 bytes
+ * only, the blocked kernel is not used: the column-by-column kernel takes its place, and a panel that needs it is
+ * refused with RRF_ERR_WORKSPACE, as is any other alignment).
+ * Any height: a panel whose slabs do not fit in the SMs' shared memory (more than about 47000 x 64 or, in double
+ * precision, 47000 x 128; 32000 x 128 in single) is factored by the blocked kernel with its slabs in global memory.
  * Does not synchronise the stream; a timeout of the in-kernel grid barrier is reported by
  * the next rrf_last_status() call.
  */

@@ -1277,9 +1277,11 @@ static rrf_status_t panel_qr_entry(rrf_handle_t h, int32_t dtype, int64_t rows, 
   if (!b_ok(dtype, b) || rows < b || rows > 0x7fffffffLL || ldy < b || ldv < b || ldt < b || ldy > 0x7fffffffLL)
     return RRF_ERR_INVALID_ARG;
   if (tree && b > kTsqrMaxB) return RRF_ERR_INVALID_ARG;
-  if (workspace_bytes < panel_scratch_bytes(kMaxSms, b, rows)) return RRF_ERR_WORKSPACE;
+  if (workspace_bytes < panel_scratch_bytes(kMaxSms, b, rows) || (reinterpret_cast<uintptr_t>(d_workspace) & 7u))
+    return RRF_ERR_WORKSPACE;
   cudaStream_t st = (cudaStream_t)cuda_stream;
   PanelScratch ps = carve_panel((unsigned char*)d_workspace, h->sms, b);
+  if (!aligned16(d_workspace)) ps.bk.Lw = nullptr;     // the flagged words of the blocked kernel are pairs of 8 bytes
   if (cudaMemsetAsync(ps.bar, 0, sizeof(unsigned), st) != cudaSuccess) return RRF_ERR_CUDA;
   if (cudaMemsetAsync(ps.blk_tags, 0, ps.blk_tag_bytes, st) != cudaSuccess) return RRF_ERR_CUDA;
   PanelSource src{};

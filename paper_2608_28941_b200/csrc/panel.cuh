@@ -945,8 +945,11 @@ __global__ void __launch_bounds__(kPanelThreads)
 #pragma unroll
   for (int i = 0; i < 2; ++i) {
     const int col = (np * 2 + i) * 8 + 2 * t, row = mt * 16 + g;
-    *reinterpret_cast<double2*>(gp + row * kHalf + col) = make_double2(acc[i][0], acc[i][1]);
-    *reinterpret_cast<double2*>(gp + (row + 8) * kHalf + col) = make_double2(acc[i][2], acc[i][3]);
+    // one by one: a caller's workspace need not start on 16 bytes
+    gp[row * kHalf + col] = acc[i][0];
+    gp[row * kHalf + col + 1] = acc[i][1];
+    gp[(row + 8) * kHalf + col] = acc[i][2];
+    gp[(row + 8) * kHalf + col + 1] = acc[i][3];
   }
 }
 // entry e of the sum over the parts, in a fixed order: four threads an entry

@@ -4,6 +4,8 @@ The factors are held to the oracle's within c u cond, the first-order perturbati
 unit round-off, cond the condition number of the panel with its columns scaled to unit length, which is what both
 factorisations see; c = 100 covers the sums over b columns).
 """
+import ctypes as C
+
 import numpy as np
 import pytest
 import torch
@@ -127,3 +129,45 @@ def test_repeats_itself(h, b, rows, kind):
     for _ in range(200):
         v, t = rrf.rrf_panel_qr(h, Y)
         assert torch.equal(v, V) and torch.equal(t, T)
+
+
+def panel_at(h, Y, offset, fn="rrf_panel_qr"):
+    """The call with a workspace that starts `offset` bytes past a 256-byte boundary: status, V, T."""
+    lib, (rows, b) = rrf.load(), Y.shape
+    dt = rrf.RRF_F64 if Y.dtype == torch.float64 else rrf.RRF_F32
+    need = C.c_size_t()
+    assert lib.rrf_panel_workspace_bytes(dt, rows, b, C.byref(need)) == rrf.RRF_OK
+    ws = torch.empty(need.value + 256, dtype=torch.uint8, device="cuda")
+    at = -ws.data_ptr() % 256 + offset
+    V, T = torch.empty_like(Y), torch.empty((b, b), dtype=Y.dtype, device="cuda")
+    s = getattr(lib, fn)(h, dt, rows, b, C.c_void_p(Y.data_ptr()), b, C.c_void_p(V.data_ptr()), b, C.c_void_p(T.data_ptr()), b,
+                         C.c_void_p(ws.data_ptr() + at), need.value, None)
+    torch.cuda.synchronize()
+    assert rrf.rrf_last_status(h) == rrf.RRF_OK
+    return s, V, T
+
+
+@pytest.mark.parametrize("dtype", [torch.float64, torch.float32])
+@pytest.mark.parametrize("rows,b", [(200, 32), (3000, 64), (9000, 64), (128, 128), (1500, 128), (30000, 128)])
+def test_workspace_on_8_bytes(h, rows, b, dtype):
+    """The same bits wherever the workspace starts, as long as a double can be stored there."""
+    Y = torch.from_numpy(panel("gauss", rows, b, np.random.default_rng(rows))).cuda().to(dtype)
+    want = panel_at(h, Y, 0)
+    for offset in (8, 16, 120):
+        got = panel_at(h, Y, offset)
+        assert got[0] == want[0] == rrf.RRF_OK
+        assert torch.equal(got[1], want[1]) and torch.equal(got[2], want[2])
+    assert panel_at(h, Y, 4)[0] == rrf.RRF_ERR_WORKSPACE
+
+
+def test_blocked_kernel_needs_a_workspace_on_16_bytes(h):
+    """On 8 bytes the column loop takes its place; a panel too tall for that is refused."""
+    Y = torch.from_numpy(panel("gauss", 2000, 64, np.random.default_rng(8))).cuda()
+    for offset in (0, 8):
+        s, V, T = panel_at(h, Y, offset, "rrf_panel_qr_blocked")
+        assert s == rrf.RRF_OK
+        Vo, _, To, _ = orc.panel_qr(Y.cpu().numpy())
+        assert np.max(np.abs(V.cpu().numpy() - Vo)) <= 1e-12 and np.max(np.abs(T.cpu().numpy() - To)) <= 1e-12
+    Y = torch.from_numpy(panel("gauss", 48000, 64, np.random.default_rng(9))).cuda()
+    assert panel_at(h, Y, 0)[0] == rrf.RRF_OK
+    assert panel_at(h, Y, 8)[0] == rrf.RRF_ERR_WORKSPACE
