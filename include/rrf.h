@@ -425,8 +425,8 @@ rrf_status_t rrf_selftest_timeout(rrf_handle_t h, double limit_ms, void* cuda_st
 /*
  * rrf_selftest_arithmetic - the arithmetic that the kernels do in the library's own way, element by element over n
  * values, for tests (no counterpart in the paper).  Does not synchronise the stream.
- *   which 0  d_x, d_first, d_second are floats: x split into two TF32 numbers, first + second = x up to 2^-22 |x|;
- *            a NaN or infinity in x is a NaN in `second`
+ *   which 0  d_x, d_first, d_second are floats: x split into two TF32 numbers (of `second` the 13 low bits do not count),
+ *            first + second = x up to 2^-22 |x|; a NaN or infinity in x is a NaN in `second`
  */
 rrf_status_t rrf_selftest_arithmetic(rrf_handle_t h, int32_t which, int64_t n, const void* d_x, void* d_first,
                                      void* d_second, void* cuda_stream);

@@ -130,6 +130,7 @@ def test_the_split_rounds_to_nearest(h):
     x = bits.view(np.float32)
     x = x[np.isfinite(x) & (np.abs(x) < np.float32(2.0) ** 127 * np.float32(2 - 2.0 ** -11))]
     hi, lo = (t.cpu().numpy() for t in rrf.rrf_selftest_arithmetic(h, 0, torch.from_numpy(x).cuda()))
+    lo = (lo.view(np.uint32) & np.uint32(0xffffe000)).view(np.float32)         # what the tensor core reads of it
 
     def tf32(v):                                             # float32 values, in float64
         v = v.astype(np.float64)
