@@ -192,7 +192,7 @@ __device__ __noinline__ bool cqr_chol(double* __restrict__ M, double* __restrict
   if (tid == 0) chol_bad = 0;
   if (tid < B) {
     const double v = M[cqr_blk(tid >> 3, tid >> 3) + (tid & 7) * 9];
-    gd[tid] = (v > 1e-280 && v < 1e280) ? v : __longlong_as_double(0x7ff0000000000000LL);   // fails the pivot test
+    gd[tid] = (v > 1e-280 && v < 1e280) ? v : __longlong_as_double(0x7ff8000000000000LL);   // NaN: fails any pivot test
   }
   __syncthreads();
 #pragma unroll 1

@@ -119,6 +119,24 @@ def test_squares_that_overflow(h):
     check(h, panel("gauss", 900, 32, np.random.default_rng(2)), "f64")
 
 
+@pytest.mark.parametrize("value", [1e160, np.inf, np.nan])
+@pytest.mark.parametrize("rows,b", [(700, 16), (900, 32), (6000, 64)])
+def test_last_column_overflows(h, rows, b, value):
+    """Its sum of squares is not finite while its products with the others may be: the columns before it are what they are
+    without it."""
+    Y = panel("gauss", rows, b, np.random.default_rng(rows))
+    if value == 1e160:
+        Y[:, -1] *= value
+    else:
+        Y[rows - 2, -1] = value
+    V, T = (t.cpu().numpy() for t in rrf.rrf_panel_qr(h, torch.from_numpy(Y).cuda()))
+    assert rrf.rrf_last_status(h) == rrf.RRF_OK
+    Vo, _, To, _ = orc.panel_qr(Y[:, :-1])
+    cond = np.linalg.cond(Y[:, :-1])
+    assert np.max(np.abs(V[:, :-1] - Vo)) <= 100.0 * 1.1e-16 * cond
+    assert np.max(np.abs(T[:-1, :-1] - To)) <= 1000.0 * 1.1e-16 * cond * np.max(np.abs(To))
+
+
 @pytest.mark.parametrize("b", [16, 32, 64])
 @pytest.mark.parametrize("rows", [700, 6000])
 @pytest.mark.parametrize("kind", ["gauss", "cond6"])
