@@ -180,16 +180,20 @@ static UpdPlan plan_upd(int sms, long long rows, long long ncols, int bm, int bn
 constexpr int kPanelVariants = 6;
 static const int kVariantRows[kPanelVariants] = {64, 128, 224, 320, 512, 224};
 static const bool kVariantPad[kPanelVariants] = {true, true, true, true, true, false};
-template <typename T>
-static const void* panel_variant(int q) {
+template <typename T, bool CQR>
+static const void* panel_variant_of(int q) {
   switch (q) {
-    case 0: return (const void*)panel_kernel<T, 2, 1>;
-    case 1: return (const void*)panel_kernel<T, 4, 1>;
-    case 2: return (const void*)panel_kernel<T, 7, 1>;
-    case 3: return (const void*)panel_kernel<T, 5, 2>;
-    case 4: return (const void*)panel_kernel<T, 8, 2>;
-    default: return (const void*)panel_kernel<T, 7, 1, false>;
+    case 0: return (const void*)panel_kernel<T, 2, 1, true, false, false, CQR>;
+    case 1: return (const void*)panel_kernel<T, 4, 1, true, false, false, CQR>;
+    case 2: return (const void*)panel_kernel<T, 7, 1, true, false, false, CQR>;
+    case 3: return (const void*)panel_kernel<T, 5, 2, true, false, false, CQR>;
+    case 4: return (const void*)panel_kernel<T, 8, 2, true, false, false, CQR>;
+    default: return (const void*)panel_kernel<T, 7, 1, false, false, false, false>;
   }
+}
+template <typename T>
+static const void* panel_variant(int q, bool cqr) {
+  return cqr ? panel_variant_of<T, true>(q) : panel_variant_of<T, false>(q);
 }
 template <typename T>
 static const void* panel_variant_cl(int q) {     // the same shapes as one thread-block cluster (padded ones only)
@@ -205,8 +209,8 @@ static const void* panel_variant_cl(int q) {     // the same shapes as one threa
 constexpr int kPanelVariantsCl = 6;
 constexpr int kPanelVariantReg = 5;
 constexpr int kClusterMaxRows = 128;
-// Padded slabs have a pitch of 4 mod 16 doubles: the fragment loads of the matrix products (eight columns x four rows)
-// hit every bank pair once.
+// Slabs for the Cholesky QR have a pitch of 4 mod 16 doubles: the fragment loads of the matrix products (eight columns x
+// four rows) hit every bank pair once.  For the column loop alone it is odd: a row read across the columns does.
 constexpr int kPanelPitch = 4;
 struct PanelPlan { int G, R, Rp, variant; size_t smem; bool cl; };
 // ctas == 0: the panel is spread over every SM (short slabs, short passes).  ctas > 0: the panel is
@@ -229,7 +233,7 @@ static bool plan_panel_cl(const rrf_ctx* h, long long rows, int b, PanelPlan* p,
   int G = 1;
   while (G < ceil_div(ext, R)) G *= 2;
   if (G > kClusterMax) return false;
-  const size_t extra = (size_t)panel_extra_doubles(b) + panel_work_doubles(b, fix) + panel_cluster_doubles(b);
+  const size_t extra = (size_t)panel_extra_doubles(b) + panel_work_doubles(b, fix, reg) + panel_cluster_doubles(b);
   if (reg) {
     p->R = R;
     p->G = G;
@@ -251,7 +255,8 @@ static bool plan_panel_cl(const rrf_ctx* h, long long rows, int b, PanelPlan* p,
   }
   return false;
 }
-static bool plan_panel(const rrf_ctx* h, long long rows, int b, PanelPlan* p, int ctas = 0, bool fix = false) {
+// `cqr`: for the kernels that try the Cholesky QR
+static bool plan_panel(const rrf_ctx* h, long long rows, int b, PanelPlan* p, int ctas, bool fix, bool cqr) {
   p->cl = false;
   if (fix && b > 64) return false;
   const long long ext = rows + (fix ? b : 0);
@@ -260,11 +265,11 @@ static bool plan_panel(const rrf_ctx* h, long long rows, int b, PanelPlan* p, in
   p->R = R;
   p->G = ceil_div(ext, R);
   if (p->G > h->sms) return false;
-  const size_t extra = (size_t)panel_extra_doubles(b) + panel_work_doubles(b, fix) + cqr_dinv_doubles(b);
+  const size_t extra = (size_t)panel_extra_doubles(b) + panel_work_doubles(b, fix, cqr) + (cqr ? cqr_dinv_doubles(b) : 0);
   for (int q = 0; q < kPanelVariants; ++q) {
     if (R > kVariantRows[q]) continue;
     if (kVariantPad[q]) {
-      p->Rp = kVariantRows[q] + kPanelPitch;
+      p->Rp = kVariantRows[q] + (cqr ? kPanelPitch : 1);
     } else {
       if (fix) continue;
       p->Rp = ((size_t)b * (R | 1) + extra) * sizeof(double) <= (size_t)h->panel_smem_max ? (R | 1) : R;
@@ -385,7 +390,7 @@ static bool plan_blk(const rrf_ctx* h, long long rows, int b, BlkPlan* p, int ct
 // Fewest CTAs whose shared memory holds a rows x b panel with the fix-up staging; 0 if none.
 static int panel_min_ctas(const rrf_ctx* h, long long rows, int b) {
   if (b > 64) return 0;
-  const size_t extra = (size_t)panel_extra_doubles(b) + panel_work_doubles(b, true) + cqr_dinv_doubles(b);
+  const size_t extra = (size_t)panel_extra_doubles(b) + panel_work_doubles(b, true, true) + cqr_dinv_doubles(b);
   int best = 0;
   for (int q = 0; q < kPanelVariants; ++q)
     if (kVariantPad[q] && ((size_t)b * (kVariantRows[q] + kPanelPitch) + extra) * sizeof(double) <= (size_t)h->panel_smem_max)
@@ -818,7 +823,7 @@ static rrf_status_t launch_panel(rrf_ctx* h, int dtype, const void* Y, PanelSour
   BlkPlan bp;
   // a panel too tall for shared memory goes to the blocked kernel with its slabs in global memory
   PanelPlan pp_probe;
-  const bool too_tall = ps.bk.Lw != nullptr && !plan_panel(h, rows, b, &pp_probe, o.ctas, o.fix.enabled != 0) &&
+  const bool too_tall = ps.bk.Lw != nullptr && !plan_panel(h, rows, b, &pp_probe, o.ctas, o.fix.enabled != 0, cqr != nullptr) &&
                         !(o.fix.enabled && b > 64);
   const bool want_global = o.global_slab || too_tall;
   if ((o.blocked || too_tall) && ps.bk.Lw != nullptr &&
@@ -844,7 +849,7 @@ static rrf_status_t launch_panel(rrf_ctx* h, int dtype, const void* Y, PanelSour
     // 16 SMs are then bound by their matrix products)
     const bool spread = o.ctas == 0 && b == 64 && rows > 2048;
     const bool as_cluster = !o.no_cluster && !spread && !o.blocked && plan_panel_cl(h, rows, b, &pp, o.fix.enabled != 0);
-    if (!as_cluster && !plan_panel(h, rows, b, &pp, o.ctas, o.fix.enabled != 0)) return RRF_ERR_WORKSPACE;
+    if (!as_cluster && !plan_panel(h, rows, b, &pp, o.ctas, o.fix.enabled != 0, cqr != nullptr)) return RRF_ERR_WORKSPACE;
     int R = pp.R, Rp = pp.Rp;
     void* args[] = {&Y,   &src, &alt, &fused_flag, &rows_i, &b,    &R,    &Rp,        &V,   &ldv,      &P,
                     &piv, &gram, &tau, &bar,       &ctrl,   &done_flag, &fix, &bar_base, &Tmerged, &ldt, &csq, &cqr};
@@ -868,7 +873,7 @@ static rrf_status_t launch_panel(rrf_ctx* h, int dtype, const void* Y, PanelSour
       cfg.numAttrs = 1;
       e = cudaLaunchKernelExC(&cfg, fn, args);
     } else {
-      const void* fn = dtype == RRF_F64 ? panel_variant<double>(pp.variant) : panel_variant<float>(pp.variant);
+      const void* fn = dtype == RRF_F64 ? panel_variant<double>(pp.variant, cqr != nullptr) : panel_variant<float>(pp.variant, cqr != nullptr);
       e = cudaLaunchCooperativeKernel(fn, dim3(pp.G), dim3(kPanelThreads), args, pp.smem, st);
     }
   }
@@ -899,14 +904,16 @@ static rrf_status_t launch_panel(rrf_ctx* h, int dtype, const void* Y, PanelSour
 // attributes of the panel and T-factor kernels; reports the dynamic shared memory a panel may use
 static cudaError_t setup_panel_kernels(int smem_optin, int* panel_smem_max, int* cluster_ok) {
   cudaError_t e;
-  const void* pk[2 * kPanelVariants + 2 * kPanelVariantsCl];
-  for (int q = 0; q < kPanelVariants; ++q) {
-    pk[q] = panel_variant<double>(q);
-    pk[kPanelVariants + q] = panel_variant<float>(q);
-  }
+  const void* pk[4 * kPanelVariants + 2 * kPanelVariantsCl];
+  const void** const pcl = pk + 4 * kPanelVariants;
+  for (int q = 0; q < kPanelVariants; ++q)
+    for (int c = 0; c < 2; ++c) {
+      pk[2 * q + c] = panel_variant<double>(q, c != 0);
+      pk[2 * kPanelVariants + 2 * q + c] = panel_variant<float>(q, c != 0);
+    }
   for (int q = 0; q < kPanelVariantsCl; ++q) {
-    pk[2 * kPanelVariants + q] = panel_variant_cl<double>(q);
-    pk[2 * kPanelVariants + kPanelVariantsCl + q] = panel_variant_cl<float>(q);
+    pcl[q] = panel_variant_cl<double>(q);
+    pcl[kPanelVariantsCl + q] = panel_variant_cl<float>(q);
   }
   size_t stat = 0;
   for (const void* f : pk) {
@@ -923,7 +930,7 @@ static cudaError_t setup_panel_kernels(int smem_optin, int* panel_smem_max, int*
   // clusters of up to kClusterMax CTAs (above the portable 8): allowed per kernel, and checked once for residency
   *cluster_ok = 1;
   for (int q = 0; q < 2 * kPanelVariantsCl; ++q) {
-    if (cudaFuncSetAttribute(pk[2 * kPanelVariants + q], cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
+    if (cudaFuncSetAttribute(pcl[q], cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
       cudaGetLastError();
       *cluster_ok = 0;
     }
@@ -941,7 +948,7 @@ static cudaError_t setup_panel_kernels(int smem_optin, int* panel_smem_max, int*
     cfg.attrs = at;
     cfg.numAttrs = 1;
     int nclusters = 0;
-    if (cudaOccupancyMaxActiveClusters(&nclusters, pk[2 * kPanelVariants + kPanelVariantsCl - 1], &cfg) != cudaSuccess || nclusters < 1) {
+    if (cudaOccupancyMaxActiveClusters(&nclusters, pcl[kPanelVariantsCl - 1], &cfg) != cudaSuccess || nclusters < 1) {
       cudaGetLastError();
       *cluster_ok = 0;
     }
@@ -1661,7 +1668,7 @@ rrf_status_t rrf_run(rrf_handle_t h, const rrf_params_t* p, void* dA, int64_t ld
       if (p->tune_panel_ctas > 0) best = std::min(cap, std::max(fewest, (int)p->tune_panel_ctas));
       PanelPlan ppl;
       const bool wanted = (p->flags & RRF_FLAG_TWO_QUEUES) || best_t < pm.step_serial();
-      if (wanted && plan_panel(h, m, b, &ppl, best, true)) look_ctas = best;
+      if (wanted && plan_panel(h, m, b, &ppl, best, true, true)) look_ctas = best;
     }
   }
   // (a panel too tall for shared memory is factored by the blocked kernel with its slabs in global memory)
@@ -2452,7 +2459,7 @@ extern "C" rrf_status_t rrf_panel_qr_static(int32_t dtype, int64_t rows, int32_t
   tmp.sms = sd->sms;
   tmp.panel_smem_max = sd->panel_smem_max;
   PanelPlan pp;
-  if (!plan_panel(&tmp, rows, b, &pp)) return RRF_ERR_WORKSPACE;   // panel too tall for on-chip storage
+  if (!plan_panel(&tmp, rows, b, &pp, 0, false, false)) return RRF_ERR_WORKSPACE;   // panel too tall for on-chip storage
   cudaStream_t st = (cudaStream_t)cuda_stream;
   Ctrl* ctrl = reinterpret_cast<Ctrl*>(sd->ptr);
   PanelScratch ps = carve_panel(sd->ptr + kStaticCtrlBytes, sd->sms, b, false);

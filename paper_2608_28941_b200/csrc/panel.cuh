@@ -17,7 +17,7 @@ __global__ void __launch_bounds__(256) split_selftest_kernel(long long n, const 
 
 // ------------------------------------------------------------------------------------------
 // Householder QR of a rows x b panel.  Each CTA keeps a slab of R consecutive rows in shared
-// memory (column-major, double precision, pitch Rp odd) for the whole factorisation.  Column j
+// memory (column-major, double precision, pitch Rp) for the whole factorisation.  Column j
 // costs one pass over the slab and ONE grid barrier: the pass applies the pending reflector
 // H_{j-1} and accumulates p[c] = sum_{row > j} Y[row, j] * X[row, c] for every column c, where
 // X[:, c] is the finished vector v_c for c < j and the current Y[:, c] for c >= j.  After the
@@ -64,8 +64,9 @@ constexpr int kFixChunk = 32;   // rows of Vp staged in shared memory at a time
 __host__ __device__ constexpr int panel_fix_doubles(int b) { return kFixChunk * (b + 8) + b * (b + 8); }
 
 // doubles of that staging area, which the Cholesky QR uses after it
-__host__ __device__ constexpr int panel_work_doubles(int b, bool fix) {
-  return fix && panel_fix_doubles(b) > cqr_work_doubles(b) ? panel_fix_doubles(b) : cqr_work_doubles(b);
+__host__ __device__ constexpr int panel_work_doubles(int b, bool fix, bool cqr) {
+  const int f = fix ? panel_fix_doubles(b) : 0, c = cqr ? cqr_work_doubles(b) : 0;
+  return f > c ? f : c;
 }
 
 template <typename T>
@@ -261,7 +262,10 @@ __device__ __forceinline__ void tfactor_block(const double* __restrict__ gram, c
 // multiply-adds and a warp reduction instead of a pass over the slab in shared memory (which is what makes a slab
 // of 256 rows, i.e. a 4096-row panel on 16 CTAs, worth its while).  Column j and the finished v_{j-1} go round
 // through two 256-element arrays in shared memory.
-template <typename T, int QMAX, int RH, bool PAD = true, bool CL = false, bool REG = false>
+// CQR: the Cholesky QR is tried first.  Panels that never take it (128 columns, square ones, those of the entry point
+// without a workspace) have kernels without: beside the call the column loop spills, 0.2 us a column (8192 x 64 without a
+// workspace 299 -> 286 us, 8192 x 128 f32 761 -> 744).
+template <typename T, int QMAX, int RH, bool PAD = true, bool CL = false, bool REG = false, bool CQR = true>
 __global__ void __launch_bounds__(kPanelThreads)
     panel_kernel(const T* __restrict__ Y, PanelSource src_fused, PanelSource src_alt, const int* __restrict__ fused_flag,
                  int rows, int b, int R, int Rp,
@@ -309,9 +313,10 @@ __global__ void __launch_bounds__(kPanelThreads)
   double* p_s = w_s + b;                  // [2][b]: per row group, then (first b) the grid-wide sums
   double* pr_s = p_s + 2 * b;             // [b]
   double* sc_s = pr_s + b;                // [4]: tau_j, 1/(alpha - beta)
+  constexpr bool kTryCqr = CQR && PAD && (!CL || REG);
   // cluster mode: partial sums [2][kClusterMax][b] and pivot rows [2][b] written by the peers, behind everything else
   double* work_s = sc_s + 4;              // staging of the fix-up, then the small matrices of the Cholesky QR
-  double* px_s = work_s + panel_work_doubles(b, fix.enabled);
+  double* px_s = work_s + panel_work_doubles(b, fix.enabled, kTryCqr);
   double* prx_s = px_s + 2 * kClusterMax * 2 * b;
   double* ycol_s = prx_s + 2 * b;         // [kRegRows] column j below its pivot (register-resident loop)
   double* vcol_s = ycol_s + kRegRows;     // [kRegRows] v_{j-1}
@@ -513,9 +518,9 @@ __global__ void __launch_bounds__(kPanelThreads)
   if (csq != nullptr && !fix.csq_before) column_squares(row0);
 
   // Cholesky QR with reconstruction where it is safe; the column loop below does the rest
-  const bool try_cqr = PAD && (!CL || REG) && cqr != nullptr && b <= 64 && rows > b;
+  const bool try_cqr = kTryCqr && cqr != nullptr && b <= 64 && rows > b;
   bool have_v = false;
-  if constexpr (PAD && (!CL || REG)) {
+  if constexpr (kTryCqr) {
     if (try_cqr) {
       __shared__ CqrArgs ca;
       if (tid == 0) {
