@@ -427,6 +427,8 @@ rrf_status_t rrf_selftest_timeout(rrf_handle_t h, double limit_ms, void* cuda_st
  * values, for tests (no counterpart in the paper).  Does not synchronise the stream.
  *   which 0  d_x, d_first, d_second are floats: x split into two TF32 numbers (of `second` the 13 low bits do not count),
  *            first + second = x up to 2^-22 |x|; a NaN or infinity in x is a NaN in `second`
+ *   which 1  doubles: first = 1 / x and second = 1 / sqrt(x) as the b x b factorisations of the panel form them, for x from
+ *            1e-300 to 1e300
  */
 rrf_status_t rrf_selftest_arithmetic(rrf_handle_t h, int32_t which, int64_t n, const void* d_x, void* d_first,
                                      void* d_second, void* cuda_stream);

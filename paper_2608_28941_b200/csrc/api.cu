@@ -1233,11 +1233,14 @@ rrf_status_t rrf_selftest_timeout(rrf_handle_t h, double limit_ms, void* cuda_st
 
 rrf_status_t rrf_selftest_arithmetic(rrf_handle_t h, int32_t which, int64_t n, const void* d_x, void* d_first,
                                      void* d_second, void* cuda_stream) {
-  if (h == nullptr || which != 0 || n < 1 || d_x == nullptr || d_first == nullptr || d_second == nullptr)
+  if (h == nullptr || which < 0 || which > 1 || n < 1 || d_x == nullptr || d_first == nullptr || d_second == nullptr)
     return RRF_ERR_INVALID_ARG;
   cudaStream_t st = (cudaStream_t)cuda_stream;
   const int grid = (int)std::min<long long>((n + 255) / 256, (long long)h->sms * 8);
-  split_selftest_kernel<<<grid, 256, 0, st>>>(n, (const float*)d_x, (float*)d_first, (float*)d_second);
+  if (which == 0)
+    split_selftest_kernel<<<grid, 256, 0, st>>>(n, (const float*)d_x, (float*)d_first, (float*)d_second);
+  else
+    recip_selftest_kernel<<<grid, 256, 0, st>>>(n, (const double*)d_x, (double*)d_first, (double*)d_second);
   return cudaGetLastError() == cudaSuccess ? RRF_OK : RRF_ERR_CUDA;
 }
 

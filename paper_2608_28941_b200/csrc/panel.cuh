@@ -14,6 +14,12 @@ __global__ void __launch_bounds__(32) timeout_selftest_kernel(unsigned* ctr, Ctr
 __global__ void __launch_bounds__(256) split_selftest_kernel(long long n, const float* __restrict__ x, float* __restrict__ hi, float* __restrict__ lo) {
   for (long long i = blockIdx.x * 256LL + threadIdx.x; i < n; i += gridDim.x * 256LL) split_tf32(x[i], hi[i], lo[i]);
 }
+__global__ void __launch_bounds__(256) recip_selftest_kernel(long long n, const double* __restrict__ x, double* __restrict__ rcp, double* __restrict__ rsq) {
+  for (long long i = blockIdx.x * 256LL + threadIdx.x; i < n; i += gridDim.x * 256LL) {
+    rcp[i] = cqr_rcp(x[i]);
+    rsq[i] = cqr_rsqrt(x[i]);
+  }
+}
 
 // ------------------------------------------------------------------------------------------
 // Householder QR of a rows x b panel.  Each CTA keeps a slab of R consecutive rows in shared

@@ -189,3 +189,21 @@ def test_blocked_kernel_needs_a_workspace_on_16_bytes(h):
     Y = torch.from_numpy(panel("gauss", 48000, 64, np.random.default_rng(9))).cuda()
     assert panel_at(h, Y, 0)[0] == rrf.RRF_OK
     assert panel_at(h, Y, 8)[0] == rrf.RRF_ERR_WORKSPACE
+
+
+def test_reciprocals(h):
+    """The factorisations' own 1/x and 1/sqrt(x) over the exponents that their pivots can have (a pivot is at least 1e-11 of
+    a diagonal entry between 1e-280 and 1e280): the third-order step leaves the approximation's error cubed, 2^-60, and two
+    roundings of its own, so 1/x is within one and 1/sqrt(x) within two units in the last place of the rounded quotient."""
+    rng = np.random.default_rng(0)
+    n = 1 << 20
+    x = np.ldexp(1.0 + rng.random(n), rng.integers(-968, 931, n))
+    edge = np.ldexp(1.0, np.arange(-968, 931)).astype(np.float64)
+    x = np.concatenate([x, edge, np.nextafter(edge, 0.0), np.nextafter(edge, np.inf), 1.0 + np.arange(1, 4097) / 4096.0])
+    rcp, rsq = (t.cpu().numpy() for t in rrf.rrf_selftest_arithmetic(h, 1, torch.from_numpy(x).cuda()))
+    exact = np.longdouble(1.0) / x.astype(np.longdouble)
+    ulp = np.spacing(exact.astype(np.float64)).astype(np.longdouble)
+    assert np.max(np.abs(rcp - exact) / ulp) <= 1.0
+    exact = np.longdouble(1.0) / np.sqrt(x.astype(np.longdouble))
+    ulp = np.spacing(exact.astype(np.float64)).astype(np.longdouble)
+    assert np.max(np.abs(rsq - exact) / ulp) <= 2.0
