@@ -433,6 +433,21 @@ rrf_status_t rrf_selftest_timeout(rrf_handle_t h, double limit_ms, void* cuda_st
 rrf_status_t rrf_selftest_arithmetic(rrf_handle_t h, int32_t which, int64_t n, const void* d_x, void* d_first,
                                      void* d_second, void* cuda_stream);
 
+/*
+ * rrf_panel_path - how the last rrf_panel_qr on this handle that used the column kernels was factored, for tests (no
+ * counterpart in the paper); for 128 columns in double precision, the second half.  Synchronises `cuda_stream`.
+ */
+enum {
+  RRF_PATH_NONE = 0,          /* no such call yet */
+  RRF_PATH_LOOP = 1,          /* the column loop, without trying the Cholesky QR */
+  RRF_PATH_FIRST_ORDER = 2,   /* Cholesky QR, the second factor to first order */
+  RRF_PATH_CHOLESKY = 3,      /* Cholesky QR, the second factor by a factorisation */
+  RRF_PATH_LOOP_Y = 4,        /* the column loop on the panel: a pivot of the first factor was too small */
+  RRF_PATH_LOOP_Q1 = 5        /* the column loop on the panel made orthonormal: G1 too far from the identity, or a column
+                                 with nothing below its pivot */
+};
+rrf_status_t rrf_panel_path(rrf_handle_t h, int32_t* path, void* cuda_stream);
+
 /* Status word of the handle's device side (set by bounded waits), read with one small
  * device-to-host copy after synchronising `cuda_stream`; clears it. */
 rrf_status_t rrf_last_status(rrf_handle_t h, void* cuda_stream);

@@ -1244,6 +1244,13 @@ rrf_status_t rrf_selftest_arithmetic(rrf_handle_t h, int32_t which, int64_t n, c
   return cudaGetLastError() == cudaSuccess ? RRF_OK : RRF_ERR_CUDA;
 }
 
+rrf_status_t rrf_panel_path(rrf_handle_t h, int32_t* path, void* cuda_stream) {
+  if (h == nullptr || path == nullptr) return RRF_ERR_INVALID_ARG;
+  cudaStream_t st = (cudaStream_t)cuda_stream;
+  if (cudaMemcpyAsync(path, &h->d_ctrl->panel_path, sizeof(int32_t), cudaMemcpyDeviceToHost, st) != cudaSuccess) return RRF_ERR_CUDA;
+  return cudaStreamSynchronize(st) == cudaSuccess ? RRF_OK : RRF_ERR_CUDA;
+}
+
 rrf_status_t rrf_workspace_bytes(const rrf_params_t* p, size_t* bytes) {
   if (bytes == nullptr) return RRF_ERR_INVALID_ARG;
   const rrf_status_t s = check_params(p);

@@ -18,7 +18,8 @@ struct Ctrl {
   int steps;       // block steps completed (the paper's i)
   int k;           // steps * b
   unsigned bar;    // arrival counter of the panel kernel's grid barrier
-  int pad[3];
+  int panel_path;  // how the last panel of the column kernels was factored (rrf_panel_path)
+  int pad[2];
   double normA2;   // ||A||_F^2
   double sigma2;   // squared absolute tolerance
   double E_sub;    // Algorithm 2 line 9

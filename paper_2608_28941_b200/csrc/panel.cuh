@@ -549,11 +549,14 @@ __global__ void __launch_bounds__(kPanelThreads)
       __syncthreads();
       const int got = b == 64 ? cqr_panel<64, CL>(ca) : (b == 32 ? cqr_panel<32, CL>(ca) : cqr_panel<16, CL>(ca));
       if (got < 0) return;
-      have_v = got & 1;
-      if (CL) nx += (unsigned)got >> 1;
-      else nbar += (unsigned)got >> 1;
+      const int path = got & 7;
+      have_v = path <= RRF_PATH_CHOLESKY;
+      if (CL) nx += (unsigned)got >> 3;
+      else nbar += (unsigned)got >> 3;
+      if (cta == 0 && tid == 0) ctrl->panel_path = path;
     }
   }
+  if (!try_cqr && cta == 0 && tid == 0) ctrl->panel_path = RRF_PATH_LOOP;
 
   double tau_prev = 0.0;
   if (have_v) {

@@ -584,9 +584,9 @@ __device__ __forceinline__ void cqr_put(void* base, size_t at, double v0, double
 }
 
 // The whole of it, called by every thread of every CTA with the panel in the slabs; the arguments lie in shared memory
-// (on the stack they go through what is left of the L1: 4 us a call).  Negative: a wait gave up.  Else bit 0 says
-// whether V and T are written (if not, the column loop has to do it, on what the slabs hold) and the rest is the
-// number of barriers passed.
+// (on the stack they go through what is left of the L1: 4 us a call).  Negative: a wait gave up.  Else the low three
+// bits say what was done (RRF_PATH_*: V and T are written, or the column loop has to do it, on what the slabs hold) and
+// the rest is the number of barriers passed.
 template <int B, bool CL>
 __device__ __noinline__ int cqr_panel(const CqrArgs& a) {
   using C = Cqr<B>;
@@ -604,7 +604,7 @@ __device__ __noinline__ int cqr_panel(const CqrArgs& a) {
   __syncthreads();
   cqr_gram<B>(a.S, Rp, a.nloc, a.work, tid);
   if (!cqr_reduce<B, CL>(a, false, tid)) return -1;
-  if (!cqr_chol<B>(M, dinv_r, small, kCqrPivot, tid)) return 2 << 1;
+  if (!cqr_chol<B>(M, dinv_r, small, kCqrPivot, tid)) return 2 << 3 | RRF_PATH_LOOP_Y;
 
   const bool has00 = row0 >= a.gr0 && row0 < a.gr0 + a.nloc;
   const double y00 = has00 ? a.S[row0 - a.gr0] : 0.0;
@@ -671,9 +671,9 @@ __device__ __noinline__ int cqr_panel(const CqrArgs& a) {
     if (far) defect_s[1] = 1;
   }
   __syncthreads();
-  if (defect_s[1]) return 4 << 1;
+  if (defect_s[1]) return 4 << 3 | RRF_PATH_LOOP_Q1;
   if (defect_s[0]) {
-    if (!cqr_chol<B>(M, dinv_r, small, 0.25, tid)) return 4 << 1;
+    if (!cqr_chol<B>(M, dinv_r, small, 0.25, tid)) return 4 << 3 | RRF_PATH_LOOP_Q1;
   } else {
     if (tid < B) {
       double* d = M + cqr_blk(tid >> 3, tid >> 3) + (tid & 7) * 9;
@@ -683,7 +683,7 @@ __device__ __noinline__ int cqr_panel(const CqrArgs& a) {
   }
   double* sgn = small + 2 * B;
   double* rinv = small + 3 * B;
-  if (!cqr_lu<B>(A, M, sgn, rinv, tid)) return 4 << 1;
+  if (!cqr_lu<B>(A, M, sgn, rinv, tid)) return 4 << 3 | RRF_PATH_LOOP_Q1;
 
   // the inverted diagonal blocks the products below need: of U', and for T of R2 and V1^T (the latter in place of R2's
   // diagonal blocks, which nothing reads any more)
@@ -756,7 +756,7 @@ __device__ __noinline__ int cqr_panel(const CqrArgs& a) {
       }
     }
   }
-  return 4 << 1 | 1;
+  return 4 << 3 | (defect_s[0] ? RRF_PATH_CHOLESKY : RRF_PATH_FIRST_ORDER);
 }
 
 }  // namespace rrf

@@ -45,7 +45,7 @@ class rrf_profile_t(C.Structure):
     _fields_ = [("ms", C.c_double * 9), ("launches", C.c_int32 * 9), ("pad", C.c_int32)]
 
 
-EXPORTS = ["rrf_run_colmajor", "rrf_colmajor_workspace_bytes", "rrf_transpose", "rrf_set_single_engine", "rrf_sample_workspace_bytes", "rrf_sample_panel", "rrf_frobenius_sq", "rrf_panel_qr_blocked", "rrf_panel_qr_tree", "rrf_transfer_workspace_bytes", "rrf_subspace_transfer", "rrf_selftest_timeout", "rrf_selftest_arithmetic", "rrf_panel_qr_static", "rrf_set_profiling", "rrf_get_profile", "rrf_measure_peak", "rrf_create", "rrf_destroy", "rrf_workspace_bytes", "rrf_run", "rrf_panel_workspace_bytes",
+EXPORTS = ["rrf_run_colmajor", "rrf_colmajor_workspace_bytes", "rrf_transpose", "rrf_set_single_engine", "rrf_sample_workspace_bytes", "rrf_sample_panel", "rrf_frobenius_sq", "rrf_panel_qr_blocked", "rrf_panel_qr_tree", "rrf_transfer_workspace_bytes", "rrf_subspace_transfer", "rrf_selftest_timeout", "rrf_selftest_arithmetic", "rrf_panel_path", "rrf_panel_qr_static", "rrf_set_profiling", "rrf_get_profile", "rrf_measure_peak", "rrf_create", "rrf_destroy", "rrf_workspace_bytes", "rrf_run", "rrf_panel_workspace_bytes",
            "rrf_panel_qr", "rrf_apply_workspace_bytes", "rrf_apply_qt", "rrf_apply_q", "rrf_form_q",
            "rrf_fill_omega", "rrf_last_status", "rrf_status_string"]
 
@@ -87,6 +87,7 @@ def load():
                                           vp, i64, vp, sz, vp]
     lib.rrf_last_status.argtypes = [vp, vp]
     lib.rrf_selftest_timeout.argtypes = [vp, C.c_double, vp]
+    lib.rrf_panel_path.argtypes = [vp, C.POINTER(C.c_int32), vp]
     lib.rrf_selftest_arithmetic.argtypes = [vp, C.c_int32, C.c_int64, vp, vp, vp, vp]
     lib.rrf_set_single_engine.argtypes = [vp, i32, i32]
     lib.rrf_set_profiling.argtypes = [vp, i32]
@@ -482,3 +483,15 @@ def rrf_selftest_arithmetic(h, which: int, x: torch.Tensor):
     if s != RRF_OK:
         raise RrfError(s, "rrf_selftest_arithmetic")
     return first, second
+
+
+RRF_PATH_LOOP, RRF_PATH_FIRST_ORDER, RRF_PATH_CHOLESKY, RRF_PATH_LOOP_Y, RRF_PATH_LOOP_Q1 = 1, 2, 3, 4, 5
+
+
+def rrf_panel_path(h) -> int:
+    """How the last panel was factored (RRF_PATH_*, see rrf.h)."""
+    path = C.c_int32()
+    s = load().rrf_panel_path(h, C.byref(path), _stream())
+    if s != RRF_OK:
+        raise RrfError(s, "rrf_panel_path")
+    return path.value

@@ -37,6 +37,10 @@ def panel(kind, rows, b, rng):
     elif kind == "nothing-below":                  # column loop, on the orthonormal panel: tau = 0 in some columns
         Y[b:] = 0.0
         Y[:b] = np.triu(Y[:b]) + 3.0 * np.eye(b)
+    elif kind == "near":                           # second factor by a factorisation: two columns 1e-5 apart
+        Y[:, b // 2] = Y[:, 1] + 1e-5 * Y[:, b // 2]
+    elif kind == "nearer":                         # column loop: 1e-7 apart, a pivot of 1e-14
+        Y[:, b // 2] = Y[:, 1] + 1e-7 * Y[:, b // 2]
     elif kind == "huge":                           # column loop: squares overflow
         Y *= 1e160
     return Y
@@ -116,6 +120,7 @@ def test_squares_that_overflow(h):
     """The column loop's sums of squares overflow too; all that is asked is that the call ends and the context lives."""
     rrf.rrf_panel_qr(h, torch.from_numpy(panel("huge", 900, 32, np.random.default_rng(1))).cuda())
     torch.cuda.synchronize()
+    assert rrf.rrf_last_status(h) == rrf.RRF_OK and rrf.rrf_panel_path(h) == rrf.RRF_PATH_LOOP_Y
     check(h, panel("gauss", 900, 32, np.random.default_rng(2)), "f64")
 
 
@@ -207,3 +212,27 @@ def test_reciprocals(h):
     exact = np.longdouble(1.0) / np.sqrt(x.astype(np.longdouble))
     ulp = np.spacing(exact.astype(np.float64)).astype(np.longdouble)
     assert np.max(np.abs(rsq - exact) / ulp) <= 2.0
+
+
+@pytest.mark.parametrize("b", [16, 32, 64, 128])
+@pytest.mark.parametrize("rows", [700, 6000])      # one cluster, the whole grid; 128 columns: the second half of two
+@pytest.mark.parametrize("kind,path", [
+    ("gauss", rrf.RRF_PATH_FIRST_ORDER), ("graded", rrf.RRF_PATH_FIRST_ORDER), ("near", rrf.RRF_PATH_CHOLESKY),
+    ("nearer", rrf.RRF_PATH_LOOP_Y), ("dependent", rrf.RRF_PATH_LOOP_Y), ("zero", rrf.RRF_PATH_LOOP_Y),
+    ("huge", rrf.RRF_PATH_LOOP_Y), ("nothing-below", rrf.RRF_PATH_LOOP_Q1)])
+def test_path_taken(h, b, rows, kind, path):
+    """Which of its ways a panel goes."""
+    if b == 128:                     # the columns that decide belong to the second half
+        Y = np.concatenate([panel("gauss", rows, 64, np.random.default_rng(b)), panel(kind, rows, 64, np.random.default_rng(rows))], 1)
+        if kind == "nothing-below":
+            Y = panel(kind, rows, b, np.random.default_rng(rows))
+    else:
+        Y = panel(kind, rows, b, np.random.default_rng(rows + b))
+    rrf.rrf_panel_qr(h, torch.from_numpy(Y).cuda())
+    assert rrf.rrf_panel_path(h) == path
+
+
+def test_panels_that_do_not_try(h):
+    for rows, b, dtype in ((64, 64, torch.float64), (3000, 128, torch.float32), (30000, 128, torch.float32)):
+        rrf.rrf_panel_qr(h, torch.randn((rows, b), dtype=dtype, device="cuda"))
+        assert rrf.rrf_panel_path(h) == rrf.RRF_PATH_LOOP
