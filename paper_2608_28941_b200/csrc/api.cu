@@ -47,6 +47,7 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t,
 
 constexpr int kMaxSmem = 232448;   // 227 KB opt-in dynamic shared memory per CTA on sm_100
 constexpr int kMaxSms = kPanelMaxG;       // workspace sizes are bounds for devices with up to this many SMs
+constexpr int kB200Sms = 148;
 
 }  // namespace rrf
 
@@ -75,6 +76,7 @@ struct rrf_ctx {
   int graph_off;                         // set when a capture failed: enqueue directly from then on
   int cand_steps;                        // block steps the last directly enqueued call ran, -1 if it did not end by its own rule
   int gsteps;                            // block steps the instantiated graph holds (it may hold fewer than max_rank / b)
+  int gextra;                            // its kernels beyond those that every pass has (extra_launches in rrf_run)
   int cluster_ok;                        // a 16-CTA cluster of the panel kernel can be resident on this device
   int f32_engine;                        // single-precision V^T W: 0 = mma.sync 3xTF32, 1 = tcgen05 3xTF32
   int tc_chunk;                          // tcgen05: 64-row tiles summed in tensor memory between round-to-nearest adds
@@ -615,7 +617,7 @@ struct Ops {
                  const int* done_flag, TzSplit sp, bool dep, cudaStream_t st) {
     // half as many columns a CTA where that still is at most one CTA per SM: a column tile then has few CTAs and many
     // partial slots, and each thread has twice as many of them in flight
-    const bool narrow = vp.npad / (kTzCols / 2) <= 148;
+    const bool narrow = vp.npad / (kTzCols / 2) <= kB200Sms;
     sp.ntz = vp.npad / (narrow ? kTzCols / 2 : kTzCols);
     const int grid = sp.ntz + (sp.o != nullptr ? B : 0);      // one CTA per row of OmegaT
     if (narrow)
@@ -702,7 +704,7 @@ struct PanelOpts {
   const int* fused_flag = nullptr; // ... which is the case when this device word is 0 (NULL: always `src`)
   PanelFix fix{};                  // look-ahead fix-up (enabled == 0: none)
   int ctas = 0;                    // 0: one slab per SM; > 0: confine the panel to this many CTAs
-  unsigned* bar_reset = nullptr;   // the T-factor kernel zeroes this word (the panel's barrier counter)
+  int* launches = nullptr;         // out: the kernels of this panel are added to it
   bool merge_t = false;            // CTA 0 of the panel kernel builds T itself: no T-factor launch
   unsigned bar_base = 0;           // value of the barrier counter when this launch starts (it is not reset
                                    // between the launches of the look-ahead schedule)
@@ -748,6 +750,7 @@ static rrf_status_t launch_panel(rrf_ctx* h, int dtype, const void* Y, PanelSour
       return RRF_ERR_CUDA;
     }
     if (o.t_aside != nullptr) *o.t_aside = false;
+    if (o.launches != nullptr) *o.launches += 1;
     return RRF_OK;
   }
   if (dtype == RRF_F64 && b == 2 * kHalf && !o.blocked && !o.global_slab && ps.gslab != nullptr && !o.fix.enabled && rows <= (long long)h->sms * 320) {
@@ -799,6 +802,7 @@ static rrf_status_t launch_panel(rrf_ctx* h, int dtype, const void* Y, PanelSour
     corner_part_kernel<<<parts, kPanelThreads, 0, st>>>((const double*)V, ldv, (int)rows, per, gpart, done_flag);
     corner_sum_kernel<<<kHalf, 256, 0, st>>>(gpart, parts, gm, done_flag);
     corner_t_kernel<<<1, kPanelThreads, kCornerSmem, st>>>(gm, (double*)Tout, ldt, (double*)V, ldv, done_flag);
+    if (o.launches != nullptr) *o.launches += 3;      // and those of the halves, which have added themselves
     const cudaError_t ce = cudaGetLastError();
     if (ce != cudaSuccess) {
       h->last_cuda = (int)ce;
@@ -878,6 +882,7 @@ static rrf_status_t launch_panel(rrf_ctx* h, int dtype, const void* Y, PanelSour
     }
   }
   if (o.t_aside != nullptr) *o.t_aside = !merge_t;
+  if (o.launches != nullptr) *o.launches += merge_t ? 1 : 2;
   if (e == cudaSuccess && !merge_t) {
     cudaStream_t tt = st;
     if (o.ev_fork != nullptr) {          // fork: the T factor runs on the side stream after the panel
@@ -888,9 +893,9 @@ static rrf_status_t launch_panel(rrf_ctx* h, int dtype, const void* Y, PanelSour
       mark(RRF_PHASE_TFACTOR, step);
     }
     if (dtype == RRF_F64)
-      tfactor_kernel<double><<<1, 256, tsmem, tt>>>(gram, tau, b, (double*)Tout, ldt, done_flag, o.bar_reset);
+      tfactor_kernel<double><<<1, 256, tsmem, tt>>>(gram, tau, b, (double*)Tout, ldt, done_flag);
     else
-      tfactor_kernel<float><<<1, 256, tsmem, tt>>>(gram, tau, b, (float*)Tout, ldt, done_flag, o.bar_reset);
+      tfactor_kernel<float><<<1, 256, tsmem, tt>>>(gram, tau, b, (float*)Tout, ldt, done_flag);
     e = cudaGetLastError();
     if (o.ev_join != nullptr) cudaEventRecord(o.ev_join, o.st_t);
   }
@@ -1019,7 +1024,7 @@ struct RunLayout {
   int init_ctas, max_norm_parts;
   long long ldw;
 };
-constexpr int kInitCtas = 148 * 8;
+constexpr int kInitCtas = kB200Sms * 8;
 
 static bool run_layout(const rrf_params_t* p, bool need_omega, RunLayout* L) {
   const int sms = kMaxSms;
@@ -1117,6 +1122,7 @@ rrf_status_t rrf_create(rrf_handle_t* out, int device) {
   h->graph_off = 0;
   h->cand_steps = -1;
   h->gsteps = 0;
+  h->gextra = 0;
   h->f32_engine = 1;      // single precision runs on tcgen05 unless rrf_set_single_engine says otherwise
   h->tc_chunk = 2;
   std::memset(&h->profile, 0, sizeof(h->profile));
@@ -1729,10 +1735,12 @@ rrf_status_t rrf_run(rrf_handle_t h, const rrf_params_t* p, void* dA, int64_t ld
   const bool fixed = (p->flags & RRF_FLAG_FIXED_RANK) != 0;
   std::vector<std::pair<int, int>> marks;   // profiling: (phase, block step) of every recorded event
   size_t nev = 0;
+  int extra_launches = 0;                   // kernels whose number differs from pass to pass: panels, second launches of an update
   bool capturing = false;
   // Everything rrf_run puts on the device, on stream `st` (and the side stream, forked from and joined
   // back to it): enqueued directly, or recorded into a CUDA graph.
   auto enqueue = [&]() -> rrf_status_t {
+  extra_launches = 0;
   if (look_ctas > 0 && cudaMemsetAsync(look_bar, 0, sizeof(unsigned), st) != cudaSuccess) return RRF_ERR_CUDA;
   if (cudaMemsetAsync(ps.blk_tags, 0, ps.blk_tag_bytes, st) != cudaSuccess) return RRF_ERR_CUDA;   // exchange tags of the blocked panel kernel
   void* W = inplace ? dA : (void*)(ws + L.w);
@@ -1872,6 +1880,7 @@ rrf_status_t rrf_run(rrf_handle_t h, const rrf_params_t* p, void* dA, int64_t ld
       sd.ldy = b;
       sd.row_off = r0;
       PanelOpts po;
+      po.launches = &extra_launches;
       po.merge_t = true;
       po.blocked = blocked;
       po.seq_base = 256u * (unsigned)i;
@@ -1896,6 +1905,7 @@ rrf_status_t rrf_run(rrf_handle_t h, const rrf_params_t* p, void* dA, int64_t ld
     for (int i = 0; i < steps_run; ++i) {
       const int r0 = i * b, rows = (int)(m - r0);
       PanelOpts po;
+      po.launches = &extra_launches;
       po.st_t = h->aux;
       po.ev_fork = h->sync_events[2 * i];
       po.ev_join = h->sync_events[2 * i + 1];
@@ -1982,6 +1992,7 @@ rrf_status_t rrf_run(rrf_handle_t h, const rrf_params_t* p, void* dA, int64_t ld
     // run because the loop has ended adds nothing, and then no later panel runs either)
     unsigned bar_next = 0, bar_used = 0;
     PanelOpts po;
+    po.launches = &extra_launches;
     po.ctas = look_ctas;
     po.tree = tree;
     po.blocked = blocked;
@@ -2107,6 +2118,7 @@ rrf_status_t rrf_run(rrf_handle_t h, const rrf_params_t* p, void* dA, int64_t ld
         // behind the panel kernel of pass i+1 on the side stream (which has waited for T Z of this pass)
         ops->update(tmV_u, tmZ, i == 0 ? tmA_u : tmW_u, tmO, W, ldw, (char*)dB + (size_t)r0 * ldb * esize, ldb, r0, rows, (int)n,
                     r0, b, j0, Ybuf[i & 1], norm_part, uh, ctrl, samp + i, false, h->aux);
+        ++extra_launches;
         cudaEventRecord(evH(i), h->aux);
         cudaStreamWaitEvent(st, evH(i), 0);
         up.tpc = um.tpc;          // what the loader of the sampled panel needs to find the partial results
@@ -2166,6 +2178,7 @@ rrf_status_t rrf_run(rrf_handle_t h, const rrf_params_t* p, void* dA, int64_t ld
     marks = h->gmarks;
     nev = marks.size();
     steps_run = h->gsteps;
+    extra_launches = h->gextra;
     launched = cudaGraphLaunch(h->gexec, user_st) == cudaSuccess;
     if (!launched) h->graph_off = 1;
   } else if (graphs_ok && key == h->gcand) {
@@ -2188,6 +2201,7 @@ rrf_status_t rrf_run(rrf_handle_t h, const rrf_params_t* p, void* dA, int64_t ld
         h->gkey = key;
         h->gmarks = marks;
         h->gsteps = steps_run;
+        h->gextra = extra_launches;
         launched = cudaGraphLaunch(h->gexec, user_st) == cudaSuccess;
       } else if (g != nullptr) {
         cudaGraphDestroy(g);
@@ -2268,16 +2282,12 @@ rrf_status_t rrf_run(rrf_handle_t h, const rrf_params_t* p, void* dA, int64_t ld
     // without the predictor every executed pass that has a later panel to sample samples it
     out->fused_samples = predicting ? hc.fused_samples : std::min(hc.steps, std::max(0, steps - lag));
     const int sl = steps_run;      // passes whose kernels were launched
-    // panel: one kernel with T in it; two halves and the corner for b = 128; the T factor apart where neither applies
-    const bool two_halves = p->dtype == RRF_F64 && b == 2 * kHalf && !blocked && m <= (long long)h->sms * 320;
-    const bool t_apart = !two_halves && look_ctas == 0 && !tree && !unchanged && (b > 64 || blocked);
-    const int pl = two_halves ? 5 : (t_apart ? 2 : 1);
     const int first = 2 + (dOmegaT == nullptr ? 1 : 0);           // sample, loop state, the library's own vectors
     if (unchanged)
-      out->kernel_launches = first - 1 + (3 + pl) * sl + 3 * sl * (sl - 1) / 2;
+      out->kernel_launches = first - 1 + 3 * sl + 3 * sl * (sl - 1) / 2 + extra_launches;
     else
-      out->kernel_launches = first + ((look_ctas > 0 && steps > 1) ? 1 : 0) + (pl + 4 + (sampled ? 1 : 0)) * sl +
-                             (predicting ? std::max(0, std::min(sl, steps - lag)) : 0);
+      out->kernel_launches = first + ((look_ctas > 0 && steps > 1) ? 1 : 0) + (4 + (sampled ? 1 : 0)) * sl +
+                             (predicting ? std::max(0, std::min(sl, steps - lag)) : 0) + extra_launches;
   }
   out->extra_samples = hc.extra_samples;
   out->panel_ctas = look_ctas;

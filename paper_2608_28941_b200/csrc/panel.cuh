@@ -1053,9 +1053,8 @@ constexpr int kCornerSmem = 3 * kHalf * (kHalf + 4) * 8;
 template <typename T>
 __global__ void __launch_bounds__(256)
     tfactor_kernel(const double* __restrict__ gram, const double* __restrict__ tau, int b,
-                   T* __restrict__ Tout, long long ldt, const int* done_flag, unsigned* bar_reset) {
+                   T* __restrict__ Tout, long long ldt, const int* done_flag) {
   if (*reinterpret_cast<const volatile int*>(done_flag)) return;
-  if (threadIdx.x == 0 && bar_reset != nullptr) *bar_reset = 0;   // the panel before this kernel is finished with it
   extern __shared__ double tsm_k[];
   tfactor_block<T>(gram, tau, b, Tout, ldt, tsm_k);
 }

@@ -726,3 +726,21 @@ def test_replayed_graph_that_holds_fewer_passes_than_the_new_input_needs(h, sche
     assert check(A_big) == k_big       # captured anew
     dA.copy_(torch.from_numpy(A_small))
     assert check(A_small) == k_small   # the longer graph serves the shorter input
+
+
+@pytest.mark.parametrize("m,n,b,max_rank,dtype,flags,launches", [
+    # sample, loop state, and per pass V^T W, T Z, update, stop beside the panel: a square last panel has its T apart
+    (128, 200, 64, 128, torch.float64, rrf.RRF_FLAG_ONE_QUEUE, 2 + 2 * 4 + 1 + 2),
+    # 128 columns: too tall for the SMs (one kernel and T), then two halves and the three kernels of the corner
+    (47400, 256, 128, 256, torch.float64, 0, 2 + 2 * 4 + 2 + 5),
+    (2000, 1000, 128, 256, torch.float32, 0, 2 + 2 * 4 + 2 * 2),
+    # look-ahead: a second sample ahead of the loop
+    (2000, 1000, 64, 256, torch.float64, rrf.RRF_FLAG_TWO_QUEUES, 3 + 4 * 4 + 4),
+])
+def test_kernel_launches_are_counted_as_they_are(h, m, n, b, max_rank, dtype, flags, launches):
+    gen = torch.Generator(device="cuda").manual_seed(m)
+    A = torch.randn((m, n), dtype=dtype, device="cuda", generator=gen)
+    OmT = torch.randn((max_rank, n), dtype=dtype, device="cuda", generator=gen)
+    for _ in range(3):                       # enqueued directly, captured into a graph, replayed
+        g = rrf.rrf_run(h, A, b, 0.0, max_rank, omegaT=OmT, flags=flags | rrf.RRF_FLAG_FIXED_RANK)
+        assert g.kernel_launches == launches
