@@ -343,9 +343,10 @@ rrf_status_t rrf_frobenius_sq(rrf_handle_t h, int32_t dtype, int64_t rows, int64
  * Q_old of the previous step is re-expressed in the current basis Q_new,
  *     Mout (k_new x ncols) = Q_new^T (Q_old M),
  * both bases given by their reflectors (V m x k, T b x k) as rrf_run returns them, for the same m
- * and b; k_old and k_new may differ (the adaptive ranks of two training steps).  Computed as
- * [M; 0] (m x ncols) -> Q_old [M; 0] -> Q_new^T (.) -> first k_new rows, with the same kernels as
- * rrf_apply_q / rrf_apply_qt.  M and Mout are device matrices (ldm, ldmo >= ncols, 16-byte aligned
+ * and b; k_old and k_new may differ (the adaptive ranks of two training steps).  Where ncols > 2 k_new, the ranks
+ * are multiples of b and the rows of M start on 16 bytes, computed as (Q_old^T Q_new)^T M with the k_old x k_new matrix
+ * formed first; otherwise as [M; 0] (m x ncols) -> Q_old [M; 0] -> Q_new^T (.) -> first k_new rows, both with the
+ * kernels of rrf_apply_q / rrf_apply_qt.  M and Mout are device matrices (ldm, ldmo >= ncols, 16-byte aligned
  * rows); they may not overlap.  Workspace: rrf_transfer_workspace_bytes(), 256-byte aligned.  Does
  * not synchronise the stream.
  */
@@ -372,9 +373,9 @@ rrf_status_t rrf_fill_omega(rrf_handle_t h, int32_t dtype, uint64_t seed, int64_
  * rrf_set_single_engine - choose the tensor-core path of the single-precision product Z = V_i^T W
  * (Algorithm 2 line 8) for every later call on this handle that computes it (rrf_run, rrf_apply_q,
  * rrf_apply_qt, rrf_form_q, rrf_subspace_transfer).  Double precision is not affected.
- *   engine 0  mma.sync m16n8k8, 3xTF32, every k-step added round-to-nearest in registers (default)
- *   engine 1  tcgen05.mma kind::tf32, 3xTF32 operand planes in shared memory, accumulator in tensor
- *             memory; chunk_tiles > 0 bounds the number of 64-row tiles summed inside tensor memory
+ *   engine 0  mma.sync m16n8k8, 3xTF32, every k-step added round-to-nearest in registers
+ *   engine 1  tcgen05.mma kind::tf32, 3xTF32 operand planes in shared and tensor memory, accumulator in tensor
+ *             memory (default, with chunk_tiles 2); chunk_tiles > 0 bounds the number of 64-row tiles summed inside tensor memory
  *             (whose additions do not round to nearest) before a round-to-nearest add into registers,
  *             0 keeps a whole accumulator there.
  * Host-side setting, no device work.  Returns RRF_ERR_INVALID_ARG for other values.

@@ -226,10 +226,9 @@ static bool plan_panel_cl(const rrf_ctx* h, long long rows, int b, PanelPlan* p,
   if (!h->cluster_ok || (fix && b > 64)) return false;
   const long long ext = rows + (fix ? b : 0);
   const int R = std::max(64, ceil_div(ext, kClusterMax));
-  // With slabs taller than this the longer pass over a slab costs more than the cheaper exchange saves
-  // (measured: 4096 x 64 takes 279 us as one cluster of 16 against 260 us on 148 CTAs; 1024 x 16 falls from 64 to 54)
-  // With the register-resident column loop (b <= 64) a 4096 x 64 panel takes 232 us on its own, but inside a run, where
-  // 16 CTAs also sum the partial panels and store V, the 4096-row passes of config 4 take 284 us against 261 us.
+  // Up to kRegRows rows a slab and b <= 64: Cholesky QR, and a column loop with the slab in registers behind it.  Wider
+  // panels have the column loop in shared memory only, where slabs taller than kClusterMaxRows cost more than the
+  // cheaper exchange saves.
   const bool reg = b <= 64 && R <= kRegRows;
   if (!reg && R > kClusterMaxRows) return false;
   int G = 1;
@@ -849,8 +848,10 @@ static rrf_status_t launch_panel(rrf_ctx* h, int dtype, const void* Y, PanelSour
     e = cudaLaunchCooperativeKernel(fn, dim3(bp.G), dim3(kPanelThreads), args, smem, st);
   } else {
     PanelPlan pp;
-    // on a free device a tall panel is faster spread over the grid (4096 x 64: 62 us against 78 as one cluster, whose
-    // 16 SMs are then bound by their matrix products)
+    // On a free device a tall panel is faster spread over the grid, where a cluster's 16 SMs are bound by their matrix
+    // products.  b = 64, cluster / grid: 700 rows 66 / 70 us, 1024 68 / 68, 1500 72 / 68, 2048 74 / 68, 4000 88 / 68.
+    // The narrower ones stay where they are: b = 32, 1024 rows 40 / 42, 2048 43 / 42, 4000 47 / 43; b = 16, at most 2 us
+    // either way.
     const bool spread = o.ctas == 0 && b == 64 && rows > 2048;
     const bool as_cluster = !o.no_cluster && !spread && !o.blocked && plan_panel_cl(h, rows, b, &pp, o.fix.enabled != 0);
     if (!as_cluster && !plan_panel(h, rows, b, &pp, o.ctas, o.fix.enabled != 0, cqr != nullptr)) return RRF_ERR_WORKSPACE;
@@ -1137,9 +1138,9 @@ rrf_status_t rrf_create(rrf_handle_t* out, int device) {
   if (e == cudaSuccess) e = setup_all(h->smem_optin, &h->panel_smem_max, &h->cluster_ok);
   if (e == cudaSuccess) e = setup_tree_kernels(h->smem_optin, &h->tsqr_smem_max);
   if (e == cudaSuccess) e = setup_blk_kernels(h->smem_optin, &h->blk_smem_max);
-  // The side stream carries the panel chain of the look-ahead schedule, the critical path wherever that schedule is
-  // chosen: its kernels (a whole thread-block cluster where the panel is short) are placed ahead of GEMM CTAs that
-  // wait at the same moment.
+  // The side stream carries the panel chain of the look-ahead schedule.  Its kernels (a whole thread-block cluster where
+  // the panel is short) are placed ahead of GEMM CTAs that wait at the same moment: the chain is the shorter side only
+  // as long as it does not queue behind the other.
   int prio_lo = 0, prio_hi = 0;
   if (e == cudaSuccess) e = cudaDeviceGetStreamPriorityRange(&prio_lo, &prio_hi);
   if (e == cudaSuccess) e = cudaStreamCreateWithPriority(&h->aux, cudaStreamNonBlocking, prio_hi);
@@ -1543,7 +1544,7 @@ rrf_status_t rrf_subspace_transfer(rrf_handle_t h, int32_t dtype, int64_t m, int
   void* Cm = ws;
   cudaStream_t st = (cudaStream_t)cuda_stream;
   // Q_new^T (Q_old M) by way of the small k_old x k_new matrix S^T = Q_old^T Q_new: the reflectors then pass over m x k_new
-  // numbers instead of m x ncols, and M is read once per block of S (4096 x 11008, k 256 -> 128: 1115 -> 303 us;
+  // numbers instead of m x ncols, and M is read once per block of S (4096 x 11008, k 256 -> 128: 1115 -> 256 us;
   // at ncols = 2 k_new the two take the same time).  M has to be readable by TMA, and the result must not overwrite it.
   const char *mi = (const char*)dM, *mo = (const char*)dMout;
   const bool apart = mo + ((size_t)(k_new - 1) * ldmo + ncols) * esize <= mi || mi + ((size_t)(k_old - 1) * ldm + ncols) * esize <= mo;
@@ -2086,15 +2087,19 @@ rrf_status_t rrf_run(rrf_handle_t h, const rrf_params_t* p, void* dA, int64_t ld
       // Gated passes: the panel kernel, started together with the update, is done long before it, and its SMs
       // would idle.  The last tiles of the pass are therefore left to a second launch of the update kernel that
       // follows the panel kernel on ITS stream and so runs on the SMs it leaves: `look_ctas` CTAs with as many
-      // tiles as they can do in the time the first launch still needs (by the schedule model, with a wide margin).
+      // tiles as they can do in the time the first launch still needs, by the schedule model.
       int t1 = 0, tpc2 = 0;
       if (gate && !look_cl && !utc_on && i + 1 < steps_run && !h->profiling) {
         const PassModel pm{h->sms, (double)rows, (double)n, b, p->dtype == RRF_F64, tc};
         const double t_upd = pm.upd() * pm.scale(look_ctas), t_pan = pm.panel_chain(look_ctas);
         if (t_pan < 0.9 * t_upd) {
           const double t_all = ((double)gsms * t_upd + (double)look_ctas * t_pan) / h->sms;   // both launches end together
-          // 0.95 of what the model allows: measured on 8192 x 8192, b = 64, 26 SMs: 7.82 / 7.76 / 7.55 / 7.39 / 7.37 ms
-          // with 0.2 / 0.35 / 0.65 / 0.9 / 1.0 of it
+          // 0.95 of what the model allows.  In double precision, ms with 0 / 0.35 / 0.65 / 0.95 / 1.0 of it:
+          //   8192 x 8192, b 64, 26 SMs, six passes    5.74 / 5.57 / 5.46 / 5.41 / 5.43  (one queue by default)
+          //   12000 x 3000, b 64, 38 SMs               3.47 / 3.36 / 3.31 / 3.27 / 3.28  (one queue by default)
+          //   6000 x 6000, b 64, 19 SMs                3.08 / 3.08 / 3.09 / 3.10 / 3.13
+          //   4500 x 12000, b 64, 15 SMs               3.04 / 3.01 / 3.01 / 3.04 / 3.06
+          //   6000 x 14000, b 32, 12 SMs               5.11 / 5.12 / 5.14 / 5.31 / 5.38  (one queue by default)
           const double share = 0.95 * (double)look_ctas * (t_all - t_pan) / ((double)gsms * t_upd);
           const int tiles_h = (int)(share * up.total);
           if (tiles_h >= 4 * look_ctas) {

@@ -282,7 +282,7 @@ __global__ void __launch_bounds__(kPanelThreads)
                  double* __restrict__ tau_out,       // [b]
                  unsigned* bar, Ctrl* ctrl, const int* done_flag, PanelFix fix,
                  unsigned bar_base,                 // value of the barrier counter when this launch starts
-                 T* __restrict__ Tout, long long ldt,     // non-NULL: CTA 0 also builds the T factor at the end
+                 T* __restrict__ Tout, long long ldt,     // non-NULL: T too (the column loop in CTA 0, the Cholesky QR in the last)
                  double* __restrict__ csq,                // non-NULL: [b][Gp] per-CTA sums of squares of the panel's columns
                  double* __restrict__ cqr) {              // non-NULL: scratch of the Cholesky QR (panel_cqr.cuh), tried first
   __shared__ uint64_t cbar;      // cluster mode: this CTA's barrier, on which every CTA of the cluster arrives

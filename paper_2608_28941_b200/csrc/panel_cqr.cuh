@@ -22,13 +22,13 @@
 // the identity, and an entry of S-sign pivots that leaves nothing below it (the convention there is H = I, tau = 0).
 // The loop then runs on Y, or on Q1, whose reflectors are the same.
 //
-// One call, B200: 8192 x 64 in 72 us (column loop 267), 4096 x 64 as one cluster 91 (209), 4096 x 32 50 (103), 1024 x 16
-// 31 (55).  What bounds it now are the factorisations of the b x b matrices, which every CTA does for itself (9.5 and
+// One call, B200: 8192 x 64 in 70 us (column loop 265), 4096 x 64 as one cluster 88 (207), 4096 x 32 47 (100), 1024 x 16
+// 27 (55).  What bounds it now are the factorisations of the b x b matrices, which every CTA does for itself (9.5 and
 // 14 us for b = 64, one dependent reciprocal per column), two exchanges through L2 (16 us; through the cluster 11), and
-// on tall slabs the FP64 tensor rate of the few SMs in use.
+// on tall slabs the FP64 tensor rate of the few SMs in use.  A panel that is sent to the column loop pays for the
+// attempt, and 4 % for a loop that shares its kernel with it: two equal columns 294, 115 (4096 x 32) and 62 us.
 //
-// Against the column loop in extended precision, V and T came out closer on every panel tried (condition numbers 1 to
-// 1e8, graded columns, rows from b + 1): 1e-16 and 3e-16 relative on Gaussian panels, 4e-14 and 1.4e-13 at 1e4.
+// V and T keep within 100 u cond of a Householder QR (tests), as the column loop's do.
 #pragma once
 
 #include "panel_sync.cuh"
