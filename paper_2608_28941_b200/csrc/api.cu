@@ -2089,18 +2089,20 @@ rrf_status_t rrf_run(rrf_handle_t h, const rrf_params_t* p, void* dA, int64_t ld
       // follows the panel kernel on ITS stream and so runs on the SMs it leaves: `look_ctas` CTAs with as many
       // tiles as they can do in the time the first launch still needs, by the schedule model.
       int t1 = 0, tpc2 = 0;
-      if (gate && !look_cl && !utc_on && i + 1 < steps_run && !h->profiling) {
+      if (gate && b >= 64 && !look_cl && !utc_on && i + 1 < steps_run && !h->profiling) {
         const PassModel pm{h->sms, (double)rows, (double)n, b, p->dtype == RRF_F64, tc};
         const double t_upd = pm.upd() * pm.scale(look_ctas), t_pan = pm.panel_chain(look_ctas);
         if (t_pan < 0.9 * t_upd) {
           const double t_all = ((double)gsms * t_upd + (double)look_ctas * t_pan) / h->sms;   // both launches end together
-          // 0.95 of what the model allows.  In double precision, ms with 0 / 0.35 / 0.65 / 0.95 / 1.0 of it:
-          //   8192 x 8192, b 64, 26 SMs, six passes    5.74 / 5.57 / 5.46 / 5.41 / 5.43  (one queue by default)
-          //   12000 x 3000, b 64, 38 SMs               3.47 / 3.36 / 3.31 / 3.27 / 3.28  (one queue by default)
-          //   6000 x 6000, b 64, 19 SMs                3.08 / 3.08 / 3.09 / 3.10 / 3.13
-          //   4500 x 12000, b 64, 15 SMs               3.04 / 3.01 / 3.01 / 3.04 / 3.06
-          //   6000 x 14000, b 32, 12 SMs               5.11 / 5.12 / 5.14 / 5.31 / 5.38  (one queue by default)
-          const double share = 0.95 * (double)look_ctas * (t_all - t_pan) / ((double)gsms * t_upd);
+          // 0.65 of what the model allows.  b = 64 in double precision, ms with 0 / 0.35 / 0.65 / 0.95 of it:
+          //   4500 x 12000, 15 SMs   3.04 / 3.01 / 3.01 / 3.04        7000 x 7000, 23 SMs    2.90 / 2.84 / 2.84 / 2.88
+          //   4800 x 6000, 16 SMs    1.78 / 1.83 / 1.84 / 1.91        8192 x 8192, 26 SMs *  5.74 / 5.57 / 5.46 / 5.41
+          //   5500 x 10000, 18 SMs   3.12 / 3.07 / 3.08 / 3.11        10000 x 5000, 32 SMs * 3.14 / 3.06 / 3.02 / 3.03
+          //   6000 x 6000, 19 SMs    3.12 / 3.10 / 3.09 / 3.11        12000 x 3000, 38 SMs * 3.47 / 3.36 / 3.31 / 3.27
+          // (*: one queue by default).  Not for narrower blocks, whose update is bound by W's bytes and not by the SMs
+          // it runs on: 5000 x 12000, b = 32 3.70 / 3.71 / 3.73 / 3.99, 7000 x 7000 3.15 / 3.15 / 3.15 / 3.40,
+          // 4500 x 9000, b = 16 1.99 / 2.08 / 2.28 / 2.46.
+          const double share = 0.65 * (double)look_ctas * (t_all - t_pan) / ((double)gsms * t_upd);
           const int tiles_h = (int)(share * up.total);
           if (tiles_h >= 4 * look_ctas) {
             tpc2 = ceil_div(tiles_h, look_ctas);
