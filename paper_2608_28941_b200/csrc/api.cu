@@ -14,6 +14,7 @@
 #include "gemm_tc.cuh"
 #include "gemm_tc_upd.cuh"
 #include "gemm_tc_vtw.cuh"
+#include "gemm_i8.cuh"
 #include "panel_blk.cuh"
 
 // NVTX ranges around the phases of rrf_run (host-side enqueue order), compiled in with -DRRF_NVTX only
@@ -79,6 +80,7 @@ struct rrf_ctx {
   int gextra;                            // its kernels beyond those that every pass has (extra_launches in rrf_run)
   int cluster_ok;                        // a 16-CTA cluster of the panel kernel can be resident on this device
   int f32_engine;                        // single-precision V^T W: 0 = mma.sync 3xTF32, 1 = tcgen05 3xTF32
+  int f64_engine;                        // double precision: 0 = mma.sync f64, 1 = integer tensor cores, 2 = by size
   int tc_chunk;                          // tcgen05: 64-row tiles summed in tensor memory between round-to-nearest adds
 };
 
@@ -431,12 +433,20 @@ struct PassModel {
   int b;
   bool f64;
   bool tc;      // single precision on tcgen05
+  bool oz = false;    // double precision on the integer tensor cores
   // flop per microsecond the two GEMM kernels sustain on the whole device; narrow blocks read and write W for less
   double rate(double wide) const { return b >= 64 ? wide : (f64 ? wide * (b == 32 ? 0.75 : 0.5) : wide * 0.5); }
-  double vtw() const { return 2.0 * rows * n * b / rate(f64 ? 34e6 : (tc ? 86e6 : 45e6)) + 10.0; }
-  double upd() const { return 4.0 * rows * n * b / rate(f64 ? 33e6 : (tc && b <= 64 ? 117e6 : 32e6)) + 15.0; }
+  // integer tensor cores: bytes of W per microsecond (8192 x 8192, 148 SMs)
+  double vtw() const {
+    if (oz) return 8.0 * rows * n / (b == 32 ? 4.3e6 : (b == 64 ? 3.6e6 : 2.1e6)) + 8.0;
+    return 2.0 * rows * n * b / rate(f64 ? 34e6 : (tc ? 86e6 : 45e6)) + 10.0;
+  }
+  double upd() const {      // with the sample of a later panel
+    if (oz) return 16.0 * rows * n / (b == 32 ? 5.1e6 : (b == 64 ? 4.4e6 : 2.7e6)) + 10.0 + vtw();
+    return 4.0 * rows * n * b / rate(f64 ? 33e6 : (tc && b <= 64 ? 117e6 : 32e6)) + 15.0;
+  }
   // T Z, the stop rule, the split planes and the hand-overs between them
-  double rest() const { return f64 ? 20.0 : 35.0; }
+  double rest() const { return f64 ? (oz ? 35.0 : 20.0) : 35.0; }
   // load + fix-up + panel on `ctas` SMs, with the launch and event hand-overs of the side stream: the b x b
   // factorisations, the products over a slab, the partial results read beside the GEMM kernels (measured inside runs:
   // 31 us for 1024 x 16 on 16 SMs, 92 for 4096 x 32 and 158 for 4096 x 64 on 16, 116 for 5003 x 64 on 45, 225 for
@@ -509,6 +519,18 @@ static bool make_map(const rrf_ctx* h, CUtensorMap* map, int dtype, const void* 
                                CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
                                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   return r == CUDA_SUCCESS;
+}
+
+// double precision, box of box_cols x box_rows elements without a swizzle
+static bool make_map_plain(const rrf_ctx* h, CUtensorMap* map, const void* base, unsigned long long rows, unsigned long long cols,
+                           unsigned long long ld, unsigned box_cols, unsigned box_rows) {
+  cuuint64_t gdim[2] = {cols, rows};
+  cuuint64_t gstr[1] = {ld * 8ull};
+  cuuint32_t box[2] = {box_cols, box_rows};
+  cuuint32_t estr[2] = {1, 1};
+  return h->encode(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT64, 2, const_cast<void*>(base), gdim, gstr, box, estr,
+                   CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
 static bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
@@ -611,7 +633,8 @@ struct Ops {
     launch_after(dep, vtw_sk_kernel<T, B, V_BN, kVtwBK, V_WM, V_WN, V_STAGES>, p.P, 9 * 32, V_SMEM, st, tmV, tmC, (T*)Zpart,
                  r0, cv0, p.KT, p.total, p.tpc, ctrl);
   }
-  static constexpr int Z_SMEM = (B * (B + 4) + B * (kTzCols + 4)) * (int)sizeof(T);   // enough for the narrow form too
+  static constexpr int Z_SMEM = (B * (B + 4) + B * (kTzCols + 4)) * (int)sizeof(T)    // enough for the narrow form too
+                                + (sizeof(T) == 8 && B >= 32 ? kTzCols * (B + 2) * 8 : 0);
   static void tz(const void* Zpart, const VtwPlan& vp, const void* Tm, long long ldt, int transpose_t, void* Zt,
                  const int* done_flag, TzSplit sp, bool dep, cudaStream_t st) {
     // half as many columns a CTA where that still is at most one CTA per SM: a column tile then has few CTAs and many
@@ -692,6 +715,126 @@ static const OpTable* get_ops(int dtype, int b) {
     }
   }
   return nullptr;
+}
+
+// ------------------------------------------------------------------ double precision on the integer tensor cores (gemm_i8.cuh)
+template <int B>
+struct OzOps {
+  static constexpr int NB = B < 64 ? B : 64;
+  static cudaError_t setup() {
+    cudaError_t e = cudaFuncSetAttribute(oz_gemm_kernel<NB, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, OzCfg<NB>::SMEM);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(oz_gemm_kernel<NB, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, OzCfg<NB>::SMEM);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(oz_update_kernel<B>, cudaFuncAttributeMaxDynamicSharedMemorySize, OzuCfg<B>::SMEM);
+    return e;
+  }
+  static void split(const OzSplit& a, int grid, const int* done_flag, bool dep, cudaStream_t st) {
+    launch_after(dep, oz_split_kernel<B>, grid, 256, 0, st, a, done_flag);
+  }
+  static void gemm(bool tr, const CUtensorMap& tm, const unsigned char* img, const int* e, const uint32_t* mag, double* part, int r0,
+                   int lines, int first, const VtwPlan& p, Ctrl* ctrl, bool dep, cudaStream_t st) {
+    launch_after(dep, tr ? oz_gemm_kernel<NB, true> : oz_gemm_kernel<NB, false>, p.P * (B / NB), kOzThreads, OzCfg<NB>::SMEM, st, tm,
+                 img, e, mag, part, B, r0, lines, first, p.KT, p.total, p.tpc, ctrl);
+  }
+  static void update(const CUtensorMap& tm, const CUtensorMap& tms, const CUtensorMap& tmt, const unsigned char* vimg, const int* ev,
+                     const unsigned char* zimg, const int* ez, int r0, int rows, int ncols, int top_rows, double* norm_part,
+                     uint32_t* colmag, uint32_t* rowmag, const UpdPlan& p, Ctrl* ctrl, bool dep, cudaStream_t st) {
+    launch_after(dep, oz_update_kernel<B>, p.P, kOzuThreads, OzuCfg<B>::SMEM, st, tm, tms, tmt, vimg, ev, zimg, ez, r0, rows, ncols,
+                 top_rows, norm_part, colmag, rowmag, p.NC, p.total, p.tpc, ctrl);
+  }
+};
+struct OzTable {
+  cudaError_t (*setup)();
+  void (*split)(const OzSplit&, int, const int*, bool, cudaStream_t);
+  void (*gemm)(bool, const CUtensorMap&, const unsigned char*, const int*, const uint32_t*, double*, int, int, int, const VtwPlan&, Ctrl*,
+               bool, cudaStream_t);
+  void (*update)(const CUtensorMap&, const CUtensorMap&, const CUtensorMap&, const unsigned char*, const int*, const unsigned char*,
+                 const int*, int, int, int, int, double*, uint32_t*, uint32_t*, const UpdPlan&, Ctrl*, bool, cudaStream_t);
+};
+static const OzTable* oz_ops(int b) {
+  static const OzTable t32{&OzOps<32>::setup, &OzOps<32>::split, &OzOps<32>::gemm, &OzOps<32>::update},
+      t64{&OzOps<64>::setup, &OzOps<64>::split, &OzOps<64>::gemm, &OzOps<64>::update},
+      t128{&OzOps<128>::setup, &OzOps<128>::split, &OzOps<128>::gemm, &OzOps<128>::update};
+  return b == 32 ? &t32 : (b == 64 ? &t64 : (b == 128 ? &t128 : nullptr));
+}
+// Stream-K plan of a product: `lines` in tiles of 128, `len` contraction indices in tiles of 64; the b / 64 CTAs that share a
+// tile of a wide block count as one
+static VtwPlan plan_oz(int sms, long long lines, long long len, int b) {
+  VtwPlan p = plan_vtw(std::max(1, sms / std::max(1, b / 64)), len, lines, 128);
+  return p;
+}
+static int oz_chunks(int steps, int first) {
+  return steps <= first ? 1 : (first > 0 ? 1 : 0) + ceil_div(steps - first, kOzChunk);
+}
+// The operands' images and scales in a workspace
+struct OzBuf {
+  unsigned char *vrow, *vcol, *zimg, *oimg;
+  int *erow, *ecol, *ez, *eo;
+  uint32_t *colmag[2], *rowmag[2];
+  size_t bytes;
+};
+static OzBuf oz_carve(unsigned char* base, long long m, long long n, int b, bool sampled) {
+  OzBuf o{};
+  size_t off = 0;
+  auto take = [&](size_t bytes) {
+    unsigned char* q = base + off;
+    off += align_up(bytes, 256);
+    return q;
+  };
+  const size_t sv = 2 * (size_t)ceil_div(m, 64), so = 2 * (size_t)ceil_div(n, 64), npad = align_up((size_t)n, 128);
+  o.vrow = take((size_t)ceil_div(m, 128) * (b / 32) * kOzS * 4096);
+  o.vcol = take(sv * kOzS * b * 32);
+  o.zimg = take(npad / 32 * (b / 32) * kOzS * 1024);
+  o.erow = (int*)take((size_t)m * 4);
+  o.ecol = (int*)take((size_t)oz_chunks((int)sv, b / 32) * b * 4);
+  o.ez = (int*)take(npad * 4);
+  for (int q = 0; q < 2; ++q) o.colmag[q] = (uint32_t*)take((size_t)n * 4);
+  if (sampled) {
+    o.oimg = take(so * kOzS * b * 32);
+    o.eo = (int*)take((size_t)oz_chunks((int)so, 0) * b * 4);
+    for (int q = 0; q < 2; ++q) o.rowmag[q] = (uint32_t*)take((size_t)m * 4);
+  }
+  o.bytes = off;
+  return o;
+}
+// What the split kernel works on: a block of V (rows x b) and / or b rows of OmegaT
+static int oz_split_args(const OzBuf& o, OzSplit* a, int b, const double* V, long long ldv, long long rows, const double* Om,
+                         long long ldo, long long n) {
+  *a = OzSplit{};
+  if (V != nullptr) {
+    a->V = V;
+    a->ldv = ldv;
+    a->rows = (int)rows;
+    a->nslab = ceil_div(rows, 128);
+    a->steps_v = 2 * ceil_div(rows, 64);
+    a->chunks_v = oz_chunks(a->steps_v, b / 32);
+    a->vrow = o.vrow;
+    a->vcol = o.vcol;
+    a->erow = o.erow;
+    a->ecol = o.ecol;
+  }
+  if (Om != nullptr) {
+    a->Om = Om;
+    a->ldo = ldo;
+    a->n = (int)n;
+    a->steps_o = 2 * ceil_div(n, 64);
+    a->chunks_o = oz_chunks(a->steps_o, 0);
+    a->oimg = o.oimg;
+    a->eo = o.eo;
+  }
+  return a->nslab + (a->chunks_v + a->chunks_o) * (b / 16);
+}
+static int oz_mag_grid(long long rows, long long cols, int most) {
+  return (int)std::min<long long>(most, (long long)ceil_div(rows, kMagRows) * ceil_div(cols, kMagCols));
+}
+// Whether a double-precision call over a rows x n matrix takes the integer tensor cores.
+static bool oz_wanted(const rrf_ctx* h, int dtype, long long rows, long long n, int b) {
+  if (dtype != RRF_F64 || b < 32 || h->f64_engine == 0) return false;
+  if (h->f64_engine == 1) return true;
+  // The digits of V and Omega are made per block, which a matrix of few columns does not repay, and the kernels are two more
+  // a pass.  Eight blocks, us without / with: b = 128, 2000 x 2000 2493 / 2331, 8192 x 8192 14321 / 9096; b = 64, 2000 x 2000
+  // 1054 / 1129, 3000 x 3000 1389 / 1421, 2000 x 6000 1596 / 1430, 8192 x 8192 7193 / 5285; b = 32, 4096 x 4096 1292 / 1472,
+  // 8192 x 8192 4280 / 4329, 20000 x 4000 5238 / 5087 (the bytes of W bound both).
+  return b >= 64 && n >= 8LL * b && rows * n >= (b == 64 ? 10000000LL : 4000000LL);
 }
 
 // panel QR + T factor, enqueued on `st`
@@ -1009,6 +1152,10 @@ static cudaError_t setup_all(int smem_optin, int* panel_smem_max, int* cluster_o
     e = get_ops(RRF_F32, b)->setup();
     if (e != cudaSuccess) return e;
   }
+  for (int b : {32, 64, 128}) {
+    e = oz_ops(b)->setup();
+    if (e != cudaSuccess) return e;
+  }
   e = cudaFuncSetAttribute(corner_t_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kCornerSmem);
   if (e != cudaSuccess) return e;
   return setup_panel_kernels(smem_optin, panel_smem_max, cluster_ok);
@@ -1022,6 +1169,7 @@ static size_t tc_split_bytes(int npad, int b, long long n) {
 // ------------------------------------------------------------------ workspace of rrf_run
 struct RunLayout {
   size_t ctrl, traces, done_after, norm_part, init_part, ypart, ypart2, zpart, zt, tcsplit, panel, look, csq, w, omega, total;
+  size_t oz, ozy, ozy2, ozz, total_oz;      // with the integer tensor cores; a workspace of `total` bytes serves the other path
   int init_ctas, max_norm_parts;
   long long ldw;
 };
@@ -1066,6 +1214,14 @@ static bool run_layout(const rrf_params_t* p, bool need_omega, RunLayout* L) {
   L->omega = off;
   if (need_omega) off += align_up((size_t)p->max_rank * (size_t)p->n * esize, 256);
   L->total = off;
+  L->oz = off;
+  if (p->dtype == RRF_F64 && b >= 32) {
+    off += oz_carve(nullptr, p->m, p->n, b, true).bytes;
+    L->ozy = off; off += align_up((size_t)(sms + ceil_div(p->m, 128)) * 128 * b * 8, 256);     // slots <= P + tiles
+    L->ozy2 = off; off += align_up((size_t)(sms + ceil_div(p->m, 128)) * 128 * b * 8, 256);
+    L->ozz = off; off += align_up((size_t)(sms + ceil_div(p->n, 128)) * 128 * b * 8, 256);
+  }
+  L->total_oz = off;
   return true;
 }
 
@@ -1125,6 +1281,7 @@ rrf_status_t rrf_create(rrf_handle_t* out, int device) {
   h->gsteps = 0;
   h->gextra = 0;
   h->f32_engine = 1;      // single precision runs on tcgen05 unless rrf_set_single_engine says otherwise
+  h->f64_engine = 2;
   h->tc_chunk = 2;
   std::memset(&h->profile, 0, sizeof(h->profile));
   cudaError_t e = cudaDeviceGetAttribute(&h->sms, cudaDevAttrMultiProcessorCount, device);
@@ -1184,6 +1341,12 @@ rrf_status_t rrf_set_single_engine(rrf_handle_t h, int32_t engine, int32_t chunk
   if (h == nullptr || engine < 0 || engine > 1 || chunk_tiles < 0) return RRF_ERR_INVALID_ARG;
   h->f32_engine = engine;
   h->tc_chunk = chunk_tiles;
+  return RRF_OK;
+}
+
+rrf_status_t rrf_set_double_engine(rrf_handle_t h, int32_t engine) {
+  if (h == nullptr || engine < 0 || engine > 2) return RRF_ERR_INVALID_ARG;
+  h->f64_engine = engine;
   return RRF_OK;
 }
 
@@ -1264,7 +1427,7 @@ rrf_status_t rrf_workspace_bytes(const rrf_params_t* p, size_t* bytes) {
   if (s != RRF_OK) return s;
   RunLayout L;
   run_layout(p, true, &L);
-  *bytes = L.total;
+  *bytes = L.total_oz;
   return RRF_OK;
 }
 
@@ -1635,6 +1798,11 @@ rrf_status_t rrf_run(rrf_handle_t h, const rrf_params_t* p, void* dA, int64_t ld
   RunLayout L;
   run_layout(p, dOmegaT == nullptr, &L);
   if (workspace_bytes < L.total) return fail(RRF_ERR_WORKSPACE);
+  // Double precision on the integer tensor cores: large problems, unless the caller chose how later panels are sampled (the
+  // sample is a product of its own there) or one of the other panel kernels.  A workspace sized without it is enough for
+  // the other path.
+  const bool oz = oz_wanted(h, p->dtype, m, n, b) && workspace_bytes >= L.total_oz &&
+                  !(p->flags & (RRF_FLAG_SAMPLE_ALWAYS | RRF_FLAG_SAMPLE_NEVER | RRF_FLAG_PANEL_TREE | RRF_FLAG_PANEL_BLOCKED));
   // Schedule.  Two queues (look-ahead) when the tallest panel fits in the shared memory of a small
   // share of the SMs, so that confining the panel there costs the GEMM kernels little; else one queue.
   const int steps_total = p->max_rank / b;
@@ -1659,8 +1827,8 @@ rrf_status_t rrf_run(rrf_handle_t h, const rrf_params_t* p, void* dA, int64_t ld
              plan_panel_cl(h, m, b, &pcl_probe0, false)) {
     // every panel of the chain fits one thread-block cluster (the first as it is, the later ones with the b rows
     // of the fix-up): the chain takes only that many SMs
-    const PassModel pm{h->sms, (double)m, (double)n, b, p->dtype == RRF_F64, p->dtype == RRF_F32 && h->f32_engine == 1};
-    const double t = std::min(pm.step_ungated(kClusterMax), pm.step_gated(kClusterMax));
+    const PassModel pm{h->sms, (double)m, (double)n, b, p->dtype == RRF_F64, p->dtype == RRF_F32 && h->f32_engine == 1, oz};
+    const double t = oz ? pm.step_ungated(kClusterMax) : std::min(pm.step_ungated(kClusterMax), pm.step_gated(kClusterMax));
     if ((p->flags & RRF_FLAG_TWO_QUEUES) || t < pm.step_serial()) {
       // The GEMM kernels get every SM the cluster does not take (4096 x 11008 fp32: 2.00 ms with 16 SMs kept free, 2.08
       // with 26, 2.33 with 44; 4096 x 4096 fp64, b = 32: 1.80 with 16, 2.05 with 44; 5003 x 3001 likewise on a grid)
@@ -1672,11 +1840,11 @@ rrf_status_t rrf_run(rrf_handle_t h, const rrf_params_t* p, void* dA, int64_t ld
     const int fewest = panel_min_ctas(h, m, b);
     const int cap = std::min(kLookMaxCtas, h->sms / 3);
     if (fewest > 0 && fewest <= cap) {
-      const PassModel pm{h->sms, (double)m, (double)n, b, p->dtype == RRF_F64, p->dtype == RRF_F32 && h->f32_engine == 1};
+      const PassModel pm{h->sms, (double)m, (double)n, b, p->dtype == RRF_F64, p->dtype == RRF_F32 && h->f32_engine == 1, oz};
       int best = fewest;
-      double best_t = std::min(pm.step_ungated(fewest), pm.step_gated(fewest));
+      double best_t = oz ? pm.step_ungated(fewest) : std::min(pm.step_ungated(fewest), pm.step_gated(fewest));
       for (int c = fewest + 1; c <= cap; ++c) {
-        const double t = std::min(pm.step_ungated(c), pm.step_gated(c));
+        const double t = oz ? pm.step_ungated(c) : std::min(pm.step_ungated(c), pm.step_gated(c));
         if (t < best_t * 0.995) {
           best_t = t;
           best = c;
@@ -1714,7 +1882,7 @@ rrf_status_t rrf_run(rrf_handle_t h, const rrf_params_t* p, void* dA, int64_t ld
   // Sampling predictor (see stop_kernel): worth its one skipped-kernel launch per pass only where a pass is
   // long, i.e. where the sample it can save is worth more than those launches cost.
   int predict = 1;
-  const bool predictor_built = b < 128 && p->dtype == RRF_F64;   // see upd_sk_kernel
+  const bool predictor_built = b < 128 && p->dtype == RRF_F64 && !oz;   // see upd_sk_kernel
   if (!predictor_built) {
     predict = 1;
   } else if (p->flags & RRF_FLAG_SAMPLE_NEVER) {
@@ -1789,6 +1957,61 @@ rrf_status_t rrf_run(rrf_handle_t h, const rrf_params_t* p, void* dA, int64_t ld
       return RRF_ERR_INVALID_ARG;
   }
 
+  const OzBuf ob = oz ? oz_carve(ws + L.oz, m, n, b, true) : OzBuf{};
+  const OzTable* const ozt = oz_ops(b);
+  double* const oz_z = reinterpret_cast<double*>(ws + L.ozz);
+  void* const Y0 = oz ? (void*)(ws + L.ozy) : Ypart;
+  void* const Y1 = oz ? (void*)(ws + L.ozy2) : (void*)(ws + L.ypart2);
+  CUtensorMap tmA_t, tmW_t, tmW_st;       // columns of A / W as lines; W as the update stores it
+  if (oz && (!make_map_plain(h, &tmA_t, dA, m, n, lda, 128, kOzK) || !make_map_plain(h, &tmW_t, W, m, n, ldw, 128, kOzK) ||
+             !make_map(h, &tmW_st, p->dtype, W, m, n, ldw, 32)))
+    return RRF_ERR_INVALID_ARG;
+  // digits of block i of V (i >= 0) and of the rows j0 ... of OmegaT (j0 >= 0); zeros for the magnitudes of parity `zero`
+  auto oz_split = [&](int i, int j0, int zero) {
+    OzSplit a;
+    const int grid = oz_split_args(ob, &a, b, i >= 0 ? (const double*)dV + (size_t)(i * b) * ldv + i * b : nullptr, ldv, m - (long long)i * b,
+                                   j0 >= 0 ? (const double*)Om + (size_t)j0 * ldom : nullptr, ldom, n);
+    if (zero >= 0) {
+      a.zero0 = ob.colmag[zero];
+      a.nzero0 = (int)n;
+      a.zero1 = ob.rowmag[zero];
+      a.nzero1 = (int)m;
+    }
+    ozt->split(a, grid, &ctrl->done, false, st);
+  };
+  // panel sampled from rows r0 ... of what `tm` maps, whose row magnitudes are those of parity q; the split before it is done
+  auto oz_sample = [&](const CUtensorMap& tm, int q, int r0, int rows_s, int sms_s, void* Y, int row_off, bool dep) {
+    const VtwPlan sq = plan_oz(sms_s, rows_s, n, b);
+    ozt->gemm(false, tm, ob.oimg, ob.eo, ob.rowmag[q], (double*)Y, r0, rows_s, 0, sq, ctrl, dep, st);
+    PanelSource ps_q{};
+    ps_q.slots = 1;
+    ps_q.row_off = row_off;
+    ps_q.bm = 128;
+    ps_q.nc = sq.KT;
+    ps_q.tpc = sq.tpc;
+    ps_q.wn = 1;
+    return ps_q;
+  };
+  // V^T W, T Z and the update of pass i on `sms_g` SMs, with T_i on the way in on the side stream if `join` is not NULL
+  auto oz_pass = [&](int i, int sms_g, cudaEvent_t join, auto&& mark_f) -> int {
+    const int r0 = i * b, rows = (int)(m - r0);
+    VtwPlan vp = plan_oz(sms_g, n, rows, b);
+    ozt->gemm(true, i == 0 ? tmA_t : tmW_t, ob.vcol, ob.ecol, ob.colmag[i & 1], oz_z, r0, (int)n, b / 32, vp, ctrl, true, st);
+    mark_f(RRF_PHASE_TZ);
+    if (join != nullptr) cudaStreamWaitEvent(st, join, 0);
+    TzSplit sp{};
+    sp.zi = ob.zimg;
+    sp.ez = ob.ez;
+    ops->tz(oz_z, vp, (const char*)dT + (size_t)r0 * 8, p->max_rank, 1, nullptr, &ctrl->done, sp, join == nullptr, st);
+    const UpdPlan up = plan_upd(sms_g, rows, n, 128, kOzuBN, 1);
+    mark_f(RRF_PHASE_UPDATE);
+    CUtensorMap tmB;                  // cannot fail: the leading dimension and the base have passed the entry checks
+    make_map(h, &tmB, p->dtype, (char*)dB + (size_t)r0 * ldb * 8, b, n, ldb, 32);
+    ozt->update(i == 0 ? tmA_s : tmW_s, tmW_st, tmB, ob.vrow, ob.erow, ob.zimg, ob.ez, r0, rows, (int)n, b, norm_part,
+                ob.colmag[(i + 1) & 1], ob.rowmag[(i + 1) & 1], up, ctrl, true, st);
+    return up.P;
+  };
+
   // profiling: one event before every kernel, tagged with (phase, block step)
   bool nvtx_open = false;
   auto mark = [&](int phase, int step) {
@@ -1837,9 +2060,22 @@ rrf_status_t rrf_run(rrf_handle_t h, const rrf_params_t* p, void* dA, int64_t ld
   src.ldy = b;
   src.row_off = 0;
   mark(RRF_PHASE_SAMPLE, 0);
-  ops->sample(tmA_s, tmO, Ypart, 0, (int)m, (int)n, 0, sp, ctrl, nullptr, init_part, st);
-  init_ctrl_kernel<<<1, 256, 0, st>>>(init_part, std::min(sp.nslabs * sp.nseg, sp.ctas), p->tol, p->tol_is_relative,
-                                      fixed ? 1 : 0, b, p->max_rank, ctrl, done_after, samp, steps, predict);
+  if (oz) {
+    // the magnitudes that the products of pass 0 scale by, and ||A||_F^2 beside them
+    if (cudaMemsetAsync(ob.colmag[0], 0, (size_t)n * 4, st) != cudaSuccess || cudaMemsetAsync(ob.rowmag[0], 0, (size_t)m * 4, st) != cudaSuccess)
+      return RRF_ERR_CUDA;
+    const int grid = oz_mag_grid(m, n, L.init_ctas);
+    oz_mag_kernel<<<grid, 256, 0, st>>>((const double*)dA, lda, (int)m, (int)n, ob.colmag[0], ob.rowmag[0], init_part);
+    init_ctrl_kernel<<<1, 256, 0, st>>>(init_part, grid, p->tol, p->tol_is_relative, fixed ? 1 : 0, b, p->max_rank, ctrl, done_after, samp,
+                                        steps, predict);
+    oz_split(-1, 0, -1);
+    src = oz_sample(tmA_s, 0, 0, (int)m, h->sms, Y0, 0, true);
+    extra_launches += 2;
+  } else {
+    ops->sample(tmA_s, tmO, Y0, 0, (int)m, (int)n, 0, sp, ctrl, nullptr, init_part, st);
+    init_ctrl_kernel<<<1, 256, 0, st>>>(init_part, std::min(sp.nslabs * sp.nseg, sp.ctas), p->tol, p->tol_is_relative,
+                                        fixed ? 1 : 0, b, p->max_rank, ctrl, done_after, samp, steps, predict);
+  }
 
   if (unchanged) {
     // The variant of the paper's outlook that leaves A unchanged and returns no B: every panel is sampled from
@@ -1857,12 +2093,20 @@ rrf_status_t rrf_run(rrf_handle_t h, const rrf_params_t* p, void* dA, int64_t ld
       const int r0 = i * b, rows = (int)(m - r0);
       if (i > 0) {
         mark(RRF_PHASE_SAMPLE, i);
-        ops->sample(tmA_s, tmO, Ypart, 0, (int)m, (int)n, r0, sp, ctrl, nullptr, nullptr, st);
+        if (oz) {
+          oz_split(-1, r0, -1);
+          src = oz_sample(tmA_s, 0, 0, (int)m, h->sms, Y0, 0, true);
+          ++extra_launches;
+        } else {
+          ops->sample(tmA_s, tmO, Y0, 0, (int)m, (int)n, r0, sp, ctrl, nullptr, nullptr, st);
+        }
       }
-      if (p->dtype == RRF_F64)
-        panel_sum_kernel<double><<<sum_grid, 256, 0, st>>>((const double*)Ypart, sp.nseg, m * b, m, b, (double*)Pbuf, ctrl);
+      if (oz)
+        oz_panel_sum_kernel<<<sum_grid, 256, 0, st>>>((const double*)Y0, src.nc, src.tpc, m, b, (double*)Pbuf, ctrl);
+      else if (p->dtype == RRF_F64)
+        panel_sum_kernel<double><<<sum_grid, 256, 0, st>>>((const double*)Y0, sp.nseg, m * b, m, b, (double*)Pbuf, ctrl);
       else
-        panel_sum_kernel<float><<<sum_grid, 256, 0, st>>>((const float*)Ypart, sp.nseg, m * b, m, b, (float*)Pbuf, ctrl);
+        panel_sum_kernel<float><<<sum_grid, 256, 0, st>>>((const float*)Y0, sp.nseg, m * b, m, b, (float*)Pbuf, ctrl);
       for (int l = 0; l < i; ++l) {
         const int q0 = l * b, rl = (int)(m - q0);
         VtwPlan vp = plan_vtw(h->sms, rl, b, ops->v_bn);
@@ -1920,12 +2164,28 @@ rrf_status_t rrf_run(rrf_handle_t h, const rrf_params_t* p, void* dA, int64_t ld
       po.g_out = &pg;
       bool t_aside = false;
       po.t_aside = &t_aside;
-      s = launch_panel(h, p->dtype, Ypart, src, rows, b, Vblk(r0), ldv, Tblk(r0), p->max_rank, ps, ctrl, &ctrl->done,
+      s = launch_panel(h, p->dtype, Y0, src, rows, b, Vblk(r0), ldv, Tblk(r0), p->max_rank, ps, ctrl, &ctrl->done,
                        st, mark, i, po);
       if (s != RRF_OK) return panel_failed(s);
       if (sampled)                     // the sampled rule looks at panel i before block i is applied
         est_kernel<<<1, 128, 0, st>>>(csq_buf(i), pg, (pg + 31) & ~31, b, p->max_rank, p->estimator, fixed ? 1 : 0, 0, i,
                                       tr_est, ctrl);
+      if (oz) {
+        const int j0 = (i + 1 < steps) ? r0 + b : -1;
+        mark(RRF_PHASE_VTW, i);
+        oz_split(i, j0, (i + 1) & 1);
+        const int parts = oz_pass(i, h->sms, t_aside ? h->sync_events[2 * i + 1] : nullptr, [&](int phase) { mark(phase, i); });
+        mark(RRF_PHASE_STOP, i);
+        launch_after(true, stop_kernel, 1, 256, 0, st, norm_part, parts, b, p->max_rank, p->estimator, fixed ? 1 : 0, tr_sub, tr_dir, ctrl,
+                     done_after, 1, nullptr, predict);
+        ++extra_launches;
+        if (j0 >= 0) {
+          mark(RRF_PHASE_SAMPLE, i);
+          src = oz_sample(tmW_s, (i + 1) & 1, r0 + b, rows - b, h->sms, Y0, 0, true);
+          ++extra_launches;
+        }
+        continue;
+      }
       VtwPlan vp = plan_vtw(h->sms, rows, n, ops->v_bn);
       vp.tc = tc;
       vp.chunk = h->tc_chunk;
@@ -1968,7 +2228,7 @@ rrf_status_t rrf_run(rrf_handle_t h, const rrf_params_t* p, void* dA, int64_t ld
     //   side stream : panel_0 | fix + panel_1 | fix + panel_2 | ...
     //   main stream :           V^T W, T Z, update, stop of pass 0 | of pass 1 | ...
     const int gsms = h->sms - look_ctas;
-    void* Ybuf[2] = {Ypart, ws + L.ypart2};
+    void* Ybuf[2] = {Y0, Y1};
     cudaEvent_t evS = h->sync_events[3 * steps], evS2 = h->sync_events[3 * steps + 1];
     auto evP = [&](int i) { return h->sync_events[3 * i]; };
     auto evU = [&](int i) { return h->sync_events[3 * i + 1]; };
@@ -1979,13 +2239,13 @@ rrf_status_t rrf_run(rrf_handle_t h, const rrf_params_t* p, void* dA, int64_t ld
     // starts as early as its inputs allow.
     auto gated = [&](int rows_i) {
       if (p->tune_gate != 0) return p->tune_gate == 2;
-      if (look_cl) return false;       // a cluster takes so few SMs that holding it back never pays (measured)
+      if (look_cl || oz) return false; // a cluster takes so few SMs that holding it back never pays (measured)
       const PassModel pm{h->sms, (double)rows_i, (double)n, b, p->dtype == RRF_F64, tc};
       return pm.step_gated(look_ctas) < pm.step_ungated(look_ctas);
     };
     PanelSource src1 = src;           // panel 1: sampled from A by the sample kernel
     src1.row_off = b;
-    src1.nseg = plan_sample(gsms, m, n, esize, ops->s_kbs).nseg;
+    if (!oz) src1.nseg = plan_sample(gsms, m, n, esize, ops->s_kbs).nseg;
     cudaEventRecord(evS, st);
     cudaStreamWaitEvent(h->aux, evS, 0);
     ps.bar = look_bar;
@@ -2009,13 +2269,20 @@ rrf_status_t rrf_run(rrf_handle_t h, const rrf_params_t* p, void* dA, int64_t ld
     cudaEventRecord(evP(0), h->aux);
     if (steps > 1) {                  // the second panel is sampled while the first is factored
       mark(RRF_PHASE_SAMPLE, 0);
-      const SamplePlan sp1 = plan_sample(gsms, m, n, esize, ops->s_kbs);   // beside the first panel
-      ops->sample(tmA_s, tmO, Ybuf[1], 0, (int)m, (int)n, b, sp1, ctrl, nullptr, nullptr, st);
+      if (oz) {
+        oz_split(-1, b, -1);
+        src1 = oz_sample(tmA_s, 0, 0, (int)m, gsms, Ybuf[1], b, true);
+        ++extra_launches;
+      } else {
+        const SamplePlan sp1 = plan_sample(gsms, m, n, esize, ops->s_kbs);   // beside the first panel
+        ops->sample(tmA_s, tmO, Ybuf[1], 0, (int)m, (int)n, b, sp1, ctrl, nullptr, nullptr, st);
+      }
       cudaEventRecord(evS2, st);
     }
     UpdPlan up_prev{};
     int pv_t1 = 0, pv_p1 = 0, pv_tpc2 = 0;   // how the update of the previous pass was split over two launches
     PanelSource alt_prev{};        // the panel of pass i+1 as the separate sample kernel would leave it
+    PanelSource oz_prev{};         // ... as the product on the integer tensor cores leaves it
     for (int i = 0; i < steps_run; ++i) {
       const int r0 = i * b, rows = (int)(m - r0);
       const bool gate = gated(rows);
@@ -2024,6 +2291,9 @@ rrf_status_t rrf_run(rrf_handle_t h, const rrf_params_t* p, void* dA, int64_t ld
         if (i == 0) cudaStreamWaitEvent(h->aux, evS2, 0);
         if (i >= 1) {
           cudaStreamWaitEvent(h->aux, evU(i - 1), 0);   // the panel sampled by the update of pass i-1
+          sn = oz_prev;
+        }
+        if (i >= 1 && !oz) {
           sn.slots = 1;
           sn.row_off = 2 * b;
           sn.bm = ops->u_bm;
@@ -2069,6 +2339,24 @@ rrf_status_t rrf_run(rrf_handle_t h, const rrf_params_t* p, void* dA, int64_t ld
       if (sampled)                     // the sampled rule looks at panel i before block i is applied
         est_kernel<<<1, 128, 0, st>>>(csq_buf(i), panel_g[i], (panel_g[i] + 31) & ~31, b, p->max_rank, p->estimator,
                                       fixed ? 1 : 0, 0, i, tr_est, ctrl);
+      if (oz) {
+        const int j0 = (i + 2 < steps) ? r0 + 2 * b : -1;
+        mark(RRF_PHASE_VTW, i);
+        oz_split(i, j0, (i + 1) & 1);
+        const int parts = oz_pass(i, gsms, nullptr, [&](int phase) { mark(phase, i); });
+        mark(RRF_PHASE_STOP, i);
+        launch_after(true, stop_kernel, 1, 256, 0, st, norm_part, parts, b, p->max_rank, p->estimator, fixed ? 1 : 0, tr_sub, tr_dir, ctrl,
+                     done_after, 0, nullptr, predict);
+        ++extra_launches;
+        if (j0 >= 0) {
+          // the first b of the sampled rows are those above the panel, which the fix-up needs
+          mark(RRF_PHASE_SAMPLE, i);
+          oz_prev = oz_sample(tmW_s, (i + 1) & 1, r0 + b, rows - b, gsms, Ybuf[i & 1], b, true);
+          ++extra_launches;
+        }
+        cudaEventRecord(evU(i), st);
+        continue;
+      }
       VtwPlan vp = plan_vtw(gate ? h->sms : gsms, rows, n, ops->v_bn);
       vp.tc = tc;
       vp.chunk = h->tc_chunk;
@@ -2172,7 +2460,7 @@ rrf_status_t rrf_run(rrf_handle_t h, const rrf_params_t* p, void* dA, int64_t ld
     };
     const void* ptrs[6] = {dA, dOmegaT, dV, dT, dB, d_workspace};
     const long long lds[4] = {lda, ldo, ldv, ldb};
-    const int ints[4] = {look_ctas, h->profiling, h->f32_engine, h->tc_chunk};
+    const int ints[5] = {look_ctas, h->profiling, h->f32_engine, h->tc_chunk, oz ? 1 : 0};
     put(p, sizeof(*p));
     put(ptrs, sizeof(ptrs));
     put(lds, sizeof(lds));
@@ -2287,7 +2575,7 @@ rrf_status_t rrf_run(rrf_handle_t h, const rrf_params_t* p, void* dA, int64_t ld
     // kernels this call put on the device (passes after the stop included: they start and return)
     const int lag = look_ctas > 0 ? 2 : 1;
     // without the predictor every executed pass that has a later panel to sample samples it
-    out->fused_samples = predicting ? hc.fused_samples : std::min(hc.steps, std::max(0, steps - lag));
+    out->fused_samples = oz ? 0 : (predicting ? hc.fused_samples : std::min(hc.steps, std::max(0, steps - lag)));
     const int sl = steps_run;      // passes whose kernels were launched
     const int first = 2 + (dOmegaT == nullptr ? 1 : 0);           // sample, loop state, the library's own vectors
     if (unchanged)
@@ -2296,7 +2584,8 @@ rrf_status_t rrf_run(rrf_handle_t h, const rrf_params_t* p, void* dA, int64_t ld
       out->kernel_launches = first + ((look_ctas > 0 && steps > 1) ? 1 : 0) + (4 + (sampled ? 1 : 0)) * sl +
                              (predicting ? std::max(0, std::min(sl, steps - lag)) : 0) + extra_launches;
   }
-  out->extra_samples = hc.extra_samples;
+  // with the integer tensor cores every later panel is sampled by a kernel of its own, which runs if the loop goes on
+  out->extra_samples = oz ? std::max(0, std::min(hc.steps - 1, steps - (look_ctas > 0 ? 2 : 1))) : hc.extra_samples;
   out->panel_ctas = look_ctas;
   if (hc.steps > 0) {
     if (h_E_sub_trace != nullptr) cudaMemcpy(h_E_sub_trace, tr_sub, sizeof(double) * hc.steps, cudaMemcpyDeviceToHost);
@@ -2357,7 +2646,7 @@ static rrf_status_t colmajor_layout(const rrf_params_t* p, ColMajorLayout* L) {
   L->ldat = (p->n + pad - 1) / pad * pad;
   RunLayout R;
   run_layout(&L->q, true, &R);
-  size_t off = align_up(R.total, 256);
+  size_t off = align_up(R.total_oz, 256);
   L->inner = off;
   L->at = off;
   off += align_up((size_t)p->m * (size_t)L->ldat * esize, 256);

@@ -2,6 +2,7 @@
 // kernels around it: compact-WY T factor, Z <- op(T) Z, norms, stop rule, Gaussian fill.
 #pragma once
 
+#include "i8_split.cuh"
 #include "panel_cqr.cuh"
 
 namespace rrf {
@@ -1081,6 +1082,8 @@ struct TzSplit {
   float* o;             // [2][B][ldo] planes of them
   long long ldo;
   int ntz;              // CTAs that work on Z
+  unsigned char* zi;    // double precision, products on the integer tensor cores: the result's images [32 columns][B / 32][7][32 x 32]
+  int* ez;              // ... and its scales, one per column, in the place of Zt (NULL: plain output)
 };
 template <typename T, int B, int COLS>
 __global__ void __launch_bounds__(kTzThreads)
@@ -1190,6 +1193,14 @@ __global__ void __launch_bounds__(kTzThreads)
       mma16x8x8(acc, af, bf);
     }
     const int j = j0 + g, col = col0 + n0 + 2 * t;
+    if constexpr (sizeof(T) == 8 && B >= 32) {
+      if (sp.zi != nullptr) {
+        T* cs = Bs + (size_t)B * PB;                // [COLS][B + 2]
+#pragma unroll
+        for (int e = 0; e < 4; ++e) cs[(n0 + 2 * t + (e & 1)) * (B + 2) + j + 8 * (e >> 1)] = acc[e];
+        continue;
+      }
+    }
     if constexpr (sizeof(T) == 4) {
       if (sp.z != nullptr) {
         const size_t plane = (size_t)sp.npad * B;
@@ -1205,6 +1216,35 @@ __global__ void __launch_bounds__(kTzThreads)
     Zt[(size_t)(col + 1) * B + j] = acc[1];
     Zt[(size_t)col * B + j + 8] = acc[2];
     Zt[(size_t)(col + 1) * B + j + 8] = acc[3];
+  }
+  if constexpr (sizeof(T) == 8 && B >= 32) {
+    if (sp.zi == nullptr) return;
+    // the digits of this CTA's columns: four rows of Z a thread, a scale per column
+    const double* cs = reinterpret_cast<const double*>(Bs + (size_t)B * PB);
+    __syncthreads();
+    constexpr int LPC = B / 4;                      // threads (lanes side by side) a column
+    for (int idx = tid; idx < COLS * LPC; idx += kTzThreads) {
+      const int cl = idx / LPC, j = (idx - cl * LPC) * 4, col = col0 + cl;
+      double x[4];
+      uint32_t mg = 0u;
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        x[e] = cs[cl * (B + 2) + j + e];
+        mg = max(mg, oz_mag(x[e]));
+      }
+#pragma unroll
+      for (int o = LPC / 2; o > 0; o >>= 1) mg = max(mg, __shfl_xor_sync(0xffffffffu, mg, o));
+      const int ex = oz_exp(mg);
+      const double s = oz_scale(ex);
+      uint32_t hi[4], lo[4], w[kOzS];
+#pragma unroll
+      for (int e = 0; e < 4; ++e) oz_digits(x[e], s, hi[e], lo[e]);
+      oz_pack4(hi, lo, w);
+      unsigned char* dst = sp.zi + ((size_t)(col >> 5) * (B / 32) + (j >> 5)) * (kOzS * 1024) + oz_at(col & 31, j & 31);
+#pragma unroll
+      for (int i = 0; i < kOzS; ++i) *reinterpret_cast<uint32_t*>(dst + i * 1024) = w[i];
+      if (j == 0) sp.ez[col] = ex;
+    }
   }
 }
 
