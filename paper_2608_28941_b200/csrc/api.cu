@@ -80,7 +80,7 @@ struct rrf_ctx {
   int gextra;                            // its kernels beyond those that every pass has (extra_launches in rrf_run)
   int cluster_ok;                        // a 16-CTA cluster of the panel kernel can be resident on this device
   int f32_engine;                        // single-precision V^T W: 0 = mma.sync 3xTF32, 1 = tcgen05 3xTF32
-  int f64_engine;                        // double precision: 0 = mma.sync f64, 1 = integer tensor cores, 2 = by size
+  int int_engine;                        // integer tensor cores: 0 = never, 1 = wherever they are built in, 2 = by size
   int tc_chunk;                          // tcgen05: 64-row tiles summed in tensor memory between round-to-nearest adds
 };
 
@@ -722,8 +722,8 @@ template <int B>
 struct OzOps {
   static constexpr int NB = B < 64 ? B : 64;
   static cudaError_t setup() {
-    cudaError_t e = cudaFuncSetAttribute(oz_gemm_kernel<NB, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, OzCfg<NB>::SMEM);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(oz_gemm_kernel<NB, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, OzCfg<NB>::SMEM);
+    cudaError_t e = cudaFuncSetAttribute(oz_gemm_kernel<NB, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, OzCfg<NB>::SMEM);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(oz_gemm_kernel<NB, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, OzCfg<NB>::SMEM);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(oz_update_kernel<B>, cudaFuncAttributeMaxDynamicSharedMemorySize, OzuCfg<B>::SMEM);
     return e;
   }
@@ -732,28 +732,30 @@ struct OzOps {
   }
   static void gemm(bool tr, const CUtensorMap& tm, const unsigned char* img, const int* e, const uint32_t* mag, double* part, int r0,
                    int lines, int first, const VtwPlan& p, Ctrl* ctrl, bool dep, cudaStream_t st) {
-    launch_after(dep, tr ? oz_gemm_kernel<NB, true> : oz_gemm_kernel<NB, false>, p.P * (B / NB), kOzThreads, OzCfg<NB>::SMEM, st, tm,
-                 img, e, mag, part, B, r0, lines, first, p.KT, p.total, p.tpc, ctrl);
+    launch_after(dep, tr ? oz_gemm_kernel<NB, true> : oz_gemm_kernel<NB, false>, p.P * (B / NB), kOzThreads, OzCfg<NB>::SMEM, st, tm, img, e, mag, part, B, r0, lines, first, p.KT, p.total,
+                 p.tpc, ctrl);
   }
   static void update(const CUtensorMap& tm, const CUtensorMap& tms, const CUtensorMap& tmt, const unsigned char* vimg, const int* ev,
                      const unsigned char* zimg, const int* ez, int r0, int rows, int ncols, int top_rows, double* norm_part,
                      uint32_t* colmag, uint32_t* rowmag, const UpdPlan& p, Ctrl* ctrl, bool dep, cudaStream_t st) {
     launch_after(dep, oz_update_kernel<B>, p.P, kOzuThreads, OzuCfg<B>::SMEM, st, tm, tms, tmt, vimg, ev, zimg, ez, r0, rows, ncols,
-                 top_rows, norm_part, colmag, rowmag, p.NC, p.total, p.tpc, ctrl);
+                   top_rows, norm_part, colmag, rowmag, p.NC, p.total, p.tpc, ctrl);
   }
 };
 struct OzTable {
   cudaError_t (*setup)();
   void (*split)(const OzSplit&, int, const int*, bool, cudaStream_t);
-  void (*gemm)(bool, const CUtensorMap&, const unsigned char*, const int*, const uint32_t*, double*, int, int, int, const VtwPlan&, Ctrl*,
-               bool, cudaStream_t);
+  void (*gemm)(bool, const CUtensorMap&, const unsigned char*, const int*, const uint32_t*, double*, int, int, int, const VtwPlan&, Ctrl*, bool,
+               cudaStream_t);
   void (*update)(const CUtensorMap&, const CUtensorMap&, const CUtensorMap&, const unsigned char*, const int*, const unsigned char*,
                  const int*, int, int, int, int, double*, uint32_t*, uint32_t*, const UpdPlan&, Ctrl*, bool, cudaStream_t);
 };
+template <int B>
+static OzTable make_oz() {
+  return OzTable{&OzOps<B>::setup, &OzOps<B>::split, &OzOps<B>::gemm, &OzOps<B>::update};
+}
 static const OzTable* oz_ops(int b) {
-  static const OzTable t32{&OzOps<32>::setup, &OzOps<32>::split, &OzOps<32>::gemm, &OzOps<32>::update},
-      t64{&OzOps<64>::setup, &OzOps<64>::split, &OzOps<64>::gemm, &OzOps<64>::update},
-      t128{&OzOps<128>::setup, &OzOps<128>::split, &OzOps<128>::gemm, &OzOps<128>::update};
+  static const OzTable t32 = make_oz<32>(), t64 = make_oz<64>(), t128 = make_oz<128>();
   return b == 32 ? &t32 : (b == 64 ? &t64 : (b == 128 ? &t128 : nullptr));
 }
 // Stream-K plan of a product: `lines` in tiles of 128, `len` contraction indices in tiles of 64; the b / 64 CTAs that share a
@@ -783,7 +785,7 @@ static OzBuf oz_carve(unsigned char* base, long long m, long long n, int b, bool
   const size_t sv = 2 * (size_t)ceil_div(m, 64), so = 2 * (size_t)ceil_div(n, 64), npad = align_up((size_t)n, 128);
   o.vrow = take((size_t)ceil_div(m, 128) * (b / 32) * kOzS * 4096);
   o.vcol = take(sv * kOzS * b * 32);
-  o.zimg = take(npad / 32 * (b / 32) * kOzS * 1024);
+  o.zimg = take(npad * (b / 32) * kOzS * 32);
   o.erow = (int*)take((size_t)m * 4);
   o.ecol = (int*)take((size_t)oz_chunks((int)sv, b / 32) * b * 4);
   o.ez = (int*)take(npad * 4);
@@ -828,8 +830,8 @@ static int oz_mag_grid(long long rows, long long cols, int most) {
 }
 // Whether a double-precision call over a rows x n matrix takes the integer tensor cores.
 static bool oz_wanted(const rrf_ctx* h, int dtype, long long rows, long long n, int b) {
-  if (dtype != RRF_F64 || b < 32 || h->f64_engine == 0) return false;
-  if (h->f64_engine == 1) return true;
+  if (dtype != RRF_F64 || b < 32 || h->int_engine == 0) return false;
+  if (h->int_engine == 1) return true;
   // The digits of V and Omega are made per block, which a matrix of few columns does not repay, and the kernels are two more
   // a pass.  Eight blocks, us without / with: b = 128, 2000 x 2000 2493 / 2331, 8192 x 8192 14321 / 9096; b = 64, 2000 x 2000
   // 1054 / 1129, 3000 x 3000 1389 / 1421, 2000 x 6000 1596 / 1430, 8192 x 8192 7193 / 5285; b = 32, 4096 x 4096 1292 / 1472,
@@ -1281,7 +1283,7 @@ rrf_status_t rrf_create(rrf_handle_t* out, int device) {
   h->gsteps = 0;
   h->gextra = 0;
   h->f32_engine = 1;      // single precision runs on tcgen05 unless rrf_set_single_engine says otherwise
-  h->f64_engine = 2;
+  h->int_engine = 2;
   h->tc_chunk = 2;
   std::memset(&h->profile, 0, sizeof(h->profile));
   cudaError_t e = cudaDeviceGetAttribute(&h->sms, cudaDevAttrMultiProcessorCount, device);
@@ -1344,9 +1346,9 @@ rrf_status_t rrf_set_single_engine(rrf_handle_t h, int32_t engine, int32_t chunk
   return RRF_OK;
 }
 
-rrf_status_t rrf_set_double_engine(rrf_handle_t h, int32_t engine) {
+rrf_status_t rrf_set_integer_engine(rrf_handle_t h, int32_t engine) {
   if (h == nullptr || engine < 0 || engine > 2) return RRF_ERR_INVALID_ARG;
-  h->f64_engine = engine;
+  h->int_engine = engine;
   return RRF_OK;
 }
 
@@ -2003,7 +2005,7 @@ rrf_status_t rrf_run(rrf_handle_t h, const rrf_params_t* p, void* dA, int64_t ld
     sp.zi = ob.zimg;
     sp.ez = ob.ez;
     ops->tz(oz_z, vp, (const char*)dT + (size_t)r0 * 8, p->max_rank, 1, nullptr, &ctrl->done, sp, join == nullptr, st);
-    const UpdPlan up = plan_upd(sms_g, rows, n, 128, kOzuBN, 1);
+    const UpdPlan up = plan_upd(sms_g, rows, n, 128, kOzBN, 1);
     mark_f(RRF_PHASE_UPDATE);
     CUtensorMap tmB;                  // cannot fail: the leading dimension and the base have passed the entry checks
     make_map(h, &tmB, p->dtype, (char*)dB + (size_t)r0 * ldb * 8, b, n, ldb, 32);

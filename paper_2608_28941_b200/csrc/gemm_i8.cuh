@@ -41,30 +41,46 @@ __device__ __forceinline__ uint64_t oz_desc(uint32_t addr) {       // K-contiguo
 __host__ __device__ constexpr uint32_t oz_idesc(int M, int N) {    // signed bytes, 32-bit integer accumulator
   return (2u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
-__device__ __forceinline__ void oz_mma(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t accumulate) {
+// The warp that issues walks its loop as a whole, and only the instructions themselves are one lane's (`lead`): descriptors and
+// addresses then stay in uniform registers.  In a branch of one lane each of them was moved there for every instruction, and a
+// step took that thread 1400 clocks in single precision, where its four products take 320.
+__device__ __forceinline__ uint32_t oz_lead() {
+  uint32_t r;
+  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(r));
+  return r;
+}
+__device__ __forceinline__ void oz_mma(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t accumulate, uint32_t lead) {
   asm volatile(
-      "{\n\t.reg .pred p;\n\t"
+      "{\n\t.reg .pred p, e;\n\t"
       "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::i8 [%0], %1, %2, %3, p;\n\t}"
-      ::"r"(d), "l"(a), "l"(b), "r"(idesc), "r"(accumulate)
+      "setp.ne.b32 e, %5, 0;\n\t"
+      "@e tcgen05.mma.cta_group::1.kind::i8 [%0], %1, %2, %3, p;\n\t}"
+      ::"r"(d), "l"(a), "l"(b), "r"(idesc), "r"(accumulate), "r"(lead)
+      : "memory");
+}
+__device__ __forceinline__ void oz_commit(uint64_t* bar, uint32_t lead) {
+  asm volatile(
+      "{\n\t.reg .pred e;\n\t"
+      "setp.ne.b32 e, %1, 0;\n\t"
+      "@e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}"
+      ::"r"(smem_u32(bar)), "r"(lead)
       : "memory");
 }
 // One step: digits of the 128-line operand at a0, those of the other (N lines each) at b0, all pairs with i + j < NG.
 template <int N, int NG>
-__device__ __forceinline__ void oz_step(uint32_t tmem, uint32_t a0, uint32_t b0, bool fresh) {
+__device__ __forceinline__ void oz_step(uint32_t tmem, uint32_t a0, uint32_t b0, bool fresh, uint32_t lead) {
   constexpr int W = 256 / N;                             // digits side by side in one instruction
 #pragma unroll
   for (int i = 0; i < kOzS; ++i) {
     const uint64_t a = oz_desc(a0 + i * 4096);
-    constexpr int all = kOzS;
-    const int nj = NG - i < all ? NG - i : all;
+    const int nj = NG - i < kOzS ? NG - i : kOzS;
 #pragma unroll
     for (int j = 0; j < nj;) {
       int w = nj - j < W ? nj - j : W;
       // a group's first product in a fresh accumulator overwrites: groups 0 ... 6 with i = 0, group 7 with i = 1, j = 6
       if (NG > kOzS && i == 1 && j + w == kOzS && w > 1) w -= 1;
       const bool over = fresh && (i == 0 || (NG > kOzS && i == 1 && j == kOzS - 1));
-      oz_mma(tmem + (i + j) * N, a, oz_desc(b0 + j * N * 32), oz_idesc(128, w * N), over ? 0u : 1u);
+      oz_mma(tmem + (i + j) * N, a, oz_desc(b0 + j * N * 32), oz_idesc(128, w * N), over ? 0u : 1u, lead);
       j += w;
     }
   }
@@ -75,30 +91,10 @@ __device__ __forceinline__ void oz_bulk_load(uint32_t dst, const void* src, uint
                ::"r"(dst), "l"(src), "r"(bytes), "r"(smem_u32(bar))
                : "memory");
 }
-// columns c ... c + 7 of NG groups N columns apart, this thread's lane
-template <int N, int NG>
-__device__ __forceinline__ void oz_ld8(uint32_t t, int (&r)[NG][8]) {
+// columns c ... c + 7 of eight groups N columns apart, this thread's lane
+template <int N>
+__device__ __forceinline__ void oz_ld8(uint32_t t, int (&r)[8][8]) {
   // the loads are asynchronous: they and the wait sit in one statement (see tmem_ld16)
-  if constexpr (NG == 7) {
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%56];\n\t"
-        "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%8,%9,%10,%11,%12,%13,%14,%15}, [%57];\n\t"
-        "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%16,%17,%18,%19,%20,%21,%22,%23}, [%58];\n\t"
-        "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%24,%25,%26,%27,%28,%29,%30,%31}, [%59];\n\t"
-        "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%32,%33,%34,%35,%36,%37,%38,%39}, [%60];\n\t"
-        "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%40,%41,%42,%43,%44,%45,%46,%47}, [%61];\n\t"
-        "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%48,%49,%50,%51,%52,%53,%54,%55}, [%62];\n\t"
-        "tcgen05.wait::ld.sync.aligned;"
-        : "=r"(r[0][0]), "=r"(r[0][1]), "=r"(r[0][2]), "=r"(r[0][3]), "=r"(r[0][4]), "=r"(r[0][5]), "=r"(r[0][6]), "=r"(r[0][7]),
-          "=r"(r[1][0]), "=r"(r[1][1]), "=r"(r[1][2]), "=r"(r[1][3]), "=r"(r[1][4]), "=r"(r[1][5]), "=r"(r[1][6]), "=r"(r[1][7]),
-          "=r"(r[2][0]), "=r"(r[2][1]), "=r"(r[2][2]), "=r"(r[2][3]), "=r"(r[2][4]), "=r"(r[2][5]), "=r"(r[2][6]), "=r"(r[2][7]),
-          "=r"(r[3][0]), "=r"(r[3][1]), "=r"(r[3][2]), "=r"(r[3][3]), "=r"(r[3][4]), "=r"(r[3][5]), "=r"(r[3][6]), "=r"(r[3][7]),
-          "=r"(r[4][0]), "=r"(r[4][1]), "=r"(r[4][2]), "=r"(r[4][3]), "=r"(r[4][4]), "=r"(r[4][5]), "=r"(r[4][6]), "=r"(r[4][7]),
-          "=r"(r[5][0]), "=r"(r[5][1]), "=r"(r[5][2]), "=r"(r[5][3]), "=r"(r[5][4]), "=r"(r[5][5]), "=r"(r[5][6]), "=r"(r[5][7]),
-          "=r"(r[6][0]), "=r"(r[6][1]), "=r"(r[6][2]), "=r"(r[6][3]), "=r"(r[6][4]), "=r"(r[6][5]), "=r"(r[6][6]), "=r"(r[6][7])
-        : "r"(t), "r"(t + N), "r"(t + 2 * N), "r"(t + 3 * N), "r"(t + 4 * N), "r"(t + 5 * N), "r"(t + 6 * N)
-        : "memory");
-  } else {
     asm volatile(
         "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%64];\n\t"
         "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%8,%9,%10,%11,%12,%13,%14,%15}, [%65];\n\t"
@@ -119,26 +115,30 @@ __device__ __forceinline__ void oz_ld8(uint32_t t, int (&r)[NG][8]) {
           "=r"(r[7][0]), "=r"(r[7][1]), "=r"(r[7][2]), "=r"(r[7][3]), "=r"(r[7][4]), "=r"(r[7][5]), "=r"(r[7][6]), "=r"(r[7][7])
         : "r"(t), "r"(t + N), "r"(t + 2 * N), "r"(t + 3 * N), "r"(t + 4 * N), "r"(t + 5 * N), "r"(t + 6 * N), "r"(t + 7 * N)
         : "memory");
-  }
 }
-// The groups of one entry put together.  A group is below 2^14 * 7 * 32 kOzChunk steps < 2^27, so both integers are below
-// 2^51 and the conversion by adding 1.5 2^52 is exact.  Value: the result times 2^(ea - kOzOut) 2^(eb - kOzOut).
-template <int NG>
-__device__ __forceinline__ double oz_join(const int (&r)[NG][8], int e) {
+// The eight groups of one entry put together.  A group is below 2^14 * 7 * 32 kOzChunk steps < 2^27, those that the two integers
+// begin with below 2^24.1 and 2^26.4, so both are below 2^51 and their conversion by the bits of 1.5 2^52 is exact.  Value: the
+// result times 2^(ea - kOzOut) 2^(eb - kOzOut).
+constexpr int kOzOut = 19;       // 2^-14 of the digits' places and the first integer's 2^-24, half to either scale
+__device__ __forceinline__ long long oz_mad(int a, int b, long long c) {
+  long long d;
+  asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(d) : "r"(a), "r"(b), "l"(c));
+  return d;
+}
+template <bool SMALL = false>      // SMALL: groups below 2^23, so that two of them fit one 32-bit integer
+__device__ __forceinline__ double oz_join(const int (&r)[8][8], int e) {
   const double m = 6755399441055744.0;
+  const long long c = 0x4338000000000000ll;
   long long hi, lo;
-  if constexpr (NG == 7) {
-    hi = (long long)r[0][e] * 65536 + ((long long)r[1][e] * 256 + r[2][e]);
-    lo = (long long)r[3][e] * 16777216 + ((long long)r[4][e] * 65536 + ((long long)r[5][e] * 256 + r[6][e]));
+  if constexpr (SMALL) {
+    hi = oz_mad(r[0][e] * 256 + r[1][e], 65536, oz_mad(r[2][e] * 256 + r[3][e], 1, c));
+    lo = oz_mad(r[4][e] * 256 + r[5][e], 65536, oz_mad(r[6][e] * 256 + r[7][e], 1, c));
   } else {
-    hi = (long long)r[0][e] * 16777216 + ((long long)r[1][e] * 65536 + ((long long)r[2][e] * 256 + r[3][e]));
-    lo = (long long)r[4][e] * 16777216 + ((long long)r[5][e] * 65536 + ((long long)r[6][e] * 256 + r[7][e]));
+    hi = oz_mad(r[0][e], 16777216, oz_mad(r[1][e], 65536, oz_mad(r[2][e], 256, oz_mad(r[3][e], 1, c))));
+    lo = oz_mad(r[4][e], 16777216, oz_mad(r[5][e], 65536, oz_mad(r[6][e], 256, oz_mad(r[7][e], 1, c))));
   }
-  const double h = __longlong_as_double(hi + 0x4338000000000000ll) - m, l = __longlong_as_double(lo + 0x4338000000000000ll) - m;
-  return fma(l, 0x1p-32, h);
+  return fma(__longlong_as_double(lo) - m, 0x1p-32, __longlong_as_double(hi) - m);
 }
-template <int NG>
-constexpr int kOzOut = NG == 7 ? 15 : 19;       // 7 groups: 2^-14 and hi's 2^-16; 8: 2^-14 and 2^-24; half to either scale
 
 // ------------------------------------------------------------------------------------------
 // Z = V^T C (TR: the contraction runs over the rows of C, a line of the 128-line operand is a column of C) and
@@ -157,9 +157,10 @@ constexpr int kOzThreads = (kOzConv + 3) * 32;
 template <int NB>
 struct OzCfg {
   static constexpr int W_BYTES = 128 * kOzK * 8, B_BYTES = kOzS * NB * 32, A_BYTES = kOzS * 128 * 32;
-  static constexpr int RW = kOzGroups, RB = 3, RA = kOzGroups;
-  static constexpr int SMEM = RW * W_BYTES + RB * B_BYTES + RA * A_BYTES + 1024;
-  static constexpr int COLS = kOzS * NB <= 256 ? 256 : 512;
+  static constexpr int RW = kOzGroups, RA = kOzGroups;
+  static constexpr int SMEM = RW * W_BYTES + RA * (A_BYTES + B_BYTES) + 1024;
+  static constexpr int COLS = 8 * NB;
+  static_assert(SMEM + 1024 <= 232448 && (COLS == 256 || COLS == 512), "shared and tensor memory");
 };
 template <int NB, bool TR>
 __global__ void __launch_bounds__(kOzThreads, 1)
@@ -172,12 +173,12 @@ __global__ void __launch_bounds__(kOzThreads, 1)
   pdl_trigger();
   if (*reinterpret_cast<volatile int*>(&ctrl->done)) return;
   using Cfg = OzCfg<NB>;
-  constexpr int RW = Cfg::RW, RB = Cfg::RB, RA = Cfg::RA;
+  constexpr int RW = Cfg::RW, RA = Cfg::RA;
   extern __shared__ unsigned char smem_raw[];
   unsigned char* ringW = align1024(smem_raw);
   unsigned char* ringA = ringW + RW * Cfg::W_BYTES;
   unsigned char* ringB = ringA + Cfg::RA * Cfg::A_BYTES;
-  __shared__ uint64_t wfull[RW], wempty[RW], bfull[RB], bempty[RB], afull[RA], aempty[RA], acc_full, acc_empty;
+  __shared__ uint64_t wfull[RW], wempty[RW], full[RA], empty[RA], acc_full, acc_empty;
   __shared__ uint32_t tmem_slot;
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -189,13 +190,9 @@ __global__ void __launch_bounds__(kOzThreads, 1)
       mbar_init(&wfull[s], 1);
       mbar_init(&wempty[s], 4);
     }
-    for (int s = 0; s < RB; ++s) {
-      mbar_init(&bfull[s], 1);
-      mbar_init(&bempty[s], 1);
-    }
     for (int s = 0; s < RA; ++s) {
-      mbar_init(&afull[s], 4);
-      mbar_init(&aempty[s], 1);
+      mbar_init(&full[s], 4 + 1);        // the group's four warps and the copy of the small operand
+      mbar_init(&empty[s], 1);
     }
     mbar_init(&acc_full, 1);
     mbar_init(&acc_empty, kOzConv);
@@ -259,33 +256,32 @@ __global__ void __launch_bounds__(kOzThreads, 1)
     // ---------------------------------------------------------------- bulk copies: images of the small operand
     if (lane == 0) {
       for (int q = 0; q < nsub; ++q, at.next()) {
-        const int s = q % RB;
-        if (q >= RB && !mbar_wait(&bempty[s], ((q / RB) - 1) & 1, ctrl)) break;
-        mbar_expect_tx(&bfull[s], Cfg::B_BYTES);
-        oz_bulk_load(smem_u32(ringB + s * Cfg::B_BYTES), img + (size_t)(at.k * nh + h) * Cfg::B_BYTES, Cfg::B_BYTES, &bfull[s]);
+        const int s = q % RA;
+        if (q >= RA && !mbar_wait(&empty[s], ((q / RA) - 1) & 1, ctrl)) break;
+        mbar_expect_tx(&full[s], Cfg::B_BYTES);
+        oz_bulk_load(smem_u32(ringB + s * Cfg::B_BYTES), img + (size_t)(at.k * nh + h) * Cfg::B_BYTES, Cfg::B_BYTES, &full[s]);
       }
     }
   } else if (warp == kOzConv + 2) {
     // ---------------------------------------------------------------- MMA issuer
-    if (lane == 0) {
-      bool fresh = true;
-      int ndrain = 0;
-      for (int q = 0; q < nsub; ++q, at.next()) {
-        const int a = q % RA, s = q % RB;
-        if (!mbar_wait(&bfull[s], (q / RB) & 1, ctrl)) break;
-        if (!mbar_wait(&afull[a], (q / RA) & 1, ctrl)) break;
-        if (fresh && ndrain > 0 && !mbar_wait(&acc_empty, (ndrain - 1) & 1, ctrl)) break;
-        tc_fence_after();
-        oz_step<NB, kOzS>(tmem, smem_u32(ringA + a * Cfg::A_BYTES), smem_u32(ringB + s * Cfg::B_BYTES), fresh);
-        fresh = false;
-        tc_commit(&aempty[a]);
-        tc_commit(&bempty[s]);
-        if (drain_after(q)) {
-          tc_commit(&acc_full);
-          fresh = true;
-          ++ndrain;
-        }
+    const uint32_t lead = oz_lead(), a0 = smem_u32(ringA), b0 = smem_u32(ringB);
+    bool fresh = true;
+    int ndrain = 0, s = 0;
+    uint32_t ph = 0;
+    for (int q = 0; q < nsub; ++q, at.next()) {
+      if (!mbar_wait(&full[s], ph, ctrl)) break;
+      if (fresh && ndrain > 0 && !mbar_wait(&acc_empty, (ndrain - 1) & 1, ctrl)) break;
+      tc_fence_after();
+      if (TR && at.k < first) oz_step<NB, 8>(tmem, a0 + s * Cfg::A_BYTES, b0 + s * Cfg::B_BYTES, fresh, lead);
+      else oz_step<NB, 7>(tmem, a0 + s * Cfg::A_BYTES, b0 + s * Cfg::B_BYTES, fresh, lead);
+      fresh = false;
+      oz_commit(&empty[s], lead);
+      if (drain_after(q)) {
+        oz_commit(&acc_full, lead);
+        fresh = true;
+        ++ndrain;
       }
+      if (++s == RA) { s = 0; ph ^= 1u; }
     }
   } else {
     // ---------------------------------------------------------------- split and drain
@@ -302,7 +298,7 @@ __global__ void __launch_bounds__(kOzThreads, 1)
     auto drain = [&](int c, int ch, bool add) {
       const int l = c * 128 + line;
       // scales first: their loads are under way while the products end
-      const double fa = oz_pow2(oz_exp(l < lines ? mag[l] : 0u) - kOzOut<kOzS>);
+      const double fa = oz_pow2(oz_exp(l < lines ? mag[l] : 0u) - kOzOut);
       double* out = part + (size_t)(p + c) * (size_t)(B * 128) + (TR ? (size_t)(h * NB) * 128 + line : (size_t)line * B + h * NB);
       const int* eb = eimg + ch * B + h * NB;
       bool waited = false;
@@ -330,18 +326,22 @@ __global__ void __launch_bounds__(kOzThreads, 1)
           waited = true;
           tc_fence_after();
         }
-        int r[kOzS][8];
-        oz_ld8<NB, kOzS>(tlane + j, r);
+        int r[8][8];
+        oz_ld8<NB>(tlane + j, r);
+        if (!(TR && ch == 0)) {          // the eighth group is there for V's unit triangle only
+#pragma unroll
+          for (int e = 0; e < 8; ++e) r[7][e] = 0;
+        }
 #pragma unroll
         for (int e = 0; e < 8; ++e)
-          v[e] = fma(oz_join<kOzS>(r, e) * fa, oz_pow2(__shfl_sync(0xffffffffu, e8, e) - kOzOut<kOzS>), v[e]);
+          v[e] = fma(oz_join(r, e) * fa, oz_pow2(__shfl_sync(0xffffffffu, e8, e) - kOzOut), v[e]);
 #pragma unroll
         for (int e = 0; e < 8; e += 2) {
           if (TR) {
             out[(size_t)(j + e) * 128] = v[e];
             out[(size_t)(j + e + 1) * 128] = v[e + 1];
           } else {
-            *reinterpret_cast<double2*>(out + j + e) = make_double2(v[e], v[e + 1]);
+            store2(out + j + e, v[e], v[e + 1]);
           }
         }
       }
@@ -370,9 +370,9 @@ __global__ void __launch_bounds__(kOzThreads, 1)
           sc = oz_scale(oz_exp(l < lines ? mag[l] : 0u));
           cur_c = at.c;
         }
-        const int use = q / kOzGroups;       // times this group's places were used before
+        const int use = q / kOzGroups;       // how often this group's places were used before
         if (!mbar_wait(&wfull[grp], use & 1, ctrl)) break;
-        if (use > 0 && !mbar_wait(&aempty[grp], (use - 1) & 1, ctrl)) break;
+        if (use > 0 && !mbar_wait(&empty[grp], (use - 1) & 1, ctrl)) break;
         const unsigned char* w = ringW + grp * Cfg::W_BYTES;
 #pragma unroll 1
         for (int half = 0; half < 2; ++half) {
@@ -393,10 +393,8 @@ __global__ void __launch_bounds__(kOzThreads, 1)
                 x[2 * e + 1] = v.y;
               }
             }
-            uint32_t hi[4], lo[4], d[kOzS];
-#pragma unroll
-            for (int e = 0; e < 4; ++e) oz_digits(x[e], sc, hi[e], lo[e]);
-            oz_pack4(hi, lo, d);
+            uint32_t d[kOzS];
+            oz_words(x, sc, d);
 #pragma unroll
             for (int i = 0; i < kOzS; ++i) word[i][k4] = d[i];
           }
@@ -408,7 +406,7 @@ __global__ void __launch_bounds__(kOzThreads, 1)
         proxy_fence_async_smem();
         __syncwarp();
         if (lane == 0) {
-          mbar_arrive(&afull[grp]);
+          mbar_arrive(&full[grp]);
           mbar_arrive(&wempty[grp]);     // every number read from the stage has gone into the stores above
         }
         pay(q);
@@ -439,12 +437,11 @@ __global__ void __launch_bounds__(kOzThreads, 1)
 // 32 (w % 4) ..., 16 columns = one TMA box), read them, put W's new values where the old ones stood and store them by TMA.
 // A tile's bytes of W take 2930 clocks at the copy rate shared by 148 SMs, its products 1140 (B = 64; 2280 for 128).
 // ------------------------------------------------------------------------------------------
-constexpr int kOzuG = 8, kOzuBN = 32;
 constexpr int kOzuEpi = 16;
 constexpr int kOzuThreads = (kOzuEpi + 3) * 32;
 template <int B>
 struct OzuCfg {
-  static constexpr int KS = B / 32, V_BYTES = KS * kOzS * 4096, Z_BYTES = KS * kOzS * kOzuBN * 32;
+  static constexpr int KS = B / 32, V_BYTES = KS * kOzS * 4096, Z_BYTES = KS * kOzS * kOzBN * 32;
   static constexpr int BOX = 128 * 128, W_BYTES = 2 * BOX;
   static constexpr int NZ = B >= 128 ? 1 : 2;
   static constexpr int NW = B >= 128 ? 2 : 4;      // even: a place is always the same group's (see the waits by parity)
@@ -465,7 +462,7 @@ __global__ void __launch_bounds__(kOzuThreads, 1)
   pdl_trigger();
   if (*reinterpret_cast<volatile int*>(&ctrl->done)) return;
   using Cfg = OzuCfg<B>;
-  constexpr int NW = Cfg::NW, NZ = Cfg::NZ, KS = Cfg::KS, BN = kOzuBN, D = kOzuG * BN;
+  constexpr int NW = Cfg::NW, NZ = Cfg::NZ, KS = Cfg::KS, BN = kOzBN, D = 8 * BN;
   extern __shared__ unsigned char smem_raw[];
   unsigned char* ringW = align1024(smem_raw);
   unsigned char* sV = ringW + NW * Cfg::W_BYTES;
@@ -473,6 +470,7 @@ __global__ void __launch_bounds__(kOzuThreads, 1)
   __shared__ uint64_t wfull[NW], wempty[NW], zfull[NZ], zempty[NZ], vfull, vempty, d_full[2], d_empty[2];
   __shared__ uint32_t tmem_slot;
   __shared__ double red[64];
+  __shared__ __align__(16) double scale_s[kOzuEpi][16];      // a warp's own: scales of its tile's columns
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int p = blockIdx.x;
@@ -539,30 +537,28 @@ __global__ void __launch_bounds__(kOzuThreads, 1)
     }
   } else if (warp == kOzuEpi + 2) {
     // ---------------------------------------------------------------- MMA issuer
-    if (lane == 0) {
-      int c = L0 % NC, nslab = 0;
-      bool open = true;
-      for (int i = 0; i < ntile; ++i) {
-        const int st = i % NZ, d = i & 1;
-        if (open) {
-          if (!mbar_wait(&vfull, nslab & 1, ctrl)) break;
-          ++nslab;
-          open = false;
-        }
-        if (!mbar_wait(&zfull[st], (i / NZ) & 1, ctrl)) break;
-        if (i >= 2 && !mbar_wait(&d_empty[d], ((i >> 1) - 1) & 1, ctrl)) break;
-        tc_fence_after();
+    const uint32_t lead = oz_lead(), v0 = smem_u32(sV), z0 = smem_u32(ringZ);
+    int c = L0 % NC, nslab = 0;
+    bool open = true;
+    for (int i = 0; i < ntile; ++i) {
+      const int st = i % NZ, d = i & 1;
+      if (open) {
+        if (!mbar_wait(&vfull, nslab & 1, ctrl)) break;
+        ++nslab;
+        open = false;
+      }
+      if (!mbar_wait(&zfull[st], (i / NZ) & 1, ctrl)) break;
+      if (i >= 2 && !mbar_wait(&d_empty[d], ((i >> 1) - 1) & 1, ctrl)) break;
+      tc_fence_after();
 #pragma unroll
-        for (int ks = 0; ks < KS; ++ks)
-          oz_step<BN, kOzuG>(tmem + d * D, smem_u32(sV) + ks * kOzS * 4096, smem_u32(ringZ + st * Cfg::Z_BYTES) + ks * kOzS * BN * 32,
-                             ks == 0);
-        tc_commit(&d_full[d]);
-        tc_commit(&zempty[st]);
-        if (++c == NC) {
-          c = 0;
-          open = true;
-          tc_commit(&vempty);
-        }
+      for (int ks = 0; ks < KS; ++ks)
+        oz_step<BN, 8>(tmem + d * D, v0 + ks * kOzS * 4096, z0 + st * Cfg::Z_BYTES + ks * kOzS * BN * 32, ks == 0, lead);
+      oz_commit(&d_full[d], lead);
+      oz_commit(&zempty[st], lead);
+      if (++c == NC) {
+        c = 0;
+        open = true;
+        oz_commit(&vempty, lead);
       }
     }
   } else {
@@ -591,10 +587,12 @@ __global__ void __launch_bounds__(kOzuThreads, 1)
         const int lr = s * 128 + r;
         in = lr < rows;
         is_top = lr < top_rows;          // top_rows is a multiple of 32: the same for the whole warp
-        fr = oz_pow2(in ? ev[lr] - kOzOut<kOzuG> : 0);
+        fr = -oz_pow2(in ? ev[lr] - kOzOut : 0);
       }
       const int col = c * BN + box * 16;
-      const int ec = (lane < 16 && col + lane < ncols) ? ez[col + lane] : 0;
+      __syncwarp();                     // the last tile's scales have been read
+      if (lane < 16) scale_s[warp][lane] = oz_pow2((col + lane < ncols ? ez[col + lane] : 0) - kOzOut);
+      __syncwarp();
       if (!mbar_wait(&wfull[st], (i / NW) & 1, ctrl)) break;
       if (!mbar_wait(&d_full[grp], (i >> 1) & 1, ctrl)) break;
       tc_fence_after();
@@ -603,9 +601,9 @@ __global__ void __launch_bounds__(kOzuThreads, 1)
       double qs = 0.0;
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
-        int g[kOzuG][8];
-        oz_ld8<BN, kOzuG>(tlane + h * 8, g);
-        if (h == 1) {
+        int g[8][8];
+        oz_ld8<BN>(tlane + h * 8, g);
+        if (h == 2 - 1) {
           tc_fence_before();
           __syncwarp();
           if (lane == 0) mbar_arrive(&d_empty[grp]);
@@ -618,8 +616,7 @@ __global__ void __launch_bounds__(kOzuThreads, 1)
 #pragma unroll
           for (int e = 0; e < 2; ++e) {
             const int cc = h * 8 + e2 * 2 + e;
-            const double fc = oz_pow2(__shfl_sync(0xffffffffu, ec, cc) - kOzOut<kOzuG>);
-            w[e] = fma(-(oz_join<kOzuG>(g, e2 * 2 + e) * fr), fc, w[e]);
+            w[e] = fma(oz_join<B <= 64>(g, e2 * 2 + e) * fr, scale_s[warp][cc], w[e]);
             qs = fma(w[e], w[e], qs);
             const uint32_t mg = oz_mag(w[e]);
             rmax = max(rmax, mg);
@@ -673,7 +670,7 @@ struct OzSplit {
   int rows, nslab, steps_v, chunks_v;
   unsigned char *vrow, *vcol;
   int *erow, *ecol;
-  const double* Om;          // B x n, a vector a row (NULL: no Omega)
+  const double* Om;           // B x n, a vector a row (NULL: no Omega)
   long long ldo;
   int n, steps_o, chunks_o;
   unsigned char* oimg;
@@ -706,11 +703,8 @@ __global__ void __launch_bounds__(256) oz_split_kernel(const OzSplit a, const in
 #pragma unroll
       for (int o = LPR / 2; o > 0; o >>= 1) mg = max(mg, __shfl_xor_sync(0xffffffffu, mg, o));
       const int e = oz_exp(mg);
-      const double s = oz_scale(e);
-      uint32_t hi[4], lo[4], w[kOzS];
-#pragma unroll
-      for (int q = 0; q < 4; ++q) oz_digits(x[q], s, hi[q], lo[q]);
-      oz_pack4(hi, lo, w);
+      uint32_t w[kOzS];
+      oz_words(x, oz_scale(e), w);
       unsigned char* dst = a.vrow + ((size_t)bx * (B / 32) + (j >> 5)) * (kOzS * 4096) + oz_at(r, j & 31);
 #pragma unroll
       for (int i = 0; i < kOzS; ++i) *reinterpret_cast<uint32_t*>(dst + i * 4096) = w[i];
@@ -773,10 +767,9 @@ __global__ void __launch_bounds__(256) oz_split_kernel(const OzSplit a, const in
     uint32_t word[kOzS][4];
 #pragma unroll
     for (int k4 = 0; k4 < 4; ++k4) {
-      uint32_t hi[4], lo[4], w[kOzS];
-#pragma unroll
-      for (int e = 0; e < 4; ++e) oz_digits(x[u][k4 * 4 + e], s, hi[e], lo[e]);
-      oz_pack4(hi, lo, w);
+      const double q[4] = {x[u][k4 * 4], x[u][k4 * 4 + 1], x[u][k4 * 4 + 2], x[u][k4 * 4 + 3]};
+      uint32_t w[kOzS];
+      oz_words(q, s, w);
 #pragma unroll
       for (int i = 0; i < kOzS; ++i) word[i][k4] = w[i];
     }
@@ -792,40 +785,51 @@ __global__ void __launch_bounds__(256) oz_split_kernel(const OzSplit a, const in
 // sq_part, per-CTA partial sums of squares: one read of the matrix, HBM bound.  Tiles of 32 rows x 512 columns, a
 // thread two columns.
 // ------------------------------------------------------------------------------------------
-constexpr int kMagRows = 32, kMagCols = 512;
+constexpr int kMagRows = 32;
+constexpr int kMagCols = 512;
 __global__ void __launch_bounds__(256)
     oz_mag_kernel(const double* __restrict__ C, long long ldc, int rows, int cols, uint32_t* __restrict__ colmag,
                   uint32_t* __restrict__ rowmag, double* __restrict__ sq_part) {
+  constexpr int VEC = 2;
   __shared__ double red[32];
   __shared__ uint32_t rm[kMagRows];
   const int tid = threadIdx.x;
   const int nc = (cols + kMagCols - 1) / kMagCols, nr = (rows + kMagRows - 1) / kMagRows;
   double sq = 0.0;
   for (int t = blockIdx.x; t < nc * nr; t += gridDim.x) {
-    const int tr = t / nc, c = (t - tr * nc) * kMagCols + 2 * tid, r0 = tr * kMagRows;
+    const int tr = t / nc, c = (t - tr * nc) * kMagCols + VEC * tid, r0 = tr * kMagRows;
     if (tid < kMagRows) rm[tid] = 0u;
     __syncthreads();
-    uint32_t m0 = 0u, m1 = 0u;
+    uint32_t m[VEC] = {};
 #pragma unroll 8
     for (int r = 0; r < kMagRows; ++r) {
-      double2 v = make_double2(0.0, 0.0);
+      double v[VEC] = {};
       if (r0 + r < rows) {
         const double* src = C + (size_t)(r0 + r) * ldc + c;
-        if (c + 1 < cols) v = *reinterpret_cast<const double2*>(src);
-        else if (c < cols) v.x = *src;
+        if (c + VEC <= cols) {
+          VecLoad16<double>::ld(reinterpret_cast<const unsigned char*>(src), v);
+        } else {
+#pragma unroll
+          for (int u = 0; u < VEC; ++u)
+            if (c + u < cols) v[u] = src[u];
+        }
       }
-      const uint32_t a = oz_mag(v.x), b = oz_mag(v.y);
-      m0 = max(m0, a);
-      m1 = max(m1, b);
-      sq = fma(v.x, v.x, sq);
-      sq = fma(v.y, v.y, sq);
+      uint32_t w = 0u;
+#pragma unroll
+      for (int u = 0; u < VEC; ++u) {
+        const uint32_t a = oz_mag(v[u]);
+        m[u] = max(m[u], a);
+        w = max(w, a);
+        sq = fma(v[u], v[u], sq);
+      }
       if (rowmag != nullptr) {
-        const uint32_t w = __reduce_max_sync(0xffffffffu, max(a, b));
+        w = __reduce_max_sync(0xffffffffu, w);
         if ((tid & 31) == 0) atomicMax(&rm[r], w);
       }
     }
-    if (c < cols && m0 != 0u) atomicMax(colmag + c, m0);
-    if (c + 1 < cols && m1 != 0u) atomicMax(colmag + c + 1, m1);
+#pragma unroll
+    for (int u = 0; u < VEC; ++u)
+      if (colmag != nullptr && c + u < cols && m[u] != 0u) atomicMax(colmag + c + u, m[u]);
     __syncthreads();
     if (rowmag != nullptr && tid < kMagRows && r0 + tid < rows && rm[tid] != 0u) atomicMax(rowmag + r0 + tid, rm[tid]);
     __syncthreads();

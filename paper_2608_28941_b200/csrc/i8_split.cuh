@@ -7,31 +7,36 @@
 namespace rrf {
 
 constexpr int kOzS = 7;                 // digits of an operand
+constexpr int kOzBN = 32;               // columns of W in a tile of the update, of Z in an image
 constexpr int kOzK = 32;                // contraction indices of one instruction
 constexpr int kOzChunk = 32;            // steps of kOzK with one scale of the small operand (at most 32: see oz_join)
 constexpr int kOzBad = 1 << 20;         // "exponent" of a row or column that is not finite
 
-// exponent e with |x| < 0.996 2^e for every x up to the magnitude whose high word this is (the largest integer of seven
-// balanced digits is 0.99608 2^55)
-__device__ __forceinline__ int oz_exp(uint32_t hi) {
-  if (hi >= 0x7ff00000u) return kOzBad;
-  return max((int)((hi + 0x3000u) >> 20) - 1022, -960);
-}
+// Magnitude as an integer that orders like it (the high word), and the exponent e with |x| < 0.996 2^e for every x up to the
+// magnitude given (the largest integer of seven balanced digits is 0.99608 2^55)
 __device__ __forceinline__ uint32_t oz_mag(double x) { return (uint32_t)__double2hiint(x) & 0x7fffffffu; }
+__device__ __forceinline__ int oz_exp(uint32_t mag) {
+  if (mag >= 0x7ff00000u) return kOzBad;
+  return max((int)((mag + 0x3000u) >> 20) - 1022, -960);
+}
 __device__ __forceinline__ double oz_pow2(int e) {      // 2^e, -1022 <= e <= 1023; NaN for the scale of what is not finite
   return e > 2000 ? __longlong_as_double(0x7ff8000000000000ll) : __hiloint2double((1023 + e) << 20, 0);
 }
 __device__ __forceinline__ double oz_scale(int e) { return oz_pow2(55 - min(e, 1024)); }      // to integers
-// The bytes of x * s rounded to an integer, 0x80 added to each: four high digits, three low ones.
-__device__ __forceinline__ void oz_digits(double x, double s, uint32_t& hi, uint32_t& lo) {
-  const double m1 = 6755399441055744.0 * 16777216.0, m2 = 6755399441055744.0;     // 1.5 2^76, 1.5 2^52
-  const double a = fma(x, s, m1);                    // low word: x s / 2^24, rounded
-  const double r = fma(x, s, m1 - a);                // what is left, exact
-  lo = (uint32_t)__double2loint(r + m2) + 0x808080u;
-  hi = (uint32_t)__double2loint(a) + 0x80808080u + (uint32_t)((int)lo >> 24);
-}
-// Words of four consecutive contraction indices (v[0] in the low byte) for the seven digits
-__device__ __forceinline__ void oz_pack4(const uint32_t (&hi)[4], const uint32_t (&lo)[4], uint32_t (&w)[kOzS]) {
+// Four numbers -> a word of four bytes (x[0] in the low one) for each of the digits, most significant digit first.
+// The bytes of x s rounded to an integer, 0x80 added to each: four high digits, three low ones.  `a` is x s rounded to a
+// multiple of 2^24 with the high digits' bias in it (its low word counts multiples of 2^24), c what has to be added to x s to
+// leave the rest beside 1.5 2^52; both are exact.
+__device__ __forceinline__ void oz_words(const double (&x)[4], double s, uint32_t (&w)[kOzS]) {
+  constexpr double m2 = 6755399441055744.0, m1 = m2 * 16777216.0 + 2155905152.0 * 16777216.0;     // 1.5 2^52; 1.5 2^76 + 0x80808080 2^24
+  uint32_t hi[4], lo[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const double a = fma(x[i], s, m1);
+    const double c = (m1 + m2) - a;
+    lo[i] = (uint32_t)__double2loint(fma(x[i], s, c)) + 0x808080u;
+    hi[i] = (uint32_t)__double2loint(a) + (uint32_t)((int)lo[i] >> 24);
+  }
   const uint32_t a = __byte_perm(hi[0], hi[1], 0x5140), b = __byte_perm(hi[2], hi[3], 0x5140);   // bytes 0, 1 of both
   const uint32_t c = __byte_perm(hi[0], hi[1], 0x7362), d = __byte_perm(hi[2], hi[3], 0x7362);   // bytes 2, 3
   w[3] = __byte_perm(a, b, 0x5410) ^ 0x80808080u;
@@ -47,4 +52,5 @@ __device__ __forceinline__ void oz_pack4(const uint32_t (&hi)[4], const uint32_t
 __host__ __device__ constexpr uint32_t oz_at(uint32_t line, uint32_t k) {      // byte k of a line of an image
   return line * 32u + ((((k >> 4) ^ (line >> 2)) & 1u) << 4) + (k & 15u);
 }
+
 }  // namespace rrf

@@ -1082,7 +1082,7 @@ struct TzSplit {
   float* o;             // [2][B][ldo] planes of them
   long long ldo;
   int ntz;              // CTAs that work on Z
-  unsigned char* zi;    // double precision, products on the integer tensor cores: the result's images [32 columns][B / 32][7][32 x 32]
+  unsigned char* zi;    // products on the integer tensor cores: the result's images [32 columns][B / 32][7][32 x 32]
   int* ez;              // ... and its scales, one per column, in the place of Zt (NULL: plain output)
 };
 template <typename T, int B, int COLS>
@@ -1220,13 +1220,13 @@ __global__ void __launch_bounds__(kTzThreads)
   if constexpr (sizeof(T) == 8 && B >= 32) {
     if (sp.zi == nullptr) return;
     // the digits of this CTA's columns: four rows of Z a thread, a scale per column
-    const double* cs = reinterpret_cast<const double*>(Bs + (size_t)B * PB);
+    const T* cs = Bs + (size_t)B * PB;
     __syncthreads();
     constexpr int LPC = B / 4;                      // threads (lanes side by side) a column
     for (int idx = tid; idx < COLS * LPC; idx += kTzThreads) {
       const int cl = idx / LPC, j = (idx - cl * LPC) * 4, col = col0 + cl;
-      double x[4];
-      uint32_t mg = 0u;
+      T x[4];
+      uint32_t mg = 0u, w[kOzS];
 #pragma unroll
       for (int e = 0; e < 4; ++e) {
         x[e] = cs[cl * (B + 2) + j + e];
@@ -1235,14 +1235,10 @@ __global__ void __launch_bounds__(kTzThreads)
 #pragma unroll
       for (int o = LPC / 2; o > 0; o >>= 1) mg = max(mg, __shfl_xor_sync(0xffffffffu, mg, o));
       const int ex = oz_exp(mg);
-      const double s = oz_scale(ex);
-      uint32_t hi[4], lo[4], w[kOzS];
+      oz_words(x, oz_scale(ex), w);
+      unsigned char* dst = sp.zi + ((size_t)(col / kOzBN) * (B / 32) + (j >> 5)) * (kOzS * kOzBN * 32) + oz_at(col % kOzBN, j & 31);
 #pragma unroll
-      for (int e = 0; e < 4; ++e) oz_digits(x[e], s, hi[e], lo[e]);
-      oz_pack4(hi, lo, w);
-      unsigned char* dst = sp.zi + ((size_t)(col >> 5) * (B / 32) + (j >> 5)) * (kOzS * 1024) + oz_at(col & 31, j & 31);
-#pragma unroll
-      for (int i = 0; i < kOzS; ++i) *reinterpret_cast<uint32_t*>(dst + i * 1024) = w[i];
+      for (int i = 0; i < kOzS; ++i) *reinterpret_cast<uint32_t*>(dst + i * kOzBN * 32) = w[i];
       if (j == 0) sp.ez[col] = ex;
     }
   }

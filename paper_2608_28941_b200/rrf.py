@@ -45,7 +45,7 @@ class rrf_profile_t(C.Structure):
     _fields_ = [("ms", C.c_double * 9), ("launches", C.c_int32 * 9), ("pad", C.c_int32)]
 
 
-EXPORTS = ["rrf_run_colmajor", "rrf_colmajor_workspace_bytes", "rrf_transpose", "rrf_set_single_engine", "rrf_set_double_engine", "rrf_sample_workspace_bytes", "rrf_sample_panel", "rrf_frobenius_sq", "rrf_panel_qr_blocked", "rrf_panel_qr_tree", "rrf_transfer_workspace_bytes", "rrf_subspace_transfer", "rrf_selftest_timeout", "rrf_selftest_arithmetic", "rrf_panel_path", "rrf_panel_qr_static", "rrf_set_profiling", "rrf_get_profile", "rrf_measure_peak", "rrf_create", "rrf_destroy", "rrf_workspace_bytes", "rrf_run", "rrf_panel_workspace_bytes",
+EXPORTS = ["rrf_run_colmajor", "rrf_colmajor_workspace_bytes", "rrf_transpose", "rrf_set_single_engine", "rrf_set_integer_engine", "rrf_sample_workspace_bytes", "rrf_sample_panel", "rrf_frobenius_sq", "rrf_panel_qr_blocked", "rrf_panel_qr_tree", "rrf_transfer_workspace_bytes", "rrf_subspace_transfer", "rrf_selftest_timeout", "rrf_selftest_arithmetic", "rrf_panel_path", "rrf_panel_qr_static", "rrf_set_profiling", "rrf_get_profile", "rrf_measure_peak", "rrf_create", "rrf_destroy", "rrf_workspace_bytes", "rrf_run", "rrf_panel_workspace_bytes",
            "rrf_panel_qr", "rrf_apply_workspace_bytes", "rrf_apply_qt", "rrf_apply_q", "rrf_form_q",
            "rrf_fill_omega", "rrf_last_status", "rrf_status_string"]
 
@@ -90,7 +90,7 @@ def load():
     lib.rrf_panel_path.argtypes = [vp, C.POINTER(C.c_int32), vp]
     lib.rrf_selftest_arithmetic.argtypes = [vp, C.c_int32, C.c_int64, vp, vp, vp, vp]
     lib.rrf_set_single_engine.argtypes = [vp, i32, i32]
-    lib.rrf_set_double_engine.argtypes = [vp, i32]
+    lib.rrf_set_integer_engine.argtypes = [vp, i32]
     lib.rrf_set_profiling.argtypes = [vp, i32]
     lib.rrf_get_profile.argtypes = [vp, C.POINTER(rrf_profile_t)]
     lib.rrf_measure_peak.argtypes = [vp, i32, C.c_double, C.POINTER(C.c_double)]
@@ -446,11 +446,11 @@ def rrf_set_single_engine(h, engine: int, chunk_tiles: int = 0) -> None:
         raise RrfError(s, "rrf_set_single_engine")
 
 
-def rrf_set_double_engine(h, engine: int) -> None:
+def rrf_set_integer_engine(h, engine: int) -> None:
     """Double-precision products: 0 = mma.sync f64, 1 = integer tensor cores, 2 = by size (default)."""
-    s = load().rrf_set_double_engine(h, int(engine))
+    s = load().rrf_set_integer_engine(h, int(engine))
     if s != RRF_OK:
-        raise RrfError(s, "rrf_set_double_engine")
+        raise RrfError(s, "rrf_set_integer_engine")
 
 
 def rrf_set_profiling(h, enable: bool) -> None:

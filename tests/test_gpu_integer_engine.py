@@ -1,4 +1,4 @@
-"""Double precision on the integer tensor cores (rrf_set_double_engine) against the float64 oracle and against mma.sync."""
+"""Double precision on the integer tensor cores (rrf_set_integer_engine) against the float64 oracle and against mma.sync."""
 import numpy as np
 import pytest
 import torch
@@ -48,11 +48,11 @@ def _problem(m, n, cap, scale, seed):
 def test_run_matches_oracle(h, m, n, b, cap, scale, sched):
     A, Om = _problem(m, n, cap, scale, m + n)
     dA, dOm = _padded(A), _padded(Om.T)
-    rrf.rrf_set_double_engine(h, 1)
+    rrf.rrf_set_integer_engine(h, 1)
     try:
         g = [rrf.rrf_run(h, dA, b, 0.0, cap, omegaT=dOm, flags=sched | rrf.RRF_FLAG_FIXED_RANK) for _ in range(3)]
     finally:
-        rrf.rrf_set_double_engine(h, 2)
+        rrf.rrf_set_integer_engine(h, 2)
     o = orc.rrf(A, Om, b, 0.0, cap, fixed_rank=True)
     assert g[0].k == o.k == cap and g[0].fused_samples == 0
     for r in g[1:]:                                  # the call, its capture and its replay
@@ -61,11 +61,11 @@ def test_run_matches_oracle(h, m, n, b, cap, scale, sched):
     # The products of a block lose a few units of 2^-53 of the largest entry that shares a scale.  What becomes of that in the
     # blocks after it is the problem's condition, which the run on mma.sync shows: its rounding errors are of the same size
     # (columns forty powers of two apart make 3e-11 of them).
-    rrf.rrf_set_double_engine(h, 0)
+    rrf.rrf_set_integer_engine(h, 0)
     try:
         g0 = rrf.rrf_run(h, dA, b, 0.0, cap, omegaT=dOm, flags=sched | rrf.RRF_FLAG_FIXED_RANK)
     finally:
-        rrf.rrf_set_double_engine(h, 2)
+        rrf.rrf_set_integer_engine(h, 2)
     err, err0 = (np.linalg.norm(x - o.B, axis=0) / np.linalg.norm(o.B, axis=0) for x in (B, g0.B[:cap].cpu().numpy()))
     assert err.max() <= max(1e-12, 3.0 * err0.max()), (err.max(), err0.max())     # column by column, whatever its scale
     V0 = g[0].V[:, :b].cpu().numpy()
@@ -80,10 +80,10 @@ def test_variant_that_leaves_a_unchanged(h, m, n, b, cap):
     out = []
     try:
         for engine in (0, 1):
-            rrf.rrf_set_double_engine(h, engine)
+            rrf.rrf_set_integer_engine(h, engine)
             out.append(rrf.rrf_run(h, dA, b, 1e-3, cap, omegaT=dOm, estimator=2, flags=rrf.RRF_FLAG_NO_UPDATE))
     finally:
-        rrf.rrf_set_double_engine(h, 2)
+        rrf.rrf_set_integer_engine(h, 2)
     a, c = out
     assert (a.k, a.status) == (c.k, c.status)
     assert float((a.V[:, :a.k] - c.V[:, :a.k]).norm()) <= 1e-11 * float(a.V[:, :a.k].norm())
@@ -94,11 +94,11 @@ def test_variant_that_leaves_a_unchanged(h, m, n, b, cap):
 def test_non_finite_input_is_reported(h, bad):
     A, Om = _problem(700, 600, 128, "plain", 3)
     A[650, 599] = bad
-    rrf.rrf_set_double_engine(h, 1)
+    rrf.rrf_set_integer_engine(h, 1)
     try:
         g = rrf.rrf_run(h, _padded(A), 64, 0.0, 128, omegaT=_padded(Om.T), flags=rrf.RRF_FLAG_FIXED_RANK, check=False)
     finally:
-        rrf.rrf_set_double_engine(h, 2)
+        rrf.rrf_set_integer_engine(h, 2)
     assert g.status == rrf.RRF_ERR_NONFINITE
 
 
@@ -107,16 +107,16 @@ def test_workspace_without_the_digits_is_enough_for_the_other_path(h):
     A, Om = _problem(m, n, cap, "plain", 9)
     dA, dOm = _padded(A), _padded(Om.T)
     need = rrf.rrf_workspace_bytes(rrf.make_params(rrf.RRF_F64, m, n, b, 0.0, cap, flags=rrf.RRF_FLAG_FIXED_RANK))
-    rrf.rrf_set_double_engine(h, 1)
+    rrf.rrf_set_integer_engine(h, 1)
     try:
         ws = torch.empty(need - cap * n * 8 - 4096, dtype=torch.uint8, device="cuda")
         g = rrf.rrf_run(h, dA, b, 0.0, cap, omegaT=dOm, flags=rrf.RRF_FLAG_FIXED_RANK, workspace=ws)
     finally:
-        rrf.rrf_set_double_engine(h, 2)
+        rrf.rrf_set_integer_engine(h, 2)
     o = orc.rrf(A, Om, b, 0.0, cap, fixed_rank=True)
     assert np.linalg.norm(g.B[:cap].cpu().numpy() - o.B) <= 1e-12 * np.linalg.norm(o.B)
 
 
 def test_engine_argument(h):
     with pytest.raises(rrf.RrfError):
-        rrf.rrf_set_double_engine(h, 3)
+        rrf.rrf_set_integer_engine(h, 3)
