@@ -384,7 +384,7 @@ rrf_status_t rrf_set_single_engine(rrf_handle_t h, int32_t engine, int32_t chunk
 
 /*
  * rrf_set_integer_engine - choose the tensor-core path of the large products in double precision (Algorithm 2 lines 7 and 8)
- * for every later call on this handle that computes them (rrf_run and its views).
+ * for every later call on this handle that computes them (rrf_run and its views, rrf_apply_qt).
  *   engine 0  mma.sync m16n8k8 f64
  *   engine 1  tcgen05.mma kind::i8: each operand split into seven 8-bit digits and a power of two per row or column, the
  *             products of digits summed exactly; wherever it is built (b >= 32)

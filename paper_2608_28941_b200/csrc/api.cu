@@ -1570,6 +1570,8 @@ rrf_status_t rrf_apply_workspace_bytes(int32_t dtype, int64_t m, int64_t ncols, 
   const size_t zslots = (size_t)(kMaxSms + vp.nct) * b * vp.bn;
   *bytes = align_up((size_t)vp.npad * b * esize, 256) + align_up(zslots * esize, 256);
   if (get_ops(dtype, b)->has_upd_tc) *bytes += tc_zsplit_bytes(vp.npad, b);
+  if (dtype == RRF_F64 && b >= 32)
+    *bytes += oz_carve(nullptr, m, ncols, b, false).bytes + align_up((size_t)(kMaxSms + ceil_div(ncols, 128)) * 128 * b * 8, 256);
   return RRF_OK;
 }
 
@@ -1596,6 +1598,46 @@ static rrf_status_t apply_blocks(rrf_handle_t h, int dtype, long long m, int b, 
   if (workspace_bytes < need || (reinterpret_cast<uintptr_t>(d_workspace) & 255u)) return RRF_ERR_WORKSPACE;
   if (k == 0) return RRF_OK;
   const OpTable* ops = get_ops(dtype, b);
+  // Double precision, Q^T: on the integer tensor cores.  (Not Q: there a block touches rows that the one before has not, whose
+  // magnitudes nobody has measured.)
+  if (transpose && oz_wanted(h, dtype, m, ncols, b)) {
+    const OzBuf o = oz_carve((unsigned char*)d_workspace, m, ncols, b, false);
+    double* zpart = reinterpret_cast<double*>((unsigned char*)d_workspace + o.bytes);
+    const OzTable* const t = oz_ops(b);
+    CUtensorMap tmT, tmR, tmS, tmTop;
+    if (!make_map_plain(h, &tmT, dC, m, ncols, ldc, 128, kOzK) || !make_map(h, &tmR, dtype, dC, m, ncols, ldc, 128) ||
+        !make_map(h, &tmS, dtype, dC, m, ncols, ldc, 32))
+      return RRF_ERR_INVALID_ARG;
+    if (cudaMemsetAsync(o.colmag[0], 0, (size_t)ncols * 4, st) != cudaSuccess) return RRF_ERR_CUDA;
+    oz_mag_kernel<<<oz_mag_grid(m, ncols, kInitCtas), 256, 0, st>>>((const double*)dC, ldc, (int)m, (int)ncols, o.colmag[0],
+                                                                                   nullptr, nullptr);
+    for (int l = 0; l < k / b; ++l) {
+      const int r0 = l * b, rows = (int)(m - r0);
+      const bool more = l + 1 < k / b;
+      double* const Crow = (double*)dC + (size_t)r0 * ldc;
+      if (!make_map(h, &tmTop, dtype, Crow, b, ncols, ldc, 32)) return RRF_ERR_INVALID_ARG;
+      OzSplit a;
+      const int grid = oz_split_args(o, &a, b, (const double*)dV + (size_t)r0 * ldv + r0, ldv, rows, nullptr, 0, 0);
+      a.zero0 = o.colmag[(l + 1) & 1];
+      a.nzero0 = (int)ncols;
+      t->split(a, grid, &h->d_ctrl->done, true, st);
+      VtwPlan vp = plan_oz(h->sms, ncols, rows, b);
+      t->gemm(true, tmT, o.vcol, o.ecol, o.colmag[l & 1], zpart, r0, (int)ncols, b / 32, vp, h->d_ctrl, true, st);
+      TzSplit sp{};
+      sp.zi = o.zimg;
+      sp.ez = o.ez;
+      ops->tz(zpart, vp, (const char*)dT + (size_t)r0 * esize, ldt, 1, nullptr, &h->d_ctrl->done, sp, true, st);
+      // the first b rows are done with this block: stored, but not among the magnitudes of the next one
+      t->update(tmR, tmS, tmTop, o.vrow, o.erow, o.zimg, o.ez, r0, rows, (int)ncols, b, nullptr, more ? o.colmag[(l + 1) & 1] : nullptr,
+                nullptr, plan_upd(h->sms, rows, ncols, 128, kOzBN, 1), h->d_ctrl, true, st);
+    }
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) {
+      h->last_cuda = (int)e;
+      return RRF_ERR_CUDA;
+    }
+    return RRF_OK;
+  }
   const VtwPlan vp0 = plan_vtw(kMaxSms, m, ncols, ops->v_bn);
   unsigned char* ws = (unsigned char*)d_workspace;
   void* Zt = ws;

@@ -90,6 +90,49 @@ def test_variant_that_leaves_a_unchanged(h, m, n, b, cap):
     np.testing.assert_allclose(c.E_est_trace, a.E_est_trace, rtol=1e-11)
 
 
+@pytest.mark.parametrize("m,n,b,k", [(128, 65, 32, 128), (1000, 770, 32, 96), (1153, 129, 64, 320), (900, 1090, 128, 384)])
+@pytest.mark.parametrize("spike", [False, True])
+def test_apply_qt_matches_oracle(h, m, n, b, k, spike):
+    rng = np.random.default_rng(m)
+    V, T = np.zeros((m, k)), np.zeros((b, k))
+    for r in range(0, k, b):
+        V[r:, r:r + b], _, T[:, r:r + b], _ = orc.panel_qr(rng.standard_normal((m - r, b)))
+    C = rng.standard_normal((m, n)) * np.exp2(rng.integers(-30, 31, n))
+    if spike:                                        # a column whose first rows dwarf the rest: gone from the scale after its block
+        C[:b, ::3] *= 1e9
+    ref = C.astype(np.longdouble)                    # in double the reference's own rounding is the larger part
+    for r in range(0, k, b):
+        v, t = V[r:, r:r + b].astype(np.longdouble), T[:, r:r + b].astype(np.longdouble)
+        ref[r:] -= v @ (t.T @ (v.T @ ref[r:]))
+    dV, dT = _padded(V), torch.from_numpy(T).cuda()
+    out = []
+    try:
+        for engine in (0, 1):
+            rrf.rrf_set_integer_engine(h, engine)
+            out.append(rrf.rrf_apply_qt(h, dV, dT, b, k, _padded(C)).cpu().numpy())
+    finally:
+        rrf.rrf_set_integer_engine(h, 2)
+    scale = np.linalg.norm(ref.astype(np.float64), axis=0)
+    err = [np.linalg.norm((o - ref).astype(np.float64), axis=0) / scale for o in out]
+    # an orthogonal transform in k / b <= 5 steps, each with a few 2^-53 of the column's norm; no worse than mma.sync as a whole
+    assert err[1].max() <= 4e-15, (err[0].max(), err[1].max())
+    assert np.sqrt(np.mean(err[1] ** 2)) <= 1.1 * np.sqrt(np.mean(err[0] ** 2))
+
+
+def test_apply_qt_passes_on_what_is_not_finite(h):
+    rng = np.random.default_rng(1)
+    V, _, T, _ = orc.panel_qr(rng.standard_normal((500, 64)))
+    C = rng.standard_normal((500, 300))
+    C[400, 7], C[3, 200] = np.nan, np.inf
+    rrf.rrf_set_integer_engine(h, 1)
+    try:
+        out = rrf.rrf_apply_qt(h, _padded(V), torch.from_numpy(T).cuda(), 64, 64, _padded(C)).cpu().numpy()
+    finally:
+        rrf.rrf_set_integer_engine(h, 2)
+    assert not np.isfinite(out[:, [7, 200]]).any()
+    assert np.isfinite(np.delete(out, [7, 200], axis=1)).all()
+
+
 @pytest.mark.parametrize("bad", [np.nan, np.inf])
 def test_non_finite_input_is_reported(h, bad):
     A, Om = _problem(700, 600, 128, "plain", 3)
