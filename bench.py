@@ -261,7 +261,22 @@ def roofline_of(pb, res, prof, steps, value_per_gpu, ms_step, ms_profiled, peaks
     if w.dtype == "f32":
         peak /= 3.0                               # three TF32 products per fp32 product
     tc = w.dtype == "f32" and getattr(pb, "f32_engine", "mma") == "tcgen05"
-    if top in gemm and tc:
+    # double precision on the integer tensor cores: no update samples, every later panel has a sample of its own
+    i8 = w.dtype == "f64" and res.fused_samples == 0 and res.extra_samples > 0
+    if top in gemm and i8:
+        # 28 products of 8-bit digits (34 in the update) stand for one in double precision, at twice the bf16 rate; the bytes of
+        # W take longer.  "sample" holds the first pass over A too.
+        hbm = peaks.get("hbm_gbs", 6650.0)
+        below = mi[1:1 + res.extra_samples]
+        rows = {"update": 2.0 * sum(mi), "vtw": sum(mi), "sample": 2.0 * w.m + sum(below)}[top]
+        achieved = steps * rows * w.n * 8.0 / (ms * 1e-3) / 1e9
+        work = steps * 2.0 * w.n * w.b * (sum(mi) if top != "sample" else w.m + sum(below))
+        peak = peaks.get("bf16_tflops", 1590.0) * 2.0 / (34.0 if top == "update" else 28.0)
+        rl = {"kernel": top, "bound": "hbm", "achieved": achieved, "peak": hbm, "unit": "GB/s", "frac": achieved / hbm,
+              "traffic": None, "peak_source": "MEASURED_PEAKS.json (of measured)" if "hbm_gbs" in peaks else "of fallback",
+              "avg_launch_ms": ms / max(cnt, 1), "launches": cnt, "tensor_tflops": work / (ms * 1e-3) / 1e12,
+              "tensor_peak_i8_digits": peak, "tensor_peak_source": "bf16 peak x 2 / digit products per product"}
+    elif top in gemm and tc:
         # Single precision on tcgen05: per 64 KB of W read and written the tensor core needs about half the time
         # HBM does, so HBM is the roof of these kernels.  Algorithmic bytes: the rows of W each launch must read
         # (update: and write back); V, Zt and OmegaT are smaller by n / b and stay in L2.
@@ -534,7 +549,7 @@ def main():
                            "l2": "inputs larger than L2 (A is %.0f MB)" % (w.m * w.n * esize / 1e6),
                            "queues": res.queues, "panel_ctas": res.panel_ctas, "panel_kernel": args.panel,
                            "variant": args.variant, "estimator": estimator,
-                           "passes_over_A_per_block": 1 if args.variant == "no-update" else 3,
+                           "passes_over_A_per_block": 1 if args.variant == "no-update" else (4 if res.fused_samples == 0 else 3),
                            "fused_samples": res.fused_samples, "extra_samples": res.extra_samples,
                            "parallelism": "replicas only" if world > 1 else "single GPU"},
                 "clocks": clocks, "e2e": e2e, "gpu_launches": launches,

@@ -438,11 +438,11 @@ struct PassModel {
   double rate(double wide) const { return b >= 64 ? wide : (f64 ? wide * (b == 32 ? 0.75 : 0.5) : wide * 0.5); }
   // integer tensor cores: bytes of W per microsecond (8192 x 8192, 148 SMs)
   double vtw() const {
-    if (oz) return 8.0 * rows * n / (b == 32 ? 4.3e6 : (b == 64 ? 3.6e6 : 2.1e6)) + 8.0;
+    if (oz) return 8.0 * rows * n / (b == 32 ? 4.6e6 : (b == 64 ? 3.8e6 : 2.1e6)) + 8.0;
     return 2.0 * rows * n * b / rate(f64 ? 34e6 : (tc ? 86e6 : 45e6)) + 10.0;
   }
   double upd() const {      // with the sample of a later panel
-    if (oz) return 16.0 * rows * n / (b == 32 ? 5.1e6 : (b == 64 ? 4.4e6 : 2.7e6)) + 10.0 + vtw();
+    if (oz) return 16.0 * rows * n / (b == 32 ? 5.4e6 : (b == 64 ? 4.9e6 : 3.0e6)) + 10.0 + vtw();
     return 4.0 * rows * n * b / rate(f64 ? 33e6 : (tc && b <= 64 ? 117e6 : 32e6)) + 15.0;
   }
   // T Z, the stop rule, the split planes and the hand-overs between them
@@ -833,10 +833,10 @@ static bool oz_wanted(const rrf_ctx* h, int dtype, long long rows, long long n, 
   if (dtype != RRF_F64 || b < 32 || h->int_engine == 0) return false;
   if (h->int_engine == 1) return true;
   // The digits of V and Omega are made per block, which a matrix of few columns does not repay, and the kernels are two more
-  // a pass.  Eight blocks, us without / with: b = 128, 2000 x 2000 2493 / 2331, 8192 x 8192 14321 / 9096; b = 64, 2000 x 2000
-  // 1054 / 1129, 3000 x 3000 1389 / 1421, 2000 x 6000 1596 / 1430, 8192 x 8192 7193 / 5285; b = 32, 4096 x 4096 1292 / 1472,
-  // 8192 x 8192 4280 / 4329, 20000 x 4000 5238 / 5087 (the bytes of W bound both).
-  return b >= 64 && n >= 8LL * b && rows * n >= (b == 64 ? 10000000LL : 4000000LL);
+  // a pass.  Eight blocks, us without / with: b = 128, 2000 x 2000 2508 / 2315, 8192 x 8192 14233 / 8645; b = 64, 2000 x 2000
+  // 1046 / 1119, 3000 x 3000 1375 / 1414, 2000 x 6000 1587 / 1391, 8192 x 8192 7155 / 4952; b = 32, 5000 x 5000 1826 / 1837,
+  // 9000 x 3000 1919 / 1949, 8192 x 8192 4272 / 4171, 20000 x 4000 5304 / 4856 (the bytes of W bound both).
+  return n >= 8LL * b && rows * n >= (b == 32 ? 60000000LL : (b == 64 ? 10000000LL : 4000000LL));
 }
 
 // panel QR + T factor, enqueued on `st`
@@ -1563,13 +1563,20 @@ rrf_status_t rrf_frobenius_sq(rrf_handle_t h, int32_t dtype, int64_t rows, int64
   return RRF_OK;
 }
 
-rrf_status_t rrf_apply_workspace_bytes(int32_t dtype, int64_t m, int64_t ncols, int32_t b, size_t* bytes) {
+// what the apply calls cannot do without; rrf_apply_workspace_bytes adds the digits of the integer tensor cores' path
+static rrf_status_t apply_least_bytes(int32_t dtype, int64_t m, int64_t ncols, int32_t b, size_t* bytes) {
   if (bytes == nullptr || !b_ok(dtype, b) || m < b || ncols < 1) return RRF_ERR_INVALID_ARG;
   const int esize = dtype == RRF_F64 ? 8 : 4;
   const VtwPlan vp = plan_vtw(kMaxSms, m, ncols, get_ops(dtype, b)->v_bn);
   const size_t zslots = (size_t)(kMaxSms + vp.nct) * b * vp.bn;
   *bytes = align_up((size_t)vp.npad * b * esize, 256) + align_up(zslots * esize, 256);
   if (get_ops(dtype, b)->has_upd_tc) *bytes += tc_zsplit_bytes(vp.npad, b);
+  return RRF_OK;
+}
+
+rrf_status_t rrf_apply_workspace_bytes(int32_t dtype, int64_t m, int64_t ncols, int32_t b, size_t* bytes) {
+  const rrf_status_t s = apply_least_bytes(dtype, m, ncols, b, bytes);
+  if (s != RRF_OK) return s;
   if (dtype == RRF_F64 && b >= 32)
     *bytes += oz_carve(nullptr, m, ncols, b, false).bytes + align_up((size_t)(kMaxSms + ceil_div(ncols, 128)) * 128 * b * 8, 256);
   return RRF_OK;
@@ -1594,13 +1601,15 @@ static rrf_status_t apply_blocks(rrf_handle_t h, int dtype, long long m, int b, 
   if (!ld_ok(ldv, k, esize) || !ld_ok(ldc, ncols, esize) || ldt < k || !aligned16(dV) || !aligned16(dC))
     return RRF_ERR_INVALID_ARG;
   size_t need = 0;
-  if (rrf_apply_workspace_bytes(dtype, m, ncols, b, &need) != RRF_OK) return RRF_ERR_INVALID_ARG;
+  if (apply_least_bytes(dtype, m, ncols, b, &need) != RRF_OK) return RRF_ERR_INVALID_ARG;
   if (workspace_bytes < need || (reinterpret_cast<uintptr_t>(d_workspace) & 255u)) return RRF_ERR_WORKSPACE;
   if (k == 0) return RRF_OK;
   const OpTable* ops = get_ops(dtype, b);
   // Double precision, Q^T: on the integer tensor cores.  (Not Q: there a block touches rows that the one before has not, whose
   // magnitudes nobody has measured.)
-  if (transpose && oz_wanted(h, dtype, m, ncols, b)) {
+  size_t with_digits = 0;
+  rrf_apply_workspace_bytes(dtype, m, ncols, b, &with_digits);
+  if (transpose && workspace_bytes >= with_digits && oz_wanted(h, dtype, m, ncols, b)) {
     const OzBuf o = oz_carve((unsigned char*)d_workspace, m, ncols, b, false);
     double* zpart = reinterpret_cast<double*>((unsigned char*)d_workspace + o.bytes);
     const OzTable* const t = oz_ops(b);
@@ -1742,7 +1751,8 @@ rrf_status_t rrf_subspace_transfer(rrf_handle_t h, int32_t dtype, int64_t m, int
   if (!b_ok(dtype, b) || k_old < 1 || k_new < 1 || k_old > m || k_new > m || ncols < 1 || ldm < ncols || ldmo < ncols)
     return RRF_ERR_INVALID_ARG;
   size_t need = 0;
-  if (rrf_transfer_workspace_bytes(dtype, m, ncols, b, &need) != RRF_OK) return RRF_ERR_INVALID_ARG;
+  if (apply_least_bytes(dtype, m, ncols, b, &need) != RRF_OK) return RRF_ERR_INVALID_ARG;
+  need += align_up((size_t)m * align_up((size_t)ncols, 16) * (dtype == RRF_F64 ? 8 : 4), 256);
   if (workspace_bytes < need || (reinterpret_cast<uintptr_t>(d_workspace) & 255u)) return RRF_ERR_WORKSPACE;
   const int esize = dtype == RRF_F64 ? 8 : 4;
   const long long ldc = (long long)align_up((size_t)ncols, 16);
